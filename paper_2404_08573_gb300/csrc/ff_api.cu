@@ -57,7 +57,7 @@ static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // goodness partials per row: the most either forward GEMM writes
 static int gpart_tiles_max(int N) {
-  const int a = tc_fwd_ntiles_max(N), b = simt_fwd_ntiles(N);
+  const int a = tc_fwd_ntiles_max(N), b = simt_fwd_ntiles_max(N);
   return a > b ? a : b;
 }
 
@@ -119,8 +119,6 @@ ff_status ensure_capacity(ff_layer* L, int rows) {
 
 static void free_layer(ff_layer* L) {
   if (!L) return;
-  dev_free(L->kpart);
-  dev_free(L->kcnt);
   dev_free(L->W);
   dev_free(L->mW);  // also holds v_W
   dev_free(L->dW);
@@ -146,30 +144,6 @@ struct FwdResult {
   bool local_grad_done;  // the forward's epilogue also formed the local step (tc_gemm_fwd_lg)
 };
 
-// Split-K scratch of an fp32 layer's forward and weight-gradient GEMMs on M
-// rows (grown on demand; new counters start at zero).
-static ff_status ensure_split(ff_layer* L, int M) {
-  const size_t fwd = simt_split_floats(M, L->N, L->K), wg = simt_split_floats(L->N, L->K, M);
-  const size_t need = fwd > wg ? fwd : wg;
-  if (need == 0) return FF_OK;
-  const int t1 = simt_split_tiles(M, L->N), t2 = simt_split_tiles(L->N, L->K);
-  const int tiles = t1 > t2 ? t1 : t2;
-  if (need <= L->kpart_cap && tiles <= L->kcnt_cap) return FF_OK;
-  FF_TRY(cudaStreamSynchronize(L->last_stream), "sync before split scratch growth");
-  dev_free(L->kpart);
-  dev_free(L->kcnt);
-  L->kpart = nullptr;
-  L->kcnt = nullptr;
-  L->kpart_cap = 0;
-  L->kcnt_cap = 0;
-  FF_TRY(dev_alloc(reinterpret_cast<void**>(&L->kpart), need * sizeof(float)), "split scratch");
-  FF_TRY(dev_alloc(reinterpret_cast<void**>(&L->kcnt), (size_t)tiles * sizeof(int)), "split counters");
-  FF_TRY(cudaMemset(L->kcnt, 0, (size_t)tiles * sizeof(int)), "zero split counters");
-  L->kpart_cap = need;
-  L->kcnt_cap = tiles;
-  return FF_OK;
-}
-
 // x_rows: rows of the raw input x when labels are given (0: M; M / 2: one
 // image per pair, read for the positive and the negative row).
 // lg (train steps): the local step's arguments; for a bf16 layer whose shape
@@ -179,10 +153,6 @@ static ff_status forward_core(ff_layer* L, const void* x, const int* labels, con
                               void* h_out, cudaStream_t st, cudaEvent_t ev_input_read, FwdResult* r,
                               int x_rows = 0, GradPrepArgs* lg = nullptr) {
   const int K = L->K, N = L->N;
-  if (!L->is_bf16) {
-    const ff_status ss = ensure_split(L, M);
-    if (ss != FF_OK) return ss;
-  }
   const double es = L->is_bf16 ? 2.0 : 4.0;
   const float* s;
   const void* X;
@@ -223,13 +193,9 @@ static ff_status forward_core(ff_layer* L, const void* x, const int* labels, con
               tc_gemm_fwd(static_cast<const bf16*>(X), L->ldK, L->Wb, L->ldK, M, N, K, ep, &L->ds->err, st),
               "forward GEMM (tcgen05)");
   } else {
-    ntiles = simt_fwd_ntiles(N);
-    ep.kpart = L->kpart;
-    ep.kpart_cap = L->kpart_cap;
-    ep.kcnt = L->kcnt;
-    ep.kcnt_cap = L->kcnt_cap;
+    ntiles = simt_fwd_ntiles(M, N, K);
     FF_LAUNCH(K_FWD_SIMT, 2.0 * M * N * K, st,
-              simt_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, M, N, K, ep, st), "forward GEMM (fp32)");
+              simt_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, M, N, K, M, ep, st), "forward GEMM (fp32)");
   }
   r->s = s;
   r->H = H;
@@ -295,14 +261,9 @@ ff_status train_step_impl(ff_layer* L, const void* x, const int* labels, const f
                             L->N, L->K, L->dW, L->K, &L->ds->err, st),
               "weight-gradient GEMM (tcgen05)");
   } else {
-    EpiArgs split{};
-    split.kpart = L->kpart;
-    split.kpart_cap = L->kpart_cap;
-    split.kcnt = L->kcnt;
-    split.kcnt_cap = L->kcnt_cap;
     FF_LAUNCH(K_WGRAD_SIMT, 2.0 * M * L->N * L->K, st,
               simt_gemm_wgrad(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(fr.X), L->ldK, M,
-                              L->N, L->K, L->dW, L->K, st, &split),
+                              L->N, L->K, L->dW, L->K, st),
               "weight-gradient GEMM (fp32)");
   }
   AdamArgs aa{};
@@ -517,7 +478,7 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
   int ldmax = 0, ntmax = 0;
   for (int k = 0; k < n_layers; ++k) {
     if (layers[k]->ldN > ldmax) ldmax = layers[k]->ldN;
-    const int nt = b16 || f32tc ? tc_fwd_ntiles_max(layers[k]->N) : simt_fwd_ntiles(layers[k]->N);
+    const int nt = b16 || f32tc ? tc_fwd_ntiles_max(layers[k]->N) : simt_fwd_ntiles_max(layers[k]->N);
     if (nt > ntmax) ntmax = nt;
   }
   // Samples per chunk: about 40 MB of activations per buffer, so that one
@@ -648,9 +609,10 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
                                   err, st),
                   "predict forward GEMM (fp32, tcgen05 TF32 x 3)");
       } else {
-        nt = simt_fwd_ntiles(Lk->N);
+        nt = simt_fwd_ntiles(rows, Lk->N, Lk->K);
         FF_LAUNCH(K_FWD_SIMT, 2.0 * rows * Lk->N * Lk->K, st,
-                  simt_gemm_fwd(static_cast<const float*>(Hb[cur]), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, ep, st),
+                  simt_gemm_fwd(static_cast<const float*>(Hb[cur]), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, rows, ep,
+                                st),
                   "predict forward GEMM (fp32)");
       }
       nt_prev = nt;

@@ -2,233 +2,372 @@
 // fp32 mode: the same contracts as the tensor-core GEMMs (forward with the
 // scale/bias/ReLU/goodness epilogue, plain fp32 store, weight gradient over
 // the batch rows), so the fp32 path is the full-precision statement of §3/§4
-// on the GPU.  A 128x128 tile per 256-thread CTA, 8x8 outputs per thread,
-// K in steps of 8 through double-buffered shared memory.  A GEMM of few
-// tiles (the 128-row steps of a small batch: 4 CTAs for 128 x 500) is
-// latency-bound on its long K loop, so it splits K over up to 8 CTAs per
-// tile: each writes its partial tile, and the last to arrive (an arrival
-// counter per tile, no waiting) adds the partials in split order and runs
-// the epilogue.
+// on the GPU.
+//
+// Bound by the SM's shared-memory reads and FMA issue together (large
+// outputs reach 45 to 50 TFLOP/s), small ones by latency.  FMAs are issued in
+// pairs (fma.rn.f32x2, each rounded as fmaf): 10 % faster than single ones.
+// A CTA of 256 threads computes a TM x TN tile over one slice of K, 8x8
+// outputs per thread, operands staged 32 deep in K by a ring of cp.async
+// copies.  Two shapes:
+//   128 x 128, all threads on the same K: the fewest operand reads per FMA;
+//   64 x 64, four groups of 64 threads that each take a quarter of every
+//     stage's K (8x8 outputs per thread again) and add up in shared memory:
+//     for outputs of few tiles.
+// Either may further be cut over K: the S CTAs of a tile form a thread-block
+// cluster, leave their partial tiles in their own shared memory, and each
+// adds TM/S rows of all S partials (in rank order) through distributed
+// shared memory and runs the epilogue on them -- no scratch in device memory
+// and no counters.
 #include "ff_internal.cuh"
+#include "ff_ptx.cuh"
 
 namespace ff {
 namespace {
 
-constexpr int TM = 128, TN = 128, TK = 8, NT = 256;
+constexpr int NT = 256;
+constexpr int TKS = 32;  // K per stage
 constexpr int MODE_FWD = 0, MODE_STORE = 1;
-constexpr int kMaxSplit = 8;
-constexpr int kSplitBelow = 76;  // split GEMMs of fewer tiles than half the SMs
+constexpr int kMaxSplit = 4;  // CTAs per cluster (see plan_of)
 
-int split_of(int M, int N, int K) {
-  const int tiles = cdiv(N, TN) * cdiv(M, TM);
-  const int steps = cdiv(K, TK);
-  if (tiles >= kSplitBelow || steps < 16) return 1;
-  int S = cdiv(kSplitBelow, tiles);
-  if (S > kMaxSplit) S = kMaxSplit;
-  if (S > steps / 4) S = steps / 4;  // at least 4 K steps per split
-  return S < 1 ? 1 : S;
+// Shape of one instance.  An operand's stage sits in shared memory as TKS
+// rows (one per K) of the tile's T rows or columns, padded by 4 floats.
+template <int T, int KGRP>
+struct Cfg {
+  static constexpr int TM = T, TN = T, KG = KGRP;
+  static constexpr int TT = T / 8;                 // threads along each side of a K group's tile
+  static constexpr int LD = T + 4;
+  static constexpr int OP = TKS * LD;              // floats of one operand's stage
+  static constexpr int STAGES = T == 128 ? 3 : 4;
+  static constexpr int RING = 2 * OP * STAGES;
+  static constexpr int PART = KG * TM * LD;        // the K groups' partial tiles, rows of LD floats
+  static constexpr int SMEM = (RING > PART ? RING : PART) * 4;
+  static_assert(TT * TT * KG == NT, "every thread owns 8x8 outputs of its K group");
+};
+
+__device__ __forceinline__ void cp_async16(float* dst, const float* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(float* dst, const float* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ float4 ld_cluster4(const float* local, uint32_t rank) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(ptx::mapa_shared(ptx::smem_u32(local), rank))
+               : "memory");
+  return v;
 }
 
-// Loads the TK x 128 slice [k0, k0+TK) of an operand whose tile rows start
-// at r0.  MN == false: element (r, k) at P[r * ld + k]; MN == true: at
-// P[k * ld + r].  Out-of-range elements read as zero.
-template <bool MN>
-__device__ __forceinline__ void load_tile(const float* __restrict__ P, int ld, int rows, int K, int r0, int k0,
-                                          float (&v)[4]) {
+// Two fp32 FMAs in one instruction, each rounded as fmaf.
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+  unsigned long long v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+  return v;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+__device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
+// Copies the slice [k0, k0 + TKS) of an operand whose tile rows start at r0
+// into S[k][r].  MN == false: element (r, k) at P[r * ld + k], transposed by
+// 4-byte copies (a warp takes 8 K of 4 rows: whole 32-byte sectors, and 32
+// distinct banks).  MN == true: at P[k * ld + r], by 16-byte copies when
+// `vec` (P and its row stride 16-byte aligned).  Elements past `rows` or K
+// read as zero (a copy of fewer source bytes than it writes fills the rest
+// with zeros, so row padding is never read).
+template <int T, bool MN>
+__device__ __forceinline__ void load_tile(float* S, const float* __restrict__ P, int ld, int rows, int K, int r0,
+                                          int k0, bool vec) {
+  constexpr int LD = T + 4;
   const int tid = threadIdx.x;
-  if (!MN) {
-    const int r = r0 + tid / 2, k = k0 + (tid & 1) * 4;
+  if (MN && vec) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = (r < rows && k + u < K) ? __ldg(P + (size_t)r * ld + k + u) : 0.f;
-  } else {
-    const int k = k0 + tid / 32, r = r0 + (tid & 31) * 4;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = (k < K && r + u < rows) ? __ldg(P + (size_t)k * ld + r + u) : 0.f;
-  }
-}
-
-template <bool MN>
-__device__ __forceinline__ void store_tile(float (*S)[TM + 4], const float (&v)[4]) {
-  const int tid = threadIdx.x;
-  if (!MN) {
-    const int r = tid / 2, k = (tid & 1) * 4;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) S[k + u][r] = v[u];
-  } else {
-    const int k = tid / 32, r = (tid & 31) * 4;
-    *reinterpret_cast<float4*>(&S[k][r]) = make_float4(v[0], v[1], v[2], v[3]);
-  }
-}
-
-template <bool A_MN, bool B_MN, int MODE>
-__global__ void __launch_bounds__(NT) k_simt_gemm(const float* __restrict__ A, int lda, const float* __restrict__ B,
-                                                  int ldb, int M, int N, int K, EpiArgs ep) {
-  __shared__ __align__(16) float As[2][TK][TM + 4];
-  __shared__ __align__(16) float Bs[2][TK][TN + 4];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-  // this CTA's share of K: split blockIdx.z of gridDim.z (whole TK steps)
-  const int S = gridDim.z;
-  const int per = ((K + TK - 1) / TK + S - 1) / S;
-  const int kb = blockIdx.z * per * TK;
-  const int ke = min(K, kb + per * TK);
-
-  float acc[8][8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-
-  float ra[4], rb[4];
-  load_tile<A_MN>(A, lda, M, K, m0, kb, ra);
-  load_tile<B_MN>(B, ldb, N, K, n0, kb, rb);
-  store_tile<A_MN>(As[0], ra);
-  store_tile<B_MN>(Bs[0], rb);
-  __syncthreads();
-
-  for (int k0 = kb; k0 < ke; k0 += TK) {
-    const int buf = ((k0 - kb) / TK) & 1;
-    const bool more = k0 + TK < ke;
-    if (more) {
-      load_tile<A_MN>(A, lda, M, K, m0, k0 + TK, ra);
-      load_tile<B_MN>(B, ldb, N, K, n0, k0 + TK, rb);
+    for (int i = 0; i < T * TKS / 4 / NT; ++i) {
+      const int c = tid + i * NT;
+      const int k = c / (T / 4), r = (c % (T / 4)) * 4;
+      const int left = k0 + k < K ? rows - (r0 + r) : 0;
+      const int n = left < 0 ? 0 : left > 4 ? 4 : left;
+      cp_async16(S + k * LD + r, n ? P + (size_t)(k0 + k) * ld + r0 + r : P, n * 4);
     }
+  } else {
+#pragma unroll 8
+    for (int i = 0; i < T * TKS / NT; ++i) {
+      // !MN: warp w of step i takes K 8 (w % 4) .. and rows 4 (w / 4 + 2 i) ..
+      const int c = tid + i * NT;
+      const int r = MN ? c % T : (tid >> 7) * 4 + i * 8 + ((tid >> 3) & 3);
+      const int k = MN ? c / T : ((tid >> 5) & 3) * 8 + (tid & 7);
+      const bool ok = r0 + r < rows && k0 + k < K;
+      const float* src = MN ? P + (size_t)(k0 + k) * ld + r0 + r : P + (size_t)(r0 + r) * ld + k0 + k;
+      cp_async4(S + k * LD + r, ok ? src : P, ok ? 4 : 0);
+    }
+  }
+}
+
+// MN: both operands MN-major (the weight gradient), else both K-major.
+template <int T, int KGRP, bool MN, int MODE>
+__global__ void __launch_bounds__(NT, 2)
+    k_simt_gemm(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb, int M, int N, int K,
+                int vecs, EpiArgs ep) {
+  using C = Cfg<T, KGRP>;
+  extern __shared__ __align__(16) float sm[];
+  const int m0 = blockIdx.x * C::TM, n0 = blockIdx.y * C::TN;
+  // this CTA's share of K: split blockIdx.z of gridDim.z (whole stages)
+  const int S = gridDim.z;
+  const int steps = (K + TKS - 1) / TKS;
+  const int per = (steps + S - 1) / S;
+  const int s0 = min(steps, (int)blockIdx.z * per), ns = min(steps, s0 + per) - s0;
+  const int tid = threadIdx.x;
+  const int grp = tid / (C::TT * C::TT), t = tid % (C::TT * C::TT);
+  const int tx = t % C::TT, ty = t / C::TT;
+  const bool va = vecs & 1, vb = vecs & 2;
+  ptx::griddep_wait();  // launched with programmatic stream serialization
+
+  auto stage = [&](int s) {
+    float* a = sm + (s % C::STAGES) * 2 * C::OP;
+    load_tile<T, MN>(a, A, lda, M, K, m0, (s0 + s) * TKS, va);
+    load_tile<T, MN>(a + C::OP, B, ldb, N, K, n0, (s0 + s) * TKS, vb);
+  };
 #pragma unroll
-    for (int k = 0; k < TK; ++k) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][k][ty * 4]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][k][64 + ty * 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][k][tx * 4]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][k][64 + tx * 4]);
-      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+  for (int s = 0; s < C::STAGES - 1; ++s) {
+    if (s < ns) stage(s);
+    cp_commit();
+  }
+
+  // outputs of row pair (rows 4 ty + {0,1}, {2,3}, TM/2 + 4 ty + {0,1}, {2,3})
+  // and column j (4 tx + j for j < 4, TN/2 + 4 tx + j - 4 above)
+  unsigned long long acc[4][8];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0ull;
+
+  for (int s = 0; s < ns; ++s) {
+    cp_wait<C::STAGES - 2>();
+    __syncthreads();  // stage s has landed for everyone, and everyone is done with stage s - 1
+    if (s + C::STAGES - 1 < ns) stage(s + C::STAGES - 1);
+    cp_commit();
+    const float* as = sm + (s % C::STAGES) * 2 * C::OP;
+    const float* bs = as + C::OP;
+    constexpr int KPG = TKS / C::KG;  // K per group and stage
+    const float* ap = as + grp * KPG * C::LD + ty * 4;
+    const float* bp = bs + grp * KPG * C::LD + tx * 4;
+#pragma unroll 8
+    for (int k = 0; k < KPG; ++k) {
+      const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(ap + k * C::LD);
+      const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(ap + k * C::LD + T / 2);
+      const float4 b0 = *reinterpret_cast<const float4*>(bp + k * C::LD);
+      const float4 b1 = *reinterpret_cast<const float4*>(bp + k * C::LD + T / 2);
+      const unsigned long long a[4] = {a0.x, a0.y, a1.x, a1.y};
       const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int j = 0; j < 8; ++j) {
+        const unsigned long long bb = pack2(b[j], b[j]);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    if (more) {
-      store_tile<A_MN>(As[buf ^ 1], ra);
-      store_tile<B_MN>(Bs[buf ^ 1], rb);
-    }
-    __syncthreads();
-  }
-
-  if (S > 1) {
-    // partial tile out (each thread its own 64 values), then the last CTA of
-    // the tile adds the S partials in split order
-    const int tile = blockIdx.y * gridDim.x + blockIdx.x;
-    const size_t ntile = (size_t)gridDim.x * gridDim.y;
-    float* mine = ep.kpart + ((size_t)blockIdx.z * ntile + tile) * (TM * TN) + threadIdx.x * 64;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      *reinterpret_cast<float4*>(mine + i * 8) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-      *reinterpret_cast<float4*>(mine + i * 8 + 4) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
-    }
-    __shared__ int last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(ep.kcnt + tile, 1) == S - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    if (threadIdx.x == 0) ep.kcnt[tile] = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-      for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-    for (int z = 0; z < S; ++z) {
-      const float* p = ep.kpart + ((size_t)z * ntile + tile) * (TM * TN) + threadIdx.x * 64;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float4 u = __ldcg(reinterpret_cast<const float4*>(p + i * 8));
-        const float4 v = __ldcg(reinterpret_cast<const float4*>(p + i * 8 + 4));
-        acc[i][0] += u.x; acc[i][1] += u.y; acc[i][2] += u.z; acc[i][3] += u.w;
-        acc[i][4] += v.x; acc[i][5] += v.y; acc[i][6] += v.z; acc[i][7] += v.w;
+        for (int i = 0; i < 4; ++i) fma2(acc[i][j], a[i], bb);
       }
     }
   }
+  cp_wait<0>();
+  if (tid == 0) ptx::griddep_launch_dependents();  // the mainloop is done
+  __syncthreads();  // the ring is idle: the partial tile takes its place
 
+  float* mine = sm + grp * C::TM * C::LD;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int gi = m0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
+  for (int i = 0; i < 4; ++i) {
+    float2 v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = unpack2(acc[i][j]);
+    float* p = mine + ((i >> 1) * (C::TM / 2) + ty * 4 + (i & 1) * 2) * C::LD + tx * 4;
+    *reinterpret_cast<float4*>(p) = make_float4(v[0].x, v[1].x, v[2].x, v[3].x);
+    *reinterpret_cast<float4*>(p + C::TN / 2) = make_float4(v[4].x, v[5].x, v[6].x, v[7].x);
+    *reinterpret_cast<float4*>(p + C::LD) = make_float4(v[0].y, v[1].y, v[2].y, v[3].y);
+    *reinterpret_cast<float4*>(p + C::LD + C::TN / 2) = make_float4(v[4].y, v[5].y, v[6].y, v[7].y);
+  }
+  __syncthreads();
+  constexpr int LPR = C::TN / 4;   // lanes per row in the steps below (4 columns each)
+  constexpr int RPP = NT / LPR;    // rows per pass
+  const int lr = tid / LPR, lc = (tid % LPR) * 4;
+  if constexpr (C::KG > 1) {
+    // the K groups' partials, in group order, into the first
+#pragma unroll
+    for (int r = lr; r < C::TM; r += RPP) {
+      float* p = sm + r * C::LD + lc;
+      float4 v = *reinterpret_cast<const float4*>(p);
+#pragma unroll
+      for (int g = 1; g < C::KG; ++g) {
+        const float4 u = *reinterpret_cast<const float4*>(p + g * C::TM * C::LD);
+        v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+      }
+      *reinterpret_cast<float4*>(p) = v;
+    }
+  }
+  if (S > 1)
+    ptx::cluster_sync();  // every partial of the tile is in place
+  else
+    __syncthreads();
+
+  // the epilogue on this CTA's TM / S rows of the tile
+  const int RS = C::TM / S;
+  for (int p = 0; p < RS; p += RPP) {
+    const int r = (int)blockIdx.z * RS + p + lr;
+    const bool row_ok = p + lr < RS && m0 + r < M;
+    const int gi = m0 + r;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    if (row_ok) {
+      if (S > 1) {
+        float4 u[kMaxSplit];
+#pragma unroll
+        for (int z = 0; z < kMaxSplit; ++z)
+          if (z < S) u[z] = ld_cluster4(sm + r * C::LD + lc, (uint32_t)z);
+#pragma unroll
+        for (int z = 0; z < kMaxSplit; ++z)
+          if (z < S) {
+            v[0] += u[z].x; v[1] += u[z].y; v[2] += u[z].z; v[3] += u[z].w;
+          }
+      } else {
+        const float4 u = *reinterpret_cast<const float4*>(sm + r * C::LD + lc);
+        v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
+      }
+    }
+    const int col = n0 + lc;
     if (MODE == MODE_FWD) {
       float g = 0.f;
-      if (gi < M) {
-        const float s = ep.row_scale[gi];
-        float* out = reinterpret_cast<float*>(ep.out) + (size_t)gi * ep.ldo;
+      if (row_ok) {
+        const float s = __ldg(ep.row_scale + gi);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int col = n0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + (j - 4));
+        for (int e = 0; e < 4; ++e) {
           float h = 0.f;
-          if (col < N) {
-            float z = s * acc[i][j];
-            if (ep.bias) z += __ldg(ep.bias + col);
+          if (col + e < N) {
+            float z = s * v[e];
+            if (ep.bias) z += __ldg(ep.bias + col + e);
             h = z != z ? z : fmaxf(z, 0.f);  // ReLU, NaN kept for the non-finite check
           }
           g = fmaf(h, h, g);
-          if (col < ep.ldo) out[col] = h;
+          v[e] = h;
         }
+        // activation rows are padded to multiples of 8: whole 16-byte words
+        if (col < ep.ldo)
+          *reinterpret_cast<float4*>(static_cast<float*>(ep.out) + (size_t)gi * ep.ldo + col) =
+              make_float4(v[0], v[1], v[2], v[3]);
       }
-      // the 16 threads sharing this row are lanes tx = 0..15 of one half-warp
+      // the LPR lanes sharing this row
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-      if (tx == 0 && gi < M) ep.gpart[(size_t)blockIdx.x * M + gi] = g;
-    } else {
-      if (gi < M) {
-        float* out = reinterpret_cast<float*>(ep.out) + (size_t)gi * ep.ldo;
+      for (int o = LPR / 2; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+      if (lc == 0 && row_ok) ep.gpart[(size_t)blockIdx.y * M + gi] = g;
+    } else if (row_ok) {
+      float* out = static_cast<float*>(ep.out) + (size_t)gi * ep.ldo + col;
+      if ((ep.ldo & 3) == 0 && col + 4 <= N) {
+        *reinterpret_cast<float4*>(out) = make_float4(v[0], v[1], v[2], v[3]);
+      } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int col = n0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + (j - 4));
-          if (col < N) out[col] = acc[i][j];
-        }
+        for (int e = 0; e < 4; ++e)
+          if (col + e < N) out[e] = v[e];
       }
     }
   }
+  if (S > 1) ptx::cluster_sync();  // no CTA leaves while another reads its partial tile
 }
 
-template <bool A_MN, bool B_MN, int MODE>
-cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int N, int K, const EpiArgs& ep,
+// Tile shape and number of K slices for an M x N output over K: the least
+// modelled time.  Measured: a CTA takes 0.95 us per stage of a 64 x 64 tile
+// and 3.3 us of a 128 x 128 one (42 and 48 TFLOP/s over 152 SMs) whether or
+// not it shares its SM -- the shared-memory operand reads and the FMAs fill
+// the SM's time -- so a GEMM takes the stages that the fullest SM runs; a
+// split costs about 1 us more.  Eight slices measured no faster than four at
+// any size (forward of 128 rows, 784 -> 500: 15.2 us with 4, 16.6 with 8;
+// clusters of 8 find fewer places).  That forward took 22 us with one CTA
+// per 128 x 128 tile and slice and partials through device memory; 512 rows
+// of 2000 -> 2000 122 us against 113 now, their weight gradient 118 against
+// 94.
+struct Plan {
+  bool large;
+  int S;
+};
+Plan plan_of(int M, int N, int K) {
+  const int steps = cdiv(K, TKS);
+  Plan best{true, 1};
+  double bt = 0.0;
+  for (int large = 1; large >= 0; --large) {
+    const int T = large ? 128 : 64;
+    const double tiles = (double)cdiv(M, T) * cdiv(N, T);
+    for (int S = 1; S <= kMaxSplit; S *= 2) {
+      if (S > 1 && steps < 2 * S) break;
+      const double per_sm = cdiv((long long)(tiles * S), 152);  // CTAs an SM runs in all
+      const double t = per_sm * cdiv(steps, S) * (large ? 3.3 : 0.95) + (S > 1 ? 1.0 : 0.0);
+      if (bt == 0.0 || t < bt) {
+        bt = t;
+        best = Plan{large != 0, S};
+      }
+    }
+  }
+  return best;
+}
+
+template <int T, int KGRP, bool MN, int MODE>
+cudaError_t launch_plan(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, const EpiArgs& ep,
+                        cudaStream_t st) {
+  using C = Cfg<T, KGRP>;
+  static const cudaError_t attr = cudaFuncSetAttribute(k_simt_gemm<T, KGRP, MN, MODE>,
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+  if (attr != cudaSuccess) return attr;
+  auto vec = [](const float* p, int ld) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (ld & 3) == 0; };
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cdiv(M, T), cdiv(N, T), S);
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = C::SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = 1;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = S;
+  cfg.attrs = at;
+  cfg.numAttrs = S > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, k_simt_gemm<T, KGRP, MN, MODE>, A, lda, B, ldb, M, N, K,
+                            (vec(A, lda) ? 1 : 0) | (vec(B, ldb) ? 2 : 0), ep);
+}
+
+template <bool MN, int MODE>
+cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int N, int K, Plan p, const EpiArgs& ep,
                    cudaStream_t st) {
-  const int tiles = cdiv(N, TN) * cdiv(M, TM);
-  int S = ep.kpart && ep.kcnt ? split_of(M, N, K) : 1;
-  if (S > 1 && ((size_t)S * tiles * TM * TN > ep.kpart_cap || tiles > ep.kcnt_cap)) S = 1;
-  dim3 grid(cdiv(N, TN), cdiv(M, TM), S);
-  k_simt_gemm<A_MN, B_MN, MODE><<<grid, NT, 0, st>>>(A, lda, B, ldb, M, N, K, ep);
-  return cudaGetLastError();
+  if (p.large) return launch_plan<128, 1, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, st);
+  return launch_plan<64, 4, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, st);
 }
 
 }  // namespace
 
-int simt_fwd_ntiles(int N) { return cdiv(N, TN); }
-size_t simt_split_floats(int M, int N, int K) {
-  const int S = split_of(M, N, K);
-  return S > 1 ? (size_t)S * cdiv(N, TN) * cdiv(M, TM) * TM * TN : 0;
-}
-int simt_split_tiles(int M, int N) { return cdiv(N, TN) * cdiv(M, TM); }
+int simt_fwd_ntiles(int M, int N, int K) { return cdiv(N, plan_of(M, N, K).large ? 128 : 64); }
+int simt_fwd_ntiles_max(int N) { return cdiv(N, 64); }
 
-cudaError_t simt_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, const EpiArgs& ep,
-                          cudaStream_t st) {
-  return launch<false, false, MODE_FWD>(A, lda, B, ldb, M, N, K, ep, st);
+cudaError_t simt_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
+                          const EpiArgs& ep, cudaStream_t st) {
+  return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, plan_of(plan_rows, N, K), ep, st);
 }
 
 cudaError_t simt_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, float* C, int ldc,
                             cudaStream_t st) {
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  return launch<false, false, MODE_STORE>(A, lda, B, ldb, M, N, K, ep, st);
+  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, plan_of(M, N, K), ep, st);
 }
 
 cudaError_t simt_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, float* C, int ldc,
-                            cudaStream_t st, const EpiArgs* split) {
+                            cudaStream_t st) {
   // C[N, K] = sum_r G[r, n] X[r, k]: rows of C index G's columns (MN-major A),
   // columns of C index X's columns (MN-major B), contraction over R.
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  if (split) {
-    ep.kpart = split->kpart;
-    ep.kpart_cap = split->kpart_cap;
-    ep.kcnt = split->kcnt;
-    ep.kcnt_cap = split->kcnt_cap;
-  }
-  return launch<true, true, MODE_STORE>(G, ldg, X, ldx, N, K, R, ep, st);
+  return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, plan_of(N, K, R), ep, st);
 }
 
 }  // namespace ff

@@ -793,7 +793,7 @@ ff_status head_workspace(ff_head* hd, ff_layer* const* layers, int L, int rows, 
   const size_t es = b16 ? 2 : 4;
   int ntmax = 0;
   for (int k = 0; k < L; ++k) {
-    const int nt = b16 ? tc_fwd_ntiles_max(layers[k]->N) : simt_fwd_ntiles(layers[k]->N);
+    const int nt = b16 ? tc_fwd_ntiles_max(layers[k]->N) : simt_fwd_ntiles_max(layers[k]->N);
     if (nt > ntmax) ntmax = nt;
   }
   size_t off = 0;
@@ -837,7 +837,9 @@ ff_status head_workspace(ff_head* hd, ff_layer* const* layers, int L, int rows, 
 // 128-column tiles when their grid is small (predict); training keeps
 // 256-column tiles at every row count, so that a row's goodness partials --
 // and with them every activity scale -- do not depend on how many rows share
-// the GEMM (ff_head_train_epoch runs many steps' rows at once).
+// the GEMM (ff_head_train_epoch runs many steps' rows at once); the fp32
+// GEMMs then take the tile shape of kTrainPlanRows rows at any row count.
+constexpr int kTrainPlanRows = 1024;
 ff_status head_forward(ff_layer* const* layers, int L, const float* x, int rows, const HeadWork& w, int* err,
                        cudaStream_t st, bool narrow) {
   ff_layer* L0 = layers[0];
@@ -867,9 +869,11 @@ ff_status head_forward(ff_layer* const* layers, int L, const float* x, int rows,
                 tc_gemm_fwd(static_cast<const bf16*>(in), Lk->ldK, Lk->Wb, Lk->ldK, rows, Lk->N, Lk->K, ep, err, st),
                 "head forward GEMM (tcgen05)");
     } else {
-      nt = simt_fwd_ntiles(Lk->N);
+      const int plan_rows = narrow ? rows : kTrainPlanRows;
+      nt = simt_fwd_ntiles(plan_rows, Lk->N, Lk->K);
       FF_LAUNCH(K_FWD_SIMT, 2.0 * rows * Lk->N * Lk->K, st,
-                simt_gemm_fwd(static_cast<const float*>(in), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, ep, st),
+                simt_gemm_fwd(static_cast<const float*>(in), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, plan_rows, ep,
+                              st),
                 "head forward GEMM (fp32)");
     }
     nt_prev = nt;
@@ -1388,9 +1392,9 @@ ff_status ff_po_train_step(ff_layer* L, ff_head* hd, const void* x, int raw_inpu
               tc_gemm_fwd(static_cast<const bf16*>(X), L->ldK, L->Wb, L->ldK, n, N, K, ep, &L->ds->err, st),
               "forward GEMM (tcgen05)");
   } else {
-    ntiles = simt_fwd_ntiles(N);
+    ntiles = simt_fwd_ntiles(n, N, K);
     FF_LAUNCH(K_FWD_SIMT, 2.0 * n * N * K, st,
-              simt_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, n, N, K, ep, st), "forward GEMM (fp32)");
+              simt_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, n, N, K, n, ep, st), "forward GEMM (fp32)");
   }
   if (!b16) {
     // the block on the raw activity: logits, cross-entropy, dz

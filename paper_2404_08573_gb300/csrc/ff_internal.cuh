@@ -261,13 +261,6 @@ struct EpiArgs {
   int ntiles_in;
   float* G_acc;
   float* s_out;
-  // fp32 SIMT GEMMs only: split-K scratch (partial tiles, capacity in floats,
-  // and one arrival counter per output tile, zero between launches); null: no
-  // split.
-  float* kpart;
-  size_t kpart_cap;
-  int* kcnt;
-  int kcnt_cap;
   // Tensor-core forward GEMMs: a grid that would fill at most half the SMs
   // may use 128-column tiles (twice the CTAs).  Set where the GEMM has the
   // GPU to itself (the layer chains of predict and of the softmax head); the
@@ -329,19 +322,19 @@ bool make_plain_map(CUtensorMap* m, const void* ptr, int esize, int cols, int ro
 bool make_sw128_map(CUtensorMap* m, const void* ptr, int esize, int cols, int rows, int ld, int box_cols,
                     int box_rows);
 
-// SIMT fp32 GEMMs with the same contracts.  A GEMM of few output tiles
-// splits its contraction over blockIdx.z when the EpiArgs carry split-K
-// scratch of the size simt_split_floats / simt_split_tiles give (the wgrad
-// form takes the scratch from `split`).
-int simt_fwd_ntiles(int N);
-size_t simt_split_floats(int M, int N, int K);
-int simt_split_tiles(int M, int N);
-cudaError_t simt_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K,
+// SIMT fp32 GEMMs with the same contracts.  The tile shape and the split of
+// the contraction depend on the output's shape; for the forward, on plan_rows
+// rows instead of M, so that a chain whose per-row results must not depend on
+// how many rows share a GEMM passes a constant.  simt_fwd_ntiles(plan_rows,
+// ...): goodness partials per row it then writes; _max: the most for any rows.
+int simt_fwd_ntiles(int plan_rows, int N, int K);
+int simt_fwd_ntiles_max(int N);
+cudaError_t simt_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
                           const EpiArgs& ep, cudaStream_t st);
 cudaError_t simt_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K,
                             float* C, int ldc, cudaStream_t st);
 cudaError_t simt_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K,
-                            float* C, int ldc, cudaStream_t st, const EpiArgs* split = nullptr);
+                            float* C, int ldc, cudaStream_t st);
 
 }  // namespace ff
 
@@ -373,9 +366,6 @@ struct ff_layer {
   float* stat_part;  // [row blocks * (2 + column blocks)] step statistics partials
   // predict scratch (owned here when this layer is layers[0] of ff_predict)
   void* pws; size_t pws_bytes;
-  // split-K scratch of the fp32 GEMMs (grown on demand; counters kept zero)
-  float* kpart; size_t kpart_cap;
-  int* kcnt; int kcnt_cap;
   // bf16 train steps: the local gradient in the forward GEMM's epilogue
   // (tc_gemm_fwd_lg) where the shape allows, else the separate kernel.  Off
   // by default: on the 784-2000x4 epoch with 4 layer streams the fused

@@ -1,0 +1,53 @@
+"""The fp32 CUDA-core GEMMs at the edges of their tiles, stages and K slices:
+forward and weight gradient of an fp32 layer against float64 products, within
+the bound of a K-term fp32 sum (K + 8 roundings of 2^-24 of the terms'
+absolute sum, whatever the order)."""
+
+import numpy as np
+import pytest
+
+from tests.gpu_common import U32, lib_ready, torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+# rows 2B, K, N: one tile and less; tile edges +-1; widths off every
+# multiple of 4 (unaligned weight rows); one and several K slices, ragged
+# stages; outputs of many large tiles
+SHAPES = [(2, 10, 8), (2, 33, 1), (62, 31, 63), (64, 32, 64), (66, 65, 65), (128, 784, 500), (130, 786, 129),
+          (254, 1001, 127), (256, 256, 2000), (600, 129, 1023), (1538, 300, 1027)]
+
+
+@pytest.mark.parametrize("M,K,N", SHAPES)
+def test_fp32_forward_and_weight_gradient_at_tile_edges(M, K, N):
+    torch = torch_cuda()
+    ff = lib_ready()
+    g = torch.Generator("cuda").manual_seed(M * 7 + K * 3 + N)
+    layer = ff.Layer(K, N, prec="fp32", theta=2.0, lr=1e-3, keep_grad=True, max_rows=M)
+    x = layer.new_activation(M, K)
+    x[:, K:] = float("nan")  # the padding of an activation row is never read
+    x[:, :K] = torch.rand(M, K, device="cuda", generator=g)
+    s = (1.0 / torch.linalg.vector_norm(x[:, :K], dim=1)).contiguous()
+    st = layer.get_state()
+    b = (np.random.default_rng(1).standard_normal(N) * 0.05).astype(np.float32)
+    layer.set_state(W=st["W"], b=b)
+    W = torch.from_numpy(st["W"]).cuda().double()
+    h = layer.new_activation(M)
+    h.fill_(7.0)
+    good = torch.empty(M, device="cuda")
+    layer.train_step(x, row_scale=s, B=M // 2, h_out=h, goodness=good)
+    torch.cuda.synchronize()
+    layer.check()
+    xs = x[:, :K].double() * s.double()[:, None]
+    bd = torch.from_numpy(b).cuda().double()
+    ref = torch.relu(xs @ W.T + bd)
+    bound = (K + 8) * U32 * (xs.abs() @ W.abs().T + bd.abs())
+    assert bool(((h[:, :N].double() - ref).abs() <= bound).all())
+    assert bool((h[:, N:] == 0).all())
+    gref = (ref * ref).sum(1)
+    gb = (2 * ref * bound + bound ** 2).sum(1) + (N + 8) * U32 * gref
+    assert bool(((good.double() - gref).abs() <= gb).all())
+    # the weight gradient of the GPU's own operand
+    G = torch.from_numpy(layer.get_grad_operand(M)).cuda()[:, :N]
+    dW = torch.from_numpy(layer.get_grad()[0]).cuda().double()
+    xd = x[:, :K].double()
+    assert bool(((dW - G.T @ xd).abs() <= (M + 8) * U32 * (G.abs().T @ xd.abs())).all())
