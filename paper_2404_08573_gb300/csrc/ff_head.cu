@@ -17,9 +17,11 @@
 //                  z = c + the splits' partials (in split order), softmax,
 //                  per-row loss and dz = (softmax(z) - onehot(y)) / n, and
 //                  the row block's partials of dc and of the loss
-//   k_head_wgrad   dV partials per 64-row block: dz^T (s_k H_k)
+//   k_head_dot_mma the same on bf16 activities, with tensor-core MMAs
+//   k_head_wgrad   dV partials per 64-row block: dz^T (s_k H_k) (fp32)
 //   k_head_adam    reduces the partials in a fixed order, Adam on V and c,
 //                  the step's loss
+//   k_head_wgrad_adam  both in one launch on bf16 activities
 //   k_po_grad      the Performance-Optimized step (§4): the gradient through
 //                  a layer's own block into the layer and the block's dV
 //                  partials; with bf16 layers it first finishes its rows'
@@ -41,7 +43,8 @@ namespace {
 constexpr int kClasses = 10;
 constexpr int kMaxSegs = 16;
 constexpr int kDotRows = 64;     // rows per block of k_head_dot (eight per warp)
-constexpr int kSplit = 1024;     // widest feature split of one segment per k_head_dot block
+constexpr int kSplit = 1024;     // widest feature split of one segment per k_head_dot block (fp32)
+constexpr int kMmaSplit = 512;   // and per k_head_dot_mma block (bf16)
 constexpr int kDotMinBlocks = 152 / 2;  // k_head_dot grids narrower than this split features finer
 constexpr int kWgRows = 64;      // rows per block of k_head_wgrad (8 per warp)
 constexpr int kWgChunk = 128;    // features per block of k_head_wgrad (4 per lane)
@@ -61,26 +64,8 @@ struct Segs {
 };
 
 
-// h[0..W) = H[row, f .. f+W) as float, zero past the segment or the rows.
-template <typename T, int W>
-__device__ __forceinline__ void load_feats(const T* __restrict__ H, int ld, int row, int n, int f, int F, float* h);
-template <>
-__device__ __forceinline__ void load_feats<bf16, 4>(const bf16* __restrict__ H, int ld, int row, int n, int f, int F,
-                                                    float* h) {
-  if (row < n && f + 4 <= F) {
-    const uint2 q = __ldg(reinterpret_cast<const uint2*>(H + (size_t)row * ld + f));
-    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q.x));
-    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q.y));
-    h[0] = a.x; h[1] = a.y; h[2] = b.x; h[3] = b.y;
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      h[i] = (row < n && f + i < F) ? __bfloat162float(H[(size_t)row * ld + f + i]) : 0.f;
-  }
-}
-template <>
-__device__ __forceinline__ void load_feats<float, 4>(const float* __restrict__ H, int ld, int row, int n, int f, int F,
-                                                     float* h) {
+// h[0..4) = H[row, f .. f+4), zero past the segment or the rows.
+__device__ __forceinline__ void load_feats4(const float* __restrict__ H, int ld, int row, int n, int f, int F, float* h) {
   if (row < n && f + 4 <= F) {
     const float4 a = __ldg(reinterpret_cast<const float4*>(H + (size_t)row * ld + f));
     h[0] = a.x; h[1] = a.y; h[2] = a.z; h[3] = a.w;
@@ -90,9 +75,9 @@ __device__ __forceinline__ void load_feats<float, 4>(const float* __restrict__ H
   }
 }
 
-// Softmax, loss and dz of one row from its logits (z has the bias added).
+// Softmax, loss and dz of one row with label y from its logits (z has the bias added).
 // Writes logits/dz when given; returns the row's loss (0 without a label).
-__device__ __forceinline__ float finish_row(const float (&z)[kClasses], int row, const int* __restrict__ labels,
+__device__ __forceinline__ float finish_row(const float (&z)[kClasses], int row, bool labelled, int y,
                                             float inv_n, float* __restrict__ logits, float* __restrict__ dz,
                                             float (&dzr)[kClasses], int* err) {
   bool finite = true;
@@ -103,7 +88,7 @@ __device__ __forceinline__ float finish_row(const float (&z)[kClasses], int row,
     dzr[c] = 0.f;
   }
   if (!finite) atomicOr(err, DEVERR_NONFINITE);
-  if (!labels) return 0.f;
+  if (!labelled) return 0.f;
   float m = z[0];
 #pragma unroll
   for (int c = 1; c < kClasses; ++c) m = fmaxf(m, z[c]);
@@ -113,7 +98,6 @@ __device__ __forceinline__ float finish_row(const float (&z)[kClasses], int row,
     e[c] = expf(z[c] - m);
     sum += e[c];
   }
-  const int y = labels[row];
   const float inv = 1.f / sum;
   float zy = 0.f;
 #pragma unroll
@@ -133,16 +117,14 @@ __host__ __device__ inline int head_splits(const int* F, int nseg, int split) {
   return S;
 }
 
-// Split width of k_head_dot for n rows: kSplit, halved (down to one 512-byte
-// chunk, 512 / es features) while the grid would cover less than half the
-// SMs, so that few rows are spread over the SMs by features.  (A block's
-// fixed costs -- its slice of V, the cross-lane sums -- make narrower splits
-// slower once the grid covers the GPU: 6000 features x 1024 rows run fastest
-// at 96 blocks of 1024 features, 2000 x 1024 at 128 blocks of 256.)
+// Split width of the logits kernels for n rows: the widest (kSplit features,
+// bf16 kMmaSplit), halved (down to 128, bf16 256) while the grid would cover
+// less than half the SMs, so that few rows are spread over the SMs by
+// features.
 int dot_split(const int* F, int nseg, int n, int es) {
-  const int ch = 512 / es;
+  const int ch = es == 2 ? 256 : 128;
   const long long rb = (n + kDotRows - 1) / kDotRows;
-  int split = kSplit;
+  int split = es == 2 ? kMmaSplit : kSplit;
   while (split > ch && head_splits(F, nseg, split) * rb < kDotMinBlocks) split /= 2;
   return split;
 }
@@ -169,14 +151,174 @@ struct FinishArgs {
   float* logits;  // [n, 10] or null
   float* dz;      // [n, 10] or null
   float* part;    // [row blocks, 11] or null
+  uint4* dzfrag;  // [segment][16-row group][part][lane]: A operands of k_head_wgrad_adam, or null
   ff_dev_state* ds;
   float beta1, beta2;
   int* counter;
   int S;          // blocks (splits) per row block
 };
 
-// One tensor map per segment: H_k as [n, ld_k] with 64-row boxes of 512
-// bytes (256 bf16 or 128 fp32 features), no swizzle.
+// ------------------------------------------------ bf16 activities: tensor cores
+// The head's two contractions are thin (10 classes) and latency-bound: 1024
+// rows of 6000 features are 12 MB of activity from L2 and 0.06 GFLOP each.
+// They run as warp-level m16n8k16 MMAs fed straight from L2: a 128-row
+// tcgen05 tile would leave most SMs idle and wait on TMEM and barrier set-up.
+// The fp32 operand (V, or dz times the row scale) enters as three bf16 parts
+// of 8 mantissa bits each, x = hi + mid + lo exactly, whose products with the
+// activity are exact and summed in fp32: nothing is lost against fp32 FMAs.
+__device__ __forceinline__ void split3(float x, bf16 (&p)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const float top = __uint_as_float(__float_as_uint(x) & 0xFFFF0000u);
+    p[i] = __float2bfloat16_rn(top);  // exact
+    x = isfinite(top) ? __fsub_rn(x, top) : 0.f;
+  }
+}
+__device__ __forceinline__ uint32_t pack_bf16(bf16 lo, bf16 hi) {
+  const __nv_bfloat162 v = __halves2bfloat162(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+// D (16 x 8, fp32) += A (16 x 16, bf16) B (16 x 8, bf16).  Lane 4 g + t holds
+// of A rows g and g + 8 at K slots 2t, 2t+1 (a0, a1) and 2t+8, 2t+9 (a2, a3),
+// of B column g at the same slots (b0, b1), of D rows g (d0, d1) and g + 8
+// (d2, d3) at columns 2t, 2t+1.
+__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                         uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+constexpr int mma_smem(int split) { return split / 16 * 3 * 32 * 16; }
+
+// The end of every logits block (256 threads) of row block blockIdx.y, rows
+// rblk .. rblk + 63: the last of the row block's fa.S blocks to arrive forms
+// its rows' logits from the splits' partials and finishes them.
+__device__ __forceinline__ void finish_row_block(const Segs& sg, const float* __restrict__ zpart, int n, int rblk,
+                                                 const FinishArgs& fa, int* err) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // Every block arrives (an aborted one too, so that the counter is reset);
+  // the last of the row block's S blocks finishes its rows.
+  __shared__ int last;
+  __shared__ float fred[kDotRows / 32][kPart];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(fa.counter + blockIdx.y, 1) == fa.S - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (threadIdx.x == 0) {
+    fa.counter[blockIdx.y] = 0;
+    if (blockIdx.y == 0 && fa.labels && fa.ds) {
+      // this step's Adam counter and bias corrections, read by k_head_adam
+      fa.ds->t += 1;
+      fa.ds->pow1 *= (double)fa.beta1;
+      fa.ds->pow2 *= (double)fa.beta2;
+      fa.ds->bc1 = (float)(1.0 - fa.ds->pow1);
+      fa.ds->bc2 = (float)(1.0 - fa.ds->pow2);
+    }
+  }
+  // z = c + the splits' partials in split order, a thread per row and class
+  // (read past L1: other blocks wrote them during this launch), eight splits'
+  // loads in flight at a time
+  __shared__ float zs[kDotRows][kClasses];
+  // the segments' row scales and the labels, loaded beside the partials
+  __shared__ float ss[kMaxSegs][kDotRows];
+  __shared__ int ys[kDotRows];
+  if (fa.dzfrag)
+    for (int u = threadIdx.x; u < sg.nseg * kDotRows; u += 256) {
+      const int k = u / kDotRows, r = u % kDotRows;
+      ss[k][r] = rblk + r < n ? (sg.s[k] ? __ldg(sg.s[k] + rblk + r) : 1.f) : 0.f;
+    }
+  if (fa.labels && threadIdx.x < kDotRows && rblk + (int)threadIdx.x < n)
+    ys[threadIdx.x] = __ldg(fa.labels + rblk + threadIdx.x);
+  {
+    constexpr int NI = (kDotRows * kClasses + 255) / 256;
+    const int items = min(kDotRows, n - rblk) * kClasses;
+    const float* zp = zpart + (size_t)rblk * kClasses + threadIdx.x;
+    const size_t zs_stride = (size_t)n * kClasses;
+    float z[NI];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) z[i] = __ldg(fa.cb + (threadIdx.x + i * 256) % kClasses);
+    for (int sp0 = 0; sp0 < fa.S; sp0 += 8) {
+      float v[NI][8];
+#pragma unroll
+      for (int i = 0; i < NI; ++i)
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          v[i][u] = sp0 + u < fa.S && (int)threadIdx.x + i * 256 < items ? __ldcg(zp + i * 256 + (sp0 + u) * zs_stride)
+                                                                         : 0.f;
+#pragma unroll
+      for (int i = 0; i < NI; ++i)
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (sp0 + u < fa.S) z[i] += v[i][u];
+    }
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+      if ((int)threadIdx.x + i * 256 < items) (&zs[0][0])[threadIdx.x + i * 256] = z[i];
+  }
+  __syncthreads();
+  // a thread per row: softmax, loss and dz (left in zs too)
+  if (threadIdx.x < kDotRows) {
+    const int row = rblk + (int)threadIdx.x;
+    float dzr[kClasses];
+    float loss = 0.f;
+#pragma unroll
+    for (int c = 0; c < kClasses; ++c) dzr[c] = 0.f;
+    if (row < n) {
+      float z[kClasses];
+#pragma unroll
+      for (int c = 0; c < kClasses; ++c) z[c] = zs[threadIdx.x][c];
+      loss = finish_row(z, row, fa.labels != nullptr, fa.labels ? ys[threadIdx.x] : 0, fa.inv_n, fa.logits, fa.dz, dzr, err);
+    }
+    if (fa.part) {
+      // the row block's sums of dz (for dc) and of the loss, in a fixed order
+#pragma unroll
+      for (int c = 0; c < kClasses; ++c) zs[threadIdx.x][c] = dzr[c];
+#pragma unroll
+      for (int c = 0; c < kClasses; ++c) dzr[c] = warp_sum(dzr[c]);
+      loss = warp_sum(loss);
+      if (lane == 0) {
+#pragma unroll
+        for (int c = 0; c < kClasses; ++c) fred[warp][c] = dzr[c];
+        fred[warp][kClasses] = loss;
+      }
+    }
+  }
+  if (!fa.part) return;
+  __syncthreads();
+  if (threadIdx.x < kPart) {
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < kDotRows / 32; ++w) t += fred[w][threadIdx.x];
+    fa.part[(size_t)blockIdx.y * kPart + threadIdx.x] = t;
+  }
+  if (!fa.dzfrag) return;
+  // dz times each segment's row scale as the weight gradient's A operands
+  // (k_head_wgrad_adam): a class and a pair of rows at a time; rows past n
+  // and classes past 9 are zero
+  const int groups = (n + 15) / 16;
+  for (int u = threadIdx.x; u < sg.nseg * (kDotRows / 2) * 16; u += 256) {
+    const int c = u & 15, p = (u >> 4) % (kDotRows / 2), k = (u >> 4) / (kDotRows / 2);
+    const int group = rblk / 16 + (p >> 3);
+    if (group >= groups) continue;
+    bf16 x[2][3];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) split3(c < kClasses ? zs[2 * p + e][c] * ss[k][2 * p + e] : 0.f, x[e]);
+    // a0: class < 8, slots 2t, 2t+1; a1: class >= 8; a2, a3: slots 8 further
+    const int word = (c >> 3) + ((p & 4) ? 2 : 0);
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      reinterpret_cast<uint32_t*>(fa.dzfrag)[((((size_t)k * groups + group) * 3 + q) * 32 + (c & 7) * 4 + (p & 3)) * 4 + word] =
+          pack_bf16(x[0][q], x[1][q]);
+  }
+}
+
+// fp32 activities.  One tensor map per segment: H_k as [n, ld_k] with 64-row
+// boxes of 512 bytes (128 features), no swizzle.
 struct HeadMaps {
   CUtensorMap m[kMaxSegs];
 };
@@ -192,11 +334,10 @@ constexpr int kDotSmem = kDotStages * kDotStageBytes + kSplit * kClasses * 4 + 6
 // have arrived on its `empty` barrier); the split's slice of V sits in shared
 // memory interleaved so that lane l's features (FPL consecutive ones per
 // chunk) are read without bank conflicts.  Every wait is bounded.
-template <typename T>
 __global__ void __launch_bounds__(256, 1) k_head_dot(const __grid_constant__ HeadMaps maps, Segs sg, int split, int n,
                                                      const float* __restrict__ V, float* __restrict__ zpart,
                                                      FinishArgs fa, int* err) {
-  constexpr int CH = 512 / (int)sizeof(T);  // features per chunk
+  constexpr int CH = 512 / 4;  // features per chunk
   constexpr int FPL = CH / 32;              // features per lane
   constexpr int NCH = kSplit / CH;          // chunks in the widest split
   extern __shared__ __align__(128) uint8_t dsm[];
@@ -233,7 +374,7 @@ __global__ void __launch_bounds__(256, 1) k_head_dot(const __grid_constant__ Hea
   ptx::griddep_wait();  // launched with programmatic stream serialization
   if (threadIdx.x == 0) {
     for (; issued < kDotStages && issued < nch; ++issued) {
-      if (!ff_dcheck(tma_x_aligned(fs + issued * CH, (int)sizeof(T)), err)) {
+      if (!ff_dcheck(tma_x_aligned(fs + issued * CH, 4), err)) {
         *abort_flag = 1;
         break;
       }
@@ -274,22 +415,11 @@ __global__ void __launch_bounds__(256, 1) k_head_dot(const __grid_constant__ Hea
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       const uint8_t* rowp = tile + (warp * 8 + r) * 512 + lane * 16;
-      if constexpr (sizeof(T) == 2) {
-        const uint4 q = *reinterpret_cast<const uint4*>(rowp);
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[i]));
-          h[r][2 * i] = v.x * srow[r];
-          h[r][2 * i + 1] = v.y * srow[r];
-        }
-      } else {
-        const float4 q = *reinterpret_cast<const float4*>(rowp);
-        h[r][0] = q.x * srow[r];
-        h[r][1] = q.y * srow[r];
-        h[r][2] = q.z * srow[r];
-        h[r][3] = q.w * srow[r];
-      }
+      const float4 q = *reinterpret_cast<const float4*>(rowp);
+      h[r][0] = q.x * srow[r];
+      h[r][1] = q.y * srow[r];
+      h[r][2] = q.z * srow[r];
+      h[r][3] = q.w * srow[r];
     }
 #pragma unroll
     for (int c = 0; c < kClasses; ++c)
@@ -308,7 +438,7 @@ __global__ void __launch_bounds__(256, 1) k_head_dot(const __grid_constant__ Hea
         atomicOr(err, DEVERR_TIMEOUT);
         break;
       }
-      if (!ff_dcheck(tma_x_aligned(fs + issued * CH, (int)sizeof(T)), err)) {
+      if (!ff_dcheck(tma_x_aligned(fs + issued * CH, 4), err)) {
         *abort_flag = 1;
         break;
       }
@@ -336,81 +466,117 @@ __global__ void __launch_bounds__(256, 1) k_head_dot(const __grid_constant__ Hea
         if (r0 + r < n) zpart[((size_t)blockIdx.x * n + r0 + r) * kClasses + c] = acc[r][c];
     }
   }
-  // Every block arrives (an aborted one too, so that the counter is reset);
-  // the last of the row block's S blocks finishes its rows.
-  __shared__ int last;
-  __shared__ float fred[kDotRows / 32][kPart];
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(fa.counter + blockIdx.y, 1) == fa.S - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  if (threadIdx.x == 0) {
-    fa.counter[blockIdx.y] = 0;
-    if (blockIdx.y == 0 && fa.labels && fa.ds) {
-      // this step's Adam counter and bias corrections, read by k_head_adam
-      fa.ds->t += 1;
-      fa.ds->pow1 *= (double)fa.beta1;
-      fa.ds->pow2 *= (double)fa.beta2;
-      fa.ds->bc1 = (float)(1.0 - fa.ds->pow1);
-      fa.ds->bc2 = (float)(1.0 - fa.ds->pow2);
-    }
+  finish_row_block(sg, zpart, n, rblk, fa, err);
+}
+
+// zpart as k_head_dot writes it, from bf16 activities.  A block takes 64 rows
+// x one split of at most 512 features: warp w the 16 rows 16 (w % 4) .. and
+// half w / 4 of the split.  A lane's 16-byte load of a row (8 features) feeds
+// the K slots of two MMAs, so K runs in a permuted order that the staged V
+// parts follow.  1024 rows x 6000 features: 192 blocks; see dot_split.
+__global__ void __launch_bounds__(256, 2) k_head_dot_mma(Segs sg, int split, int n, const float* __restrict__ V,
+                                                      float* __restrict__ zpart, FinishArgs fa, int* err) {
+  extern __shared__ __align__(16) uint4 vfrag[];  // [K step of 16][part][lane]: b0, b1 of classes 0-7, of 8-15
+  __shared__ float red[kDotRows][kClasses];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = lane >> 2, t = lane & 3;
+  int k = 0, sp = blockIdx.x;
+  while (k + 1 < sg.nseg && sp >= (sg.F[k] + split - 1) / split) {
+    sp -= (sg.F[k] + split - 1) / split;
+    ++k;
   }
-  if (threadIdx.x >= kDotRows) return;
-  // one thread per row: z = c + the splits' partials in split order (read
-  // past L1: other blocks wrote them during this launch)
-  const int row = rblk + (int)threadIdx.x;
-  float dzr[kClasses];
-  float loss = 0.f;
+  const bf16* H = static_cast<const bf16*>(sg.H[k]);
+  const int ld = sg.ld[k];
+  const int fs = sp * split, fe = min(fs + split, sg.F[k]);
+  const int rblk = blockIdx.y * kDotRows;
+  ptx::griddep_wait();  // launched with programmatic stream serialization
+  // this warp's rows over its half of the split, 8 features a lane and row
+  constexpr int NB = kMmaSplit / 2 / 32;  // blocks of 32 features per warp
+  const int half = split / 2;             // a multiple of 32
+  const int f0 = fs + (warp >> 2) * half + 8 * t;
+  const int ra = rblk + (warp & 3) * 16 + g, rb = ra + 8;
+  uint4 ha[NB], hb[NB];
 #pragma unroll
-  for (int c = 0; c < kClasses; ++c) dzr[c] = 0.f;
-  if (row < n) {
-    float z[kClasses];
+  for (int i = 0; i < NB; ++i) {
+    // rows are padded to whole 8-feature words, the padding zero
+    const bool ok = 32 * i < half && f0 + 32 * i < fe;
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+    ha[i] = ok && ra < n ? __ldg(reinterpret_cast<const uint4*>(H + (size_t)ra * ld + f0 + 32 * i)) : z;
+    hb[i] = ok && rb < n ? __ldg(reinterpret_cast<const uint4*>(H + (size_t)rb * ld + f0 + 32 * i)) : z;
+  }
+  // the split's V as B operands: unit (block of 32 features, class, t) holds
+  // features 8t .. 8t+7 of the block, zero past the segment and class 9
+  const float* Vk = V + sg.off[k];
+  const bool vec = ((sg.F_total | sg.off[k]) & 3) == 0;  // V itself is 256-byte aligned
+#pragma unroll 4
+  for (int u = threadIdx.x; u < split / 32 * 64; u += 256) {
+    const int ut = u & 3, c = (u >> 2) & 15, b = u >> 6;
+    const int f = fs + 32 * b + 8 * ut;
+    const float* vp = Vk + (size_t)c * sg.F_total + f;
+    float v[8];
+    if (vec && c < kClasses && f + 8 <= fe) {
+      const float4 lo = __ldg(reinterpret_cast<const float4*>(vp)), hi = __ldg(reinterpret_cast<const float4*>(vp) + 1);
+      v[0] = lo.x; v[1] = lo.y; v[2] = lo.z; v[3] = lo.w;
+      v[4] = hi.x; v[5] = hi.y; v[6] = hi.z; v[7] = hi.w;
+    } else {
 #pragma unroll
-    for (int c = 0; c < kClasses; ++c) z[c] = __ldg(fa.cb + c);
-    // four splits' loads in flight at a time, added in split order
-    for (int sp0 = 0; sp0 < fa.S; sp0 += 4) {
-      float t[4][kClasses];
+      for (int e = 0; e < 8; ++e) v[e] = c < kClasses && f + e < fe ? __ldg(vp + e) : 0.f;
+    }
+    bf16 p[8][3];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float* zp = zpart + ((size_t)(sp0 + u) * n + row) * kClasses;
+    for (int e = 0; e < 8; ++e) split3(v[e], p[e]);
 #pragma unroll
-        for (int c = 0; c < kClasses; ++c) t[u][c] = sp0 + u < fa.S ? __ldcg(zp + c) : 0.f;
+    for (int q = 0; q < 3; ++q)
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        uint2* dst = reinterpret_cast<uint2*>(&vfrag[((2 * b + s) * 3 + q) * 32 + (c & 7) * 4 + ut]) + (c >> 3);
+        *dst = make_uint2(pack_bf16(p[4 * s][q], p[4 * s + 1][q]), pack_bf16(p[4 * s + 2][q], p[4 * s + 3][q]));
       }
+  }
+  __syncthreads();
+  float d[2][4] = {};
+  const uint4* vf = vfrag + (warp >> 2) * (half / 16) * 3 * 32 + lane;
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (sp0 + u < fa.S) {
+  for (int i = 0; i < NB; ++i) {
+    if (32 * i >= half) break;
 #pragma unroll
-          for (int c = 0; c < kClasses; ++c) z[c] += t[u][c];
-        }
+    for (int q = 0; q < 3; ++q) {
+      const uint4 v0 = vf[(2 * i * 3 + q) * 32], v1 = vf[((2 * i + 1) * 3 + q) * 32];
+      mma16816(d[0], ha[i].x, hb[i].x, ha[i].y, hb[i].y, v0.x, v0.y);
+      mma16816(d[1], ha[i].x, hb[i].x, ha[i].y, hb[i].y, v0.z, v0.w);
+      mma16816(d[0], ha[i].z, hb[i].z, ha[i].w, hb[i].w, v1.x, v1.y);
+      mma16816(d[1], ha[i].z, hb[i].z, ha[i].w, hb[i].w, v1.z, v1.w);
     }
-    loss = finish_row(z, row, fa.labels, fa.inv_n, fa.logits, fa.dz, dzr, err);
   }
-  if (!fa.part) return;
-  // the row block's sums of dz (for dc) and of the loss, in a fixed order
+  // the two halves' sums, times the row scale
+  const int lr = (warp & 3) * 16 + g;
+  if (warp >= 4) {
 #pragma unroll
-  for (int c = 0; c < kClasses; ++c) dzr[c] = warp_sum(dzr[c]);
-  loss = warp_sum(loss);
-  if (lane == 0) {
-#pragma unroll
-    for (int c = 0; c < kClasses; ++c) fred[warp][c] = dzr[c];
-    fred[warp][kClasses] = loss;
+    for (int e = 0; e < 4; ++e) {
+      red[lr + (e >> 1) * 8][2 * t + (e & 1)] = d[0][e];
+      if (t == 0) red[lr + (e >> 1) * 8][8 + (e & 1)] = d[1][e];
+    }
   }
-  asm volatile("bar.sync 1, %0;" ::"n"(kDotRows) : "memory");  // the row block's warps only
-  if (threadIdx.x < kPart) {
-    float t = 0.f;
+  __syncthreads();
+  if (warp < 4) {
 #pragma unroll
-    for (int w = 0; w < kDotRows / 32; ++w) t += fred[w][threadIdx.x];
-    fa.part[(size_t)blockIdx.y * kPart + threadIdx.x] = t;
+    for (int r = 0; r < 2; ++r) {
+      const int row = rblk + lr + 8 * r;
+      if (row >= n) continue;
+      const float s = sg.s[k] ? __ldg(sg.s[k] + row) : 1.f;
+      float2* z = reinterpret_cast<float2*>(zpart + ((size_t)blockIdx.x * n + row) * kClasses);
+      const float* o = red[lr + 8 * r];
+      z[t] = make_float2(s * (d[0][2 * r] + o[2 * t]), s * (d[0][2 * r + 1] + o[2 * t + 1]));
+      if (t == 0) z[4] = make_float2(s * (d[1][2 * r] + o[8]), s * (d[1][2 * r + 1] + o[9]));
+    }
   }
+  finish_row_block(sg, zpart, n, rblk, fa, err);
 }
 
 // dV partials of one 128-row block for one 128-feature chunk of one segment:
 // dVpart[rb, c, f] = sum over the block's rows i of dz[i, c] s_k[i] H_k[i, f].
 // Eight warps take 16 rows each (lane = 4 features); the eight partial sums
 // are added in warp order.
-template <typename T>
 __global__ void __launch_bounds__(256) k_head_wgrad(Segs sg, int n, const float* __restrict__ dz,
                                                     float* __restrict__ dVpart) {
   __shared__ float dzs[kWgRows][kClasses];
@@ -423,7 +589,7 @@ __global__ void __launch_bounds__(256) k_head_wgrad(Segs sg, int n, const float*
     chunk -= (sg.F[k] + kWgChunk - 1) / kWgChunk;
     ++k;
   }
-  const T* H = static_cast<const T*>(sg.H[k]);
+  const float* H = static_cast<const float*>(sg.H[k]);
   const int ld = sg.ld[k], Fk = sg.F[k], off = sg.off[k];
   const int f0 = chunk * kWgChunk;
   const int rb0 = blockIdx.y * kWgRows;
@@ -442,7 +608,7 @@ __global__ void __launch_bounds__(256) k_head_wgrad(Segs sg, int n, const float*
 #pragma unroll 4
   for (int i = warp * (kWgRows / 8); i < (warp + 1) * (kWgRows / 8); ++i) {
     float h[4];
-    load_feats<T, 4>(H, ld, rb0 + i, n, f, Fk, h);
+    load_feats4(H, ld, rb0 + i, n, f, Fk, h);
 #pragma unroll
     for (int c = 0; c < kClasses; ++c) {
       const float d = dzs[i][c];
@@ -551,7 +717,7 @@ __global__ void __launch_bounds__(256) k_po_grad(PoGradArgs a, const T* __restri
       for (int c = 0; c < kClasses; ++c) z[c] = dzs[lane][c];
       float loss = 0.f;
       if (r0 + lane < a.n) {
-        loss = finish_row(z, r0 + lane, a.labels, a.inv_n, nullptr, nullptr, dzr, &a.hds->err);
+        loss = finish_row(z, r0 + lane, true, __ldg(a.labels + r0 + lane), a.inv_n, nullptr, nullptr, dzr, &a.hds->err);
       } else {
 #pragma unroll
         for (int c = 0; c < kClasses; ++c) dzr[c] = 0.f;
@@ -675,27 +841,19 @@ struct HeadAdamArgs {
 };
 
 
-// Threads 0 .. 10F-1 of the grid own one V element each; the last block owns
-// the 10 biases (warp w: columns w and w + 8 of the partials, column 10 being
-// the loss).
-__global__ void __launch_bounds__(256) k_head_adam(HeadAdamArgs a) {
-  ptx::griddep_wait();  // launched with programmatic stream serialization
-  const float a1 = a.lr / a.ds->bc1, r2 = 1.f / a.ds->bc2;
-  const int total = kClasses * a.F;
-  const int vblocks = (total + 255) / 256;
-  if ((int)blockIdx.x < vblocks) {
-    const int idx = blockIdx.x * 256 + threadIdx.x;
-    if (idx >= total) return;
-    // the row blocks' partials in order, eight loads in flight
-    const float g = sum_partials(a.dVpart, a.nrb, total, idx);
-    if (a.dV_out) a.dV_out[idx] = g;
-    float w = a.V[idx], m = a.mV[idx], v = a.vV[idx];
-    adam1(w, m, v, g, a1, a.beta1, a.beta2, a.eps, r2);
-    a.V[idx] = w;
-    a.mV[idx] = m;
-    a.vV[idx] = v;
-    return;
-  }
+// One Adam step of one element of V, and its gradient kept.
+__device__ __forceinline__ void head_adam_v(const HeadAdamArgs& a, int idx, float g, float a1, float r2) {
+  if (a.dV_out) a.dV_out[idx] = g;
+  float w = a.V[idx], m = a.mV[idx], v = a.vV[idx];
+  adam1(w, m, v, g, a1, a.beta1, a.beta2, a.eps, r2);
+  a.V[idx] = w;
+  a.mV[idx] = m;
+  a.vV[idx] = v;
+}
+
+// The 10 biases and the loss, by one block of 256 threads (warp w: columns w
+// and w + 8 of the partials, column 10 being the loss).
+__device__ __forceinline__ void head_adam_c(const HeadAdamArgs& a, float a1, float r2) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int col = warp; col < kPart; col += 8) {
     float t = 0.f;
@@ -712,6 +870,97 @@ __global__ void __launch_bounds__(256) k_head_adam(HeadAdamArgs a) {
     a.c[col] = w;
     a.mc[col] = m;
     a.vc[col] = v;
+  }
+}
+
+// Threads 0 .. 10F-1 of the grid own one V element each; the last block owns
+// the 10 biases.
+__global__ void __launch_bounds__(256) k_head_adam(HeadAdamArgs a) {
+  ptx::griddep_wait();  // launched with programmatic stream serialization
+  const float a1 = a.lr / a.ds->bc1, r2 = 1.f / a.ds->bc2;
+  const int total = kClasses * a.F;
+  const int vblocks = (total + 255) / 256;
+  if ((int)blockIdx.x >= vblocks) {
+    head_adam_c(a, a1, r2);
+    return;
+  }
+  const int idx = blockIdx.x * 256 + threadIdx.x;
+  // the row blocks' partials in order, eight loads in flight
+  if (idx < total) head_adam_v(a, idx, sum_partials(a.dVpart, a.nrb, total, idx), a1, r2);
+}
+
+// The head's weight gradient and Adam of bf16 activities in one kernel: a
+// block owns 32 features of one segment over all n rows (so its dV is
+// complete: no partials through memory, no second launch), the last block the
+// biases.  dV is 16 (classes) x 32 (features) per block, K = the rows: warp w
+// takes every eighth group of 16 rows.  dz times the segment's row scale
+// comes as A operands of three bf16 parts, written once by the logits
+// kernel's finishing blocks; the activity is loaded as 8 bytes of four rows
+// per lane -- 64 contiguous bytes per row -- and pairs of rows are interleaved
+// into B operands.  No staging: every load is independent of the others.
+constexpr int kWgaFeats = 32;
+
+__global__ void __launch_bounds__(256, 2) k_head_wgrad_adam(Segs sg, int n, const uint4* __restrict__ dzfrag,
+                                                         HeadAdamArgs a) {
+  __shared__ float red[8][kClasses][kWgaFeats + 1];
+  ptx::griddep_wait();  // launched with programmatic stream serialization
+  const float a1 = a.lr / a.ds->bc1, r2 = 1.f / a.ds->bc2;
+  if (blockIdx.x + 1 == gridDim.x) {
+    head_adam_c(a, a1, r2);
+    return;
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = lane >> 2, t = lane & 3;
+  int k = 0, chunk = blockIdx.x;
+  while (k + 1 < sg.nseg && chunk >= (sg.F[k] + kWgaFeats - 1) / kWgaFeats) {
+    chunk -= (sg.F[k] + kWgaFeats - 1) / kWgaFeats;
+    ++k;
+  }
+  const bf16* H = static_cast<const bf16*>(sg.H[k]);
+  const int ld = sg.ld[k], Fk = sg.F[k], off = sg.off[k];
+  const int f0 = chunk * kWgaFeats;
+  // rows are padded to whole 8-feature words, the padding zero
+  const bool f_ok = f0 + 4 * g < ld;
+  const int groups = (n + 15) / 16;
+  const uint4* df = dzfrag + (size_t)k * groups * 3 * 32 + lane;
+  float d[4][4] = {};  // feature f0 + 4 (column) + j of column tile j
+#pragma unroll 4
+  for (int gr = warp; gr < groups; gr += 8) {
+    const int row = gr * 16 + 2 * t;
+    uint2 h[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int r = row + (e & 1) + (e >> 1) * 8;
+      h[e] = f_ok && r < n ? __ldg(reinterpret_cast<const uint2*>(H + (size_t)r * ld + f0 + 4 * g)) : make_uint2(0u, 0u);
+    }
+    uint4 av[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) av[q] = __ldg(df + (gr * 3 + q) * 32);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t sel = j & 1 ? 0x7632u : 0x5410u;
+      const uint32_t b0 = __byte_perm(j < 2 ? h[0].x : h[0].y, j < 2 ? h[1].x : h[1].y, sel);
+      const uint32_t b1 = __byte_perm(j < 2 ? h[2].x : h[2].y, j < 2 ? h[3].x : h[3].y, sel);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) mma16816(d[j], av[q].x, av[q].y, av[q].z, av[q].w, b0, b1);
+    }
+  }
+  // the eight warps' sums in warp order, then Adam: a thread per element
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      red[warp][g][4 * (2 * t + e) + j] = d[j][e];
+      if (g < kClasses - 8) red[warp][8 + g][4 * (2 * t + e) + j] = d[j][2 + e];
+    }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < kClasses * kWgaFeats; idx += 256) {
+    const int c = idx / kWgaFeats, j = idx % kWgaFeats;
+    if (f0 + j >= Fk) continue;
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) v += red[w][c][j];
+    head_adam_v(a, c * a.F + off + f0 + j, v, a1, r2);
   }
 }
 
@@ -773,7 +1022,8 @@ struct HeadWork {
   float* zpart;
   float* dz;
   float* part;
-  float* dVpart;
+  float* dVpart;   // fp32 layers
+  uint4* dzfrag;   // bf16 layers
 };
 
 // Partial-logit floats for up to `rows` rows of the layer chain's segments.
@@ -806,9 +1056,11 @@ ff_status head_workspace(ff_head* hd, ff_layer* const* layers, int L, int rows, 
   size_t oG2 = off; off += align256(b16 ? (size_t)ntmax * rows * 4 : 0);
   size_t oZ = off; off += align256((size_t)rows * kClasses * 4);
   size_t oZP = off; off += align256(chain_zpart_floats(layers, L, rows) * 4);
-  size_t oD = off; off += align256(train ? (size_t)rows * kClasses * 4 : 0);
+  size_t oD = off; off += align256(train && !b16 ? (size_t)rows * kClasses * 4 : 0);
+  const int nseg = L > 1 ? L - 1 : 1;
+  size_t oF = off; off += align256(train && b16 ? (size_t)nseg * cdiv(rows, 16) * 3 * 32 * sizeof(uint4) : 0);
   size_t oP = off; off += align256(train ? (size_t)cdiv(rows, kDotRows) * kPart * 4 : 0);
-  size_t oV = off; off += align256(train ? (size_t)cdiv(rows, kWgRows) * kClasses * hd->F * 4 : 0);
+  size_t oV = off; off += align256(train && !b16 ? (size_t)cdiv(rows, kWgRows) * kClasses * hd->F * 4 : 0);
   if (off > wsb) {
     FF_TRY(cudaStreamSynchronize(hd->last_stream), "sync before head workspace growth");
     if (hd->side) FF_TRY(cudaStreamSynchronize(hd->side), "sync before head workspace growth");
@@ -826,7 +1078,8 @@ ff_status head_workspace(ff_head* hd, ff_layer* const* layers, int L, int rows, 
   w->gpart2 = reinterpret_cast<float*>(base + (b16 ? oG2 : oG));
   w->logits = reinterpret_cast<float*>(base + oZ);
   w->zpart = reinterpret_cast<float*>(base + oZP);
-  w->dz = train ? reinterpret_cast<float*>(base + oD) : nullptr;
+  w->dz = train && !b16 ? reinterpret_cast<float*>(base + oD) : nullptr;
+  w->dzfrag = train && b16 ? reinterpret_cast<uint4*>(base + oF) : nullptr;
   w->part = train ? reinterpret_cast<float*>(base + oP) : nullptr;
   w->dVpart = train ? reinterpret_cast<float*>(base + oV) : nullptr;
   return FF_OK;
@@ -925,7 +1178,7 @@ ff_status ensure_counters(ff_head* hd, int blocks) {
 // partials) of n rows: k_head_dot over the feature splits, whose last block
 // per row block finishes the rows.
 ff_status head_logits(ff_head* hd, const Segs& sg, bool b16, int n, const int* labels, float* logits, float* zpart,
-                      float* dz, float* part, int* err, cudaStream_t st) {
+                      float* dz, float* part, uint4* dzfrag, int* err, cudaStream_t st) {
   const int es = b16 ? 2 : 4;
   const int split = dot_split(sg.F, sg.nseg, n, es);
   const int S = head_splits(sg.F, sg.nseg, split);
@@ -938,37 +1191,50 @@ ff_status head_logits(ff_head* hd, const Segs& sg, bool b16, int n, const int* l
   fa.logits = logits;
   fa.dz = dz;
   fa.part = part;
+  fa.dzfrag = dzfrag;
   fa.ds = labels ? hd->ds : nullptr;
   fa.beta1 = hd->cfg.beta1;
   fa.beta2 = hd->cfg.beta2;
   fa.counter = hd->counters;
   fa.S = S;
   const float* V = hd->V;
+  dim3 grid(S, cdiv(n, kDotRows));
+  const double work = (double)n * sg.F_total * es + (double)n * (2 * S + 2) * kClasses * 4;
+  if (b16) {
+    static const cudaError_t attr = cudaFuncSetAttribute(k_head_dot_mma, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                         mma_smem(kMmaSplit));
+    FF_TRY(attr, "head kernel attributes");
+    PdlLaunch l(grid, dim3(256), st, mma_smem(split));
+    FF_LAUNCH(K_HEAD_LOGITS, work, st, cudaLaunchKernelEx(&l.cfg, k_head_dot_mma, sg, split, n, V, zpart, fa, err),
+              "head logits, softmax and cross-entropy");
+    return FF_OK;
+  }
   HeadMaps maps;
   std::memset(&maps, 0, sizeof(maps));
   for (int k = 0; k < sg.nseg; ++k)
     if (!make_plain_map(&maps.m[k], sg.H[k], es, sg.ld[k], n, sg.ld[k], 512 / es, kDotRows))
       return FF_ERR_INVALID_ARG;
-  static const cudaError_t attr_b = cudaFuncSetAttribute(k_head_dot<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  static const cudaError_t attr_f = cudaFuncSetAttribute(k_head_dot, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                          kDotSmem);
-  static const cudaError_t attr_f = cudaFuncSetAttribute(k_head_dot<float>,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kDotSmem);
-  FF_TRY(b16 ? attr_b : attr_f, "head kernel attributes");
-  dim3 grid(S, cdiv(n, kDotRows));
+  FF_TRY(attr_f, "head kernel attributes");
   PdlLaunch l(grid, dim3(256), st, kDotSmem);
-  FF_LAUNCH(K_HEAD_LOGITS, (double)n * sg.F_total * es + (double)n * (2 * S + 2) * kClasses * 4, st,
-            (b16 ? cudaLaunchKernelEx(&l.cfg, k_head_dot<bf16>, maps, sg, split, n, V, zpart, fa, err)
-                 : cudaLaunchKernelEx(&l.cfg, k_head_dot<float>, maps, sg, split, n, V, zpart, fa, err)),
+  FF_LAUNCH(K_HEAD_LOGITS, work, st, cudaLaunchKernelEx(&l.cfg, k_head_dot, maps, sg, split, n, V, zpart, fa, err),
             "head logits, softmax and cross-entropy");
   return FF_OK;
 }
 
-cudaError_t launch_head_wgrad(const Segs& sg, bool b16, int n, const float* dz, float* dVpart, cudaStream_t st) {
+cudaError_t launch_head_wgrad(const Segs& sg, int n, const float* dz, float* dVpart, cudaStream_t st) {
   int chunks = 0;
   for (int k = 0; k < sg.nseg; ++k) chunks += cdiv(sg.F[k], kWgChunk);
   PdlLaunch l(dim3(chunks, cdiv(n, kWgRows)), dim3(256), st);
-  return b16 ? cudaLaunchKernelEx(&l.cfg, k_head_wgrad<bf16>, sg, n, dz, dVpart)
-             : cudaLaunchKernelEx(&l.cfg, k_head_wgrad<float>, sg, n, dz, dVpart);
+  return cudaLaunchKernelEx(&l.cfg, k_head_wgrad, sg, n, dz, dVpart);
+}
+
+cudaError_t launch_head_wgrad_adam(const Segs& sg, int n, const uint4* dzfrag, const HeadAdamArgs& a, cudaStream_t st) {
+  int chunks = 0;
+  for (int k = 0; k < sg.nseg; ++k) chunks += cdiv(sg.F[k], kWgaFeats);
+  PdlLaunch l(dim3(chunks + 1), dim3(256), st);
+  return cudaLaunchKernelEx(&l.cfg, k_head_wgrad_adam, sg, n, dzfrag, a);
 }
 
 }  // namespace
@@ -1150,11 +1416,17 @@ static ff_status head_step_on_features(ff_head* hd, ff_layer* const* layers, int
     sg.s[j] += r0;
   }
   int* err = &hd->ds->err;
-  ff_status s = head_logits(hd, sg, b16, n, labels, nullptr, w.zpart, w.dz, w.part, err, st);
+  ff_status s = head_logits(hd, sg, b16, n, labels, nullptr, w.zpart, w.dz, w.part, w.dzfrag, err, st);
   if (s != FF_OK) return s;
+  const HeadAdamArgs a =
+      head_adam_args(hd, w.dVpart, b16 ? 0 : cdiv(n, kWgRows), w.part, cdiv(n, kDotRows), n, loss);
+  if (b16) {
+    FF_LAUNCH(K_HEAD_WGRAD, (double)n * hd->F * es + (double)kClasses * hd->F * 28, st,
+              launch_head_wgrad_adam(sg, n, w.dzfrag, a, st), "head weight gradient and Adam");
+    return FF_OK;
+  }
   FF_LAUNCH(K_HEAD_WGRAD, (double)n * hd->F * es + (double)cdiv(n, kWgRows) * kClasses * hd->F * 4, st,
-            launch_head_wgrad(sg, b16, n, w.dz, w.dVpart, st), "head weight gradient");
-  const HeadAdamArgs a = head_adam_args(hd, w.dVpart, cdiv(n, kWgRows), w.part, cdiv(n, kDotRows), n, loss);
+            launch_head_wgrad(sg, n, w.dz, w.dVpart, st), "head weight gradient");
   const int vblocks = cdiv((long long)kClasses * hd->F, 256);
   PdlLaunch l(dim3(vblocks + 1), dim3(256), st);
   FF_LAUNCH(K_HEAD_ADAM, (double)kClasses * hd->F * (a.nrb * 4.0 + 28), st, cudaLaunchKernelEx(&l.cfg, k_head_adam, a),
@@ -1259,7 +1531,7 @@ ff_status ff_head_predict(ff_head* hd, ff_layer* const* layers, int n_layers, co
     if (s != FF_OK) return s;
     const Segs sg = make_segs(layers, n_layers, w, hd->F);
     float* z = logits ? logits + (size_t)r0 * kClasses : w.logits;
-    s = head_logits(hd, sg, b16, cn, nullptr, z, w.zpart, nullptr, nullptr, err, st);
+    s = head_logits(hd, sg, b16, cn, nullptr, z, w.zpart, nullptr, nullptr, nullptr, err, st);
     if (s != FF_OK) return s;
     if (pred)
       FF_LAUNCH(K_ARGMAX, (double)cn * 44, st, launch_argmax(z, cn, nullptr, pred + r0, st), "head argmax");
@@ -1406,7 +1678,7 @@ ff_status ff_po_train_step(ff_layer* L, ff_head* hd, const void* x, int raw_inpu
     sg.off[0] = 0;
     sg.nseg = 1;
     sg.F_total = N;
-    s = head_logits(hd, sg, b16, n, labels, nullptr, w.zpart, w.dz, w.part, &hd->ds->err, st);
+    s = head_logits(hd, sg, b16, n, labels, nullptr, w.zpart, w.dz, w.part, nullptr, &hd->ds->err, st);
     if (s != FF_OK) return s;
   }
   // the gradient reaching the layer, with the block's weights before its
@@ -1541,7 +1813,7 @@ ff_status ff_po_predict(ff_layer* const* layers, int n_layers, ff_head* hd, cons
     sg.nseg = 1;
     sg.F_total = top->N;
     float* z = logits ? logits + (size_t)r0 * kClasses : w.logits;
-    s = head_logits(hd, sg, b16, cn, nullptr, z, w.zpart, nullptr, nullptr, err, st);
+    s = head_logits(hd, sg, b16, cn, nullptr, z, w.zpart, nullptr, nullptr, nullptr, err, st);
     if (s != FF_OK) return s;
     if (pred)
       FF_LAUNCH(K_ARGMAX, (double)cn * 44, st, launch_argmax(z, cn, nullptr, pred + r0, st), "block argmax");
