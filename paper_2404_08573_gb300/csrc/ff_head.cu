@@ -1390,8 +1390,25 @@ ff_status ff_head_destroy(ff_head* hd) {
   return FF_OK;
 }
 
-// Rows of stored features ff_head_train_epoch forms per forward pass.
+// Rows of stored features ff_head_train_epoch forms per forward pass: whole
+// steps of B rows, at least one, at most kEpochFeatureRows; with bf16 layers
+// also at most what the widest layer's GEMM does in two full waves of CTAs.
+// The first pass's forward has nothing to run beside, and a pass's activities
+// are read again by its steps, from L2 if they still are there: 20000 rows of
+// 784-2000x4 in steps of 1024 take 891 us with 16384 rows a pass, 827 with
+// 9728 (two waves), 816 with 4864, 1112 with 2432.
 constexpr int kEpochFeatureRows = 16384;
+static int epoch_pass_steps(ff_layer* const* layers, int n_layers, int B) {
+  int steps = kEpochFeatureRows / B > 0 ? kEpochFeatureRows / B : 1;
+  if (!layers[0]->is_bf16) return steps;
+  int dev = 0, sms = 0, Nw = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return steps;
+  for (int k = 0; k < n_layers; ++k) Nw = std::max(Nw, layers[k]->N);
+  while (steps > 1 && tc_gemm_fwd_ctas(steps * B, Nw, false) > 2 * sms) --steps;
+  return steps;
+}
 
 // The head's side stream and its events (created on first use).
 static ff_status ensure_side(ff_head* hd) {
@@ -1462,9 +1479,7 @@ ff_status ff_head_train_epoch(ff_head* hd, ff_layer* const* layers, int n_layers
   if (n == 0) return FF_OK;
   if (!x || !labels || B > hd->cfg.max_rows) return FF_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // Rows whose features one forward pass forms: whole steps, up to
-  // kEpochFeatureRows (at least one step).
-  const int steps_per_chunk = kEpochFeatureRows / B > 0 ? kEpochFeatureRows / B : 1;
+  const int steps_per_chunk = epoch_pass_steps(layers, n_layers, B);
   const int R = (int)((long long)steps_per_chunk * B < n ? (long long)steps_per_chunk * B : n);
   const int npass = cdiv(n, R);
   if (npass > 1) {
