@@ -255,17 +255,19 @@ ff_status train_step_impl(ff_layer* L, const void* x, const int* labels, const f
   }
   if (ev_forward_done) FF_TRY(cudaEventRecord(ev_forward_done, st), "event record");
 
-  if (L->is_bf16) {
-    FF_LAUNCH(K_WGRAD_TC, 2.0 * M * L->N * L->K, st,
-              tc_gemm_wgrad(static_cast<const bf16*>(L->dZ), L->ldN, static_cast<const bf16*>(fr.X), L->ldK, M,
-                            L->N, L->K, L->dW, L->K, &L->ds->err, st),
-              "weight-gradient GEMM (tcgen05)");
-  } else {
-    FF_LAUNCH(K_WGRAD_SIMT, 2.0 * M * L->N * L->K, st,
-              simt_gemm_wgrad(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(fr.X), L->ldK, M,
-                              L->N, L->K, L->dW, L->K, st),
-              "weight-gradient GEMM (fp32)");
-  }
+  AdamArgs aa = adam_args(L, M);
+  aa.loss_part = L->loss_part;
+  aa.stat_part = L->stat_part;
+  aa.ncb = cdiv(L->ldN, 256);
+  aa.stats_out = L->ds->stats;
+  aa.loss_out = loss ? loss : &L->ds->loss;
+  aa.B = B;
+  return weight_update(L, fr.X, M, aa, st);
+}
+
+// Adam arguments of the layer's parameters after a step on M rows (without
+// loss and statistics).
+AdamArgs adam_args(ff_layer* L, int M) {
   AdamArgs aa{};
   aa.W = L->W;
   aa.mW = L->mW;
@@ -287,20 +289,40 @@ ff_status train_step_impl(ff_layer* L, const void* x, const int* labels, const f
   aa.beta2 = L->cfg.beta2;
   aa.eps = L->cfg.eps;
   aa.ds = L->ds;
-  aa.loss_part = L->loss_part;
-  aa.stat_part = L->stat_part;
-  aa.ncb = cdiv(L->ldN, 256);
-  aa.stats_out = L->ds->stats;
-  aa.loss_out = loss ? loss : &L->ds->loss;
-  aa.B = B;
+  return aa;
+}
+
+// The weight gradient from the operand in L->dZ and the layer input X (M
+// rows), and the Adam step: one kernel for small fp32 GEMMs, else the GEMM
+// and the Adam kernel.
+ff_status weight_update(ff_layer* L, const void* X, int M, AdamArgs& aa, cudaStream_t st) {
+  const double flops = 2.0 * M * L->N * L->K;
+  const double state = (double)L->N * L->K * 24.0 + (double)L->N * (aa.nrb * 4.0 + 28);
+  aa.keep_dW = L->cfg.keep_grad ? L->dW : nullptr;
+  if (!L->is_bf16 && simt_wgrad_adam_fits(M, L->N, L->K)) {
+    FF_LAUNCH(K_WGRAD_SIMT, flops, st,
+              simt_gemm_wgrad_adam(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(X), L->ldK, M,
+                                   aa, st),
+              "weight-gradient GEMM and Adam (fp32)");
+    return FF_OK;
+  }
+  if (L->is_bf16) {
+    FF_LAUNCH(K_WGRAD_TC, flops, st,
+              tc_gemm_wgrad(static_cast<const bf16*>(L->dZ), L->ldN, static_cast<const bf16*>(X), L->ldK, M, L->N,
+                            L->K, L->dW, L->K, &L->ds->err, st),
+              "weight-gradient GEMM (tcgen05)");
+  } else {
+    FF_LAUNCH(K_WGRAD_SIMT, flops, st,
+              simt_gemm_wgrad(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(X), L->ldK, M, L->N,
+                              L->K, L->dW, L->K, st),
+              "weight-gradient GEMM (fp32)");
+  }
   // Data nobody reads after this step, so its dirty lines need not reach HBM:
   // dW (unless kept for ff_layer_get_grad) and the local-gradient operand.
   // (Dropping the activities' lines as well measured no further gain.)
   aa.discard_dW = !L->cfg.keep_grad && ((uintptr_t)L->dW & 127u) == 0;
-  if (!L->cfg.keep_grad) add_dead(aa, L->dZ, (size_t)M * L->ldN * (size_t)es);
-  FF_LAUNCH(K_ADAM, (double)L->N * L->K * (28.0 + (L->is_bf16 ? 2.0 : 0.0)) + (double)L->N * (aa.nrb * 4.0 + 28), st,
-            launch_adam(aa, st),
-            "Adam");
+  if (!L->cfg.keep_grad) add_dead(aa, L->dZ, (size_t)M * L->ldN * (L->is_bf16 ? 2 : 4));
+  FF_LAUNCH(K_ADAM, state + (double)L->N * L->K * (L->is_bf16 ? 6.0 : 4.0), st, launch_adam(aa, st), "Adam");
   return FF_OK;
 }
 

@@ -15,6 +15,7 @@
 //                the 9 wrong labels for AdaptiveNEG negatives (§5)
 // Reductions use fixed orders (no floating-point atomics), so results do not
 // depend on scheduling.
+#include "ff_adam.cuh"
 #include "ff_internal.cuh"
 #include "ff_ptx.cuh"
 
@@ -288,27 +289,17 @@ __global__ void __launch_bounds__(256) k_adam(AdamArgs a, int w_blocks) {
       const bool dense_b = a.ldb == a.K;
       for (long long q = (long long)blockIdx.x * 256 + threadIdx.x; q * 4 < total; q += stride) {
         const long long idx = q * 4;
-        // W, m, v and dW are touched once per step: evict-first, so the
-        // stream leaves the GEMMs' operands in L2
-        float4 w = __ldcs(reinterpret_cast<const float4*>(a.W + idx));
-        float4 m = __ldcs(reinterpret_cast<const float4*>(a.mW + idx));
-        float4 v = __ldcs(reinterpret_cast<const float4*>(a.vW + idx));
+        AdamVec s;
+        s.load(a, idx);
         const float4 g = __ldcs(reinterpret_cast<const float4*>(a.dW + idx));
-        adam1(w.x, m.x, v.x, g.x, a1, a.beta1, a.beta2, a.eps, r2);
-        adam1(w.y, m.y, v.y, g.y, a1, a.beta1, a.beta2, a.eps, r2);
-        adam1(w.z, m.z, v.z, g.z, a1, a.beta1, a.beta2, a.eps, r2);
-        adam1(w.w, m.w, v.w, g.w, a1, a.beta1, a.beta2, a.eps, r2);
-        __stcs(reinterpret_cast<float4*>(a.W + idx), w);
-        __stcs(reinterpret_cast<float4*>(a.mW + idx), m);
-        __stcs(reinterpret_cast<float4*>(a.vW + idx), v);
+        s.update(a, g, a1, r2);
+        s.store(a, idx);
         // the first of every 8 threads drops the 128-byte dW line the 8 just
         // read (the warp's loads have all returned: g was used above)
         if (a.discard_dW && (threadIdx.x & 7) == 0 && idx + 32 <= total) ptx::discard_l2(a.dW + idx);
         if (a.Wb) {
           const long long o = dense_b ? idx : (idx / a.K) * a.ldb + idx % a.K;
-          __nv_bfloat162 p0 = __floats2bfloat162_rn(w.x, w.y), p1 = __floats2bfloat162_rn(w.z, w.w);
-          uint2 u = make_uint2(*reinterpret_cast<uint32_t*>(&p0), *reinterpret_cast<uint32_t*>(&p1));
-          *reinterpret_cast<uint2*>(a.Wb + o) = u;
+          *reinterpret_cast<uint2*>(a.Wb + o) = s.packed();
         }
       }
     } else {
@@ -322,57 +313,7 @@ __global__ void __launch_bounds__(256) k_adam(AdamArgs a, int w_blocks) {
       }
     }
   } else {
-    // 32 bias elements per block: warp w sums row blocks w, w+8, ... for the
-    // block's 32 columns (lane = column), then warp 0 adds the 8 warp sums in
-    // order -- a fixed reduction order, with the loads batched.
-    __shared__ float part[8][33];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int j = (blockIdx.x - w_blocks) * 32 + lane;
-    float acc = 0.f;
-    if (j < a.N) {
-      for (int rb0 = w; rb0 < a.nrb; rb0 += 64) {
-        float v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int rb = rb0 + 8 * u;
-          v[u] = rb < a.nrb ? __ldg(a.dbpart + (size_t)rb * a.N + j) : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) acc += v[u];
-      }
-    }
-    part[w][lane] = acc;
-    __syncthreads();
-    if (blockIdx.x == w_blocks && w == 1 && a.loss_part) {
-      // the step's loss: grad_prep's per-row-block partials, lane-strided then
-      // a fixed-order warp tree
-      float tot = 0.f;
-      for (int rb = lane; rb < a.nrb; rb += 32) tot += a.loss_part[rb];
-      tot = warp_sum(tot);
-      if (lane == 0) a.loss_out[0] = tot / (float)a.B;
-    }
-    if (blockIdx.x == w_blocks && w >= 2 && w <= 4 && a.stat_part) {
-      // the step's statistics: mean goodness of the positive and of the
-      // negative rows, and the fraction of active ReLUs
-      const int n = w == 4 ? a.nrb * a.ncb : a.nrb;
-      const float* src = a.stat_part + (w == 2 ? 0 : w == 3 ? a.nrb : 2 * a.nrb);
-      float tot = 0.f;
-      for (int k = lane; k < n; k += 32) tot += src[k];
-      tot = warp_sum(tot);
-      if (lane == 0) a.stats_out[w - 2] = w == 4 ? tot / (2.f * (float)a.B * (float)a.N) : tot / (float)a.B;
-    }
-    if (w != 0 || j >= a.N) return;
-    float db = 0.f;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) db += part[u][lane];
-    if (a.db_out) a.db_out[j] = db;
-    if (a.has_bias) {
-      float b = a.b[j], m = a.mb[j], v = a.vb[j];
-      adam1(b, m, v, db, a1, a.beta1, a.beta2, a.eps, r2);
-      a.b[j] = b;
-      a.mb[j] = m;
-      a.vb[j] = v;
-    }
+    adam_bias_block(a, (int)blockIdx.x - w_blocks, a1, r2);
   }
 }
 
@@ -571,7 +512,7 @@ void add_dead(AdamArgs& a, void* p, size_t bytes) {
 cudaError_t launch_adam(const AdamArgs& a, cudaStream_t st) {
   const long long total = (long long)a.N * a.K;
   const int w_blocks = grid_for((a.K & 3) == 0 ? total / 4 : total, 256, 152 * 16);
-  const int b_blocks = cdiv(a.N, 32);
+  const int b_blocks = adam_bias_blocks(a.N);
   PdlLaunch l(dim3(w_blocks + b_blocks), dim3(256), st);
   return cudaLaunchKernelEx(&l.cfg, k_adam, a, w_blocks);
 }

@@ -19,6 +19,7 @@
 // adds TM/S rows of all S partials (in rank order) through distributed
 // shared memory and runs the epilogue on them -- no scratch in device memory
 // and no counters.
+#include "ff_adam.cuh"
 #include "ff_internal.cuh"
 #include "ff_ptx.cuh"
 
@@ -27,7 +28,7 @@ namespace {
 
 constexpr int NT = 256;
 constexpr int TKS = 32;  // K per stage
-constexpr int MODE_FWD = 0, MODE_STORE = 1;
+constexpr int MODE_FWD = 0, MODE_STORE = 1, MODE_ADAM = 2;
 constexpr int kMaxSplit = 4;  // CTAs per cluster (see plan_of)
 
 // Shape of one instance.  An operand's stage sits in shared memory as TKS
@@ -117,7 +118,7 @@ __device__ __forceinline__ void load_tile(float* S, const float* __restrict__ P,
 template <int T, int KGRP, bool MN, int MODE>
 __global__ void __launch_bounds__(NT, 2)
     k_simt_gemm(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb, int M, int N, int K,
-                int vecs, EpiArgs ep) {
+                int vecs, EpiArgs ep, AdamArgs ad) {
   using C = Cfg<T, KGRP>;
   extern __shared__ __align__(16) float sm[];
   const int m0 = blockIdx.x * C::TM, n0 = blockIdx.y * C::TN;
@@ -130,6 +131,18 @@ __global__ void __launch_bounds__(NT, 2)
   const int grp = tid / (C::TT * C::TT), t = tid % (C::TT * C::TT);
   const int tx = t % C::TT, ty = t / C::TT;
   const bool va = vecs & 1, vb = vecs & 2;
+  if constexpr (MODE == MODE_ADAM) {
+    if (blockIdx.y + 1 == gridDim.y) {
+      // the last row of CTAs: the bias elements, loss and statistics
+      ptx::griddep_wait();
+      const float a1 = ad.lr / ad.ds->bc1, r2 = 1.f / ad.ds->bc2;
+      for (int blk = blockIdx.x * S + blockIdx.z; blk * 32 < ad.N; blk += gridDim.x * S) {
+        adam_bias_block(ad, blk, a1, r2);
+        __syncthreads();
+      }
+      return;
+    }
+  }
   ptx::griddep_wait();  // launched with programmatic stream serialization
 
   auto stage = [&](int s) {
@@ -218,60 +231,105 @@ __global__ void __launch_bounds__(NT, 2)
 
   // the epilogue on this CTA's TM / S rows of the tile
   const int RS = C::TM / S;
-  for (int p = 0; p < RS; p += RPP) {
-    const int r = (int)blockIdx.z * RS + p + lr;
-    const bool row_ok = p + lr < RS && m0 + r < M;
-    const int gi = m0 + r;
-    float v[4] = {0.f, 0.f, 0.f, 0.f};
-    if (row_ok) {
-      if (S > 1) {
-        float4 u[kMaxSplit];
+  const int col = n0 + lc;
+  // four values of row r of the tile: the sum of the S partials in rank order
+  auto tile4 = [&](int r, float (&v)[4]) {
+    if (S > 1) {
+      float4 u[kMaxSplit];
 #pragma unroll
-        for (int z = 0; z < kMaxSplit; ++z)
-          if (z < S) u[z] = ld_cluster4(sm + r * C::LD + lc, (uint32_t)z);
+      for (int z = 0; z < kMaxSplit; ++z)
+        if (z < S) u[z] = ld_cluster4(sm + r * C::LD + lc, (uint32_t)z);
+      v[0] = v[1] = v[2] = v[3] = 0.f;
 #pragma unroll
-        for (int z = 0; z < kMaxSplit; ++z)
-          if (z < S) {
-            v[0] += u[z].x; v[1] += u[z].y; v[2] += u[z].z; v[3] += u[z].w;
+      for (int z = 0; z < kMaxSplit; ++z)
+        if (z < S) {
+          v[0] += u[z].x; v[1] += u[z].y; v[2] += u[z].z; v[3] += u[z].w;
+        }
+    } else {
+      const float4 u = *reinterpret_cast<const float4*>(sm + r * C::LD + lc);
+      v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
+    }
+  };
+  if constexpr (MODE == MODE_ADAM) {
+    // Adam on the tile's weights: the state of kBatch rows in flight at a time
+    constexpr int kBatch = 4;
+    const float a1 = ad.lr / ad.ds->bc1, r2 = 1.f / ad.ds->bc2;
+    const bool vec = (ad.K & 3) == 0;
+    for (int p = 0; p < RS; p += kBatch * RPP) {
+      AdamVec st[kBatch];
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        const int o = p + q * RPP + lr;
+        const int gi = m0 + (int)blockIdx.z * RS + o;
+        if (vec && o < RS && gi < M && col < N) st[q].load(ad, (size_t)gi * N + col);
+      }
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        const int o = p + q * RPP + lr;
+        const int gi = m0 + (int)blockIdx.z * RS + o;
+        if (o >= RS || gi >= M || col >= N) continue;
+        float v[4];
+        tile4((int)blockIdx.z * RS + o, v);
+        const size_t idx = (size_t)gi * N + col;
+        if (vec) {
+          const float4 dw = make_float4(v[0], v[1], v[2], v[3]);
+          if (ad.keep_dW) *reinterpret_cast<float4*>(ad.keep_dW + idx) = dw;
+          st[q].update(ad, dw, a1, r2);
+          st[q].store(ad, idx);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            if (col + e >= N) break;
+            float w = ad.W[idx + e], m = ad.mW[idx + e], vv = ad.vW[idx + e];
+            adam1(w, m, vv, v[e], a1, ad.beta1, ad.beta2, ad.eps, r2);
+            ad.W[idx + e] = w;
+            ad.mW[idx + e] = m;
+            ad.vW[idx + e] = vv;
+            if (ad.keep_dW) ad.keep_dW[idx + e] = v[e];
           }
-      } else {
-        const float4 u = *reinterpret_cast<const float4*>(sm + r * C::LD + lc);
-        v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
+        }
       }
     }
-    const int col = n0 + lc;
-    if (MODE == MODE_FWD) {
-      float g = 0.f;
-      if (row_ok) {
-        const float s = __ldg(ep.row_scale + gi);
+  } else {
+    for (int p = 0; p < RS; p += RPP) {
+      const int r = (int)blockIdx.z * RS + p + lr;
+      const bool row_ok = p + lr < RS && m0 + r < M;
+      const int gi = m0 + r;
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      if (row_ok) tile4(r, v);
+      if (MODE == MODE_FWD) {
+        float g = 0.f;
+        if (row_ok) {
+          const float s = __ldg(ep.row_scale + gi);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          float h = 0.f;
-          if (col + e < N) {
-            float z = s * v[e];
-            if (ep.bias) z += __ldg(ep.bias + col + e);
-            h = z != z ? z : fmaxf(z, 0.f);  // ReLU, NaN kept for the non-finite check
+          for (int e = 0; e < 4; ++e) {
+            float h = 0.f;
+            if (col + e < N) {
+              float z = s * v[e];
+              if (ep.bias) z += __ldg(ep.bias + col + e);
+              h = z != z ? z : fmaxf(z, 0.f);  // ReLU, NaN kept for the non-finite check
+            }
+            g = fmaf(h, h, g);
+            v[e] = h;
           }
-          g = fmaf(h, h, g);
-          v[e] = h;
+          // activation rows are padded to multiples of 8: whole 16-byte words
+          if (col < ep.ldo)
+            *reinterpret_cast<float4*>(static_cast<float*>(ep.out) + (size_t)gi * ep.ldo + col) =
+                make_float4(v[0], v[1], v[2], v[3]);
         }
-        // activation rows are padded to multiples of 8: whole 16-byte words
-        if (col < ep.ldo)
-          *reinterpret_cast<float4*>(static_cast<float*>(ep.out) + (size_t)gi * ep.ldo + col) =
-              make_float4(v[0], v[1], v[2], v[3]);
-      }
-      // the LPR lanes sharing this row
+        // the LPR lanes sharing this row
 #pragma unroll
-      for (int o = LPR / 2; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-      if (lc == 0 && row_ok) ep.gpart[(size_t)blockIdx.y * M + gi] = g;
-    } else if (row_ok) {
-      float* out = static_cast<float*>(ep.out) + (size_t)gi * ep.ldo + col;
-      if ((ep.ldo & 3) == 0 && col + 4 <= N) {
-        *reinterpret_cast<float4*>(out) = make_float4(v[0], v[1], v[2], v[3]);
-      } else {
+        for (int o = LPR / 2; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+        if (lc == 0 && row_ok) ep.gpart[(size_t)blockIdx.y * M + gi] = g;
+      } else if (row_ok) {
+        float* out = static_cast<float*>(ep.out) + (size_t)gi * ep.ldo + col;
+        if ((ep.ldo & 3) == 0 && col + 4 <= N) {
+          *reinterpret_cast<float4*>(out) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (col + e < N) out[e] = v[e];
+          for (int e = 0; e < 4; ++e)
+            if (col + e < N) out[e] = v[e];
+        }
       }
     }
   }
@@ -315,14 +373,14 @@ Plan plan_of(int M, int N, int K) {
 
 template <int T, int KGRP, bool MN, int MODE>
 cudaError_t launch_plan(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, const EpiArgs& ep,
-                        cudaStream_t st) {
+                        const AdamArgs& ad, cudaStream_t st) {
   using C = Cfg<T, KGRP>;
   static const cudaError_t attr = cudaFuncSetAttribute(k_simt_gemm<T, KGRP, MN, MODE>,
                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (attr != cudaSuccess) return attr;
   auto vec = [](const float* p, int ld) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (ld & 3) == 0; };
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cdiv(M, T), cdiv(N, T), S);
+  cfg.gridDim = dim3(cdiv(M, T), cdiv(N, T) + (MODE == MODE_ADAM ? 1 : 0), S);
   cfg.blockDim = dim3(NT);
   cfg.dynamicSmemBytes = C::SMEM;
   cfg.stream = st;
@@ -336,14 +394,14 @@ cudaError_t launch_plan(const float* A, int lda, const float* B, int ldb, int M,
   cfg.attrs = at;
   cfg.numAttrs = S > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k_simt_gemm<T, KGRP, MN, MODE>, A, lda, B, ldb, M, N, K,
-                            (vec(A, lda) ? 1 : 0) | (vec(B, ldb) ? 2 : 0), ep);
+                            (vec(A, lda) ? 1 : 0) | (vec(B, ldb) ? 2 : 0), ep, ad);
 }
 
 template <bool MN, int MODE>
 cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int N, int K, Plan p, const EpiArgs& ep,
-                   cudaStream_t st) {
-  if (p.large) return launch_plan<128, 1, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, st);
-  return launch_plan<64, 4, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, st);
+                   const AdamArgs& ad, cudaStream_t st) {
+  if (p.large) return launch_plan<128, 1, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, ad, st);
+  return launch_plan<64, 4, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, ad, st);
 }
 
 }  // namespace
@@ -353,21 +411,32 @@ int simt_fwd_ntiles_max(int N) { return cdiv(N, 64); }
 
 cudaError_t simt_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
                           const EpiArgs& ep, cudaStream_t st) {
-  return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, plan_of(plan_rows, N, K), ep, st);
+  return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, plan_of(plan_rows, N, K), ep, AdamArgs{}, st);
 }
 
 cudaError_t simt_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, float* C, int ldc,
                             cudaStream_t st) {
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, plan_of(M, N, K), ep, st);
+  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, plan_of(M, N, K), ep, AdamArgs{}, st);
 }
 
 cudaError_t simt_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, float* C, int ldc,
                             cudaStream_t st) {
-  // C[N, K] = sum_r G[r, n] X[r, k]: rows of C index G's columns (MN-major A),
+  // C[n, k] = sum_r G[r, n] X[r, k]: rows of C index G's columns (MN-major A),
   // columns of C index X's columns (MN-major B), contraction over R.
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, plan_of(N, K, R), ep, st);
+  return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, plan_of(N, K, R), ep, AdamArgs{}, st);
+}
+
+bool simt_wgrad_adam_fits(int R, int N, int K) {
+  const Plan p = plan_of(N, K, R);
+  const int T = p.large ? 128 : 64;
+  return (long long)cdiv(N, T) * cdiv(K, T) * p.S <= 2 * 152;
+}
+
+cudaError_t simt_gemm_wgrad_adam(const float* G, int ldg, const float* X, int ldx, int R, const AdamArgs& a,
+                                 cudaStream_t st) {
+  return launch<true, MODE_ADAM>(G, ldg, X, ldx, a.N, a.K, R, plan_of(a.N, a.K, R), EpiArgs{}, a, st);
 }
 
 }  // namespace ff

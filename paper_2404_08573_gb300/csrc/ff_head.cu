@@ -34,6 +34,7 @@
 
 #include "ff_api_internal.h"
 #include "ff_internal.cuh"
+#include "ff_mma.cuh"
 #include "ff_prof.h"
 #include "ff_ptx.cuh"
 
@@ -178,21 +179,6 @@ __device__ __forceinline__ uint32_t pack_bf16(bf16 lo, bf16 hi) {
   const __nv_bfloat162 v = __halves2bfloat162(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);
 }
-// D (16 x 8, fp32) += A (16 x 16, bf16) B (16 x 8, bf16).  Lane 4 g + t holds
-// of A rows g and g + 8 at K slots 2t, 2t+1 (a0, a1) and 2t+8, 2t+9 (a2, a3),
-// of B column g at the same slots (b0, b1), of D rows g (d0, d1) and g + 8
-// (d2, d3) at columns 2t, 2t+1.
-__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                         uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-      "{%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-constexpr int mma_smem(int split) { return split / 16 * 3 * 32 * 16; }
-
 // The end of every logits block (256 threads) of row block blockIdx.y, rows
 // rblk .. rblk + 63: the last of the row block's fa.S blocks to arrive forms
 // its rows' logits from the splits' partials and finishes them.
@@ -1752,45 +1738,10 @@ ff_status ff_po_train_step(ff_layer* L, ff_head* hd, const void* x, int raw_inpu
               (k_head_adam<<<vblocks + 1, 256, 0, hd->side>>>(ha), cudaGetLastError()), "block Adam");
   }
   FF_TRY(cudaEventRecord(hd->ev_join, hd->side), "event record");
-  if (b16) {
-    FF_LAUNCH(K_WGRAD_TC, 2.0 * n * N * K, st,
-              tc_gemm_wgrad(static_cast<const bf16*>(L->dZ), L->ldN, static_cast<const bf16*>(X), L->ldK, n, N, K,
-                            L->dW, K, &L->ds->err, st),
-              "weight-gradient GEMM (tcgen05)");
-  } else {
-    FF_LAUNCH(K_WGRAD_SIMT, 2.0 * n * N * K, st,
-              simt_gemm_wgrad(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(X), L->ldK, n, N,
-                              K, L->dW, K, st),
-              "weight-gradient GEMM (fp32)");
-  }
-  AdamArgs aa{};
-  aa.W = L->W;
-  aa.mW = L->mW;
-  aa.vW = L->vW;
-  aa.dW = L->dW;
-  aa.N = N;
-  aa.K = K;
-  aa.Wb = b16 ? L->Wb : nullptr;
-  aa.ldb = L->ldK;
-  aa.b = L->b;
-  aa.mb = L->mb;
-  aa.vb = L->vb;
-  aa.dbpart = L->dbpart;
-  aa.nrb = cdiv(n, kPoRows);
-  aa.db_out = L->db;
-  aa.has_bias = L->cfg.has_bias;
-  aa.lr = L->cfg.lr;
-  aa.beta1 = L->cfg.beta1;
-  aa.beta2 = L->cfg.beta2;
-  aa.eps = L->cfg.eps;
-  aa.ds = L->ds;
-  aa.loss_part = nullptr;
-  aa.loss_out = nullptr;
+  AdamArgs aa = adam_args(L, n);
   aa.B = n;
-  // data nobody reads after this step (see the FF train step)
-  aa.discard_dW = !L->cfg.keep_grad && ((uintptr_t)L->dW & 127u) == 0;
-  if (!L->cfg.keep_grad) add_dead(aa, L->dZ, (size_t)n * L->ldN * (size_t)es);
-  FF_LAUNCH(K_ADAM, (double)N * K * (28.0 + (b16 ? 2.0 : 0.0)), st, launch_adam(aa, st), "layer Adam");
+  s = weight_update(L, X, n, aa, st);
+  if (s != FF_OK) return s;
   FF_TRY(cudaStreamWaitEvent(st, hd->ev_join, 0), "stream wait");
   return FF_OK;
 }

@@ -207,6 +207,9 @@ struct AdamArgs {
   int ndead;
   char* dead[2];
   long long dead_lines[2];
+  // simt_gemm_wgrad_adam, which forms dW itself: where to keep it
+  // (ff_layer_get_grad), or null
+  float* keep_dW;
 };
 // Adds [p, p + bytes) to the Adam step's dead buffers (its whole 128-byte
 // lines; nothing when p is not 128-byte aligned).
@@ -335,6 +338,16 @@ cudaError_t simt_gemm_store(const float* A, int lda, const float* B, int ldb, in
                             float* C, int ldc, cudaStream_t st);
 cudaError_t simt_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K,
                             float* C, int ldc, cudaStream_t st);
+// The weight gradient of a.N x a.K outputs over R rows and the Adam step it
+// feeds, in the GEMM's epilogue (dW itself only to a.keep_dW).  Pays where
+// the GEMM's CTAs are all resident at once (simt_wgrad_adam_fits): the step
+// is latency-bound and a launch shorter (784-500-500, batch 64: 9.8 us against
+// 7 + 5).  A larger GEMM fills the FMA pipes, and a separate Adam, bound by
+// HBM, runs beside the other layers' GEMMs: 784-2000x4, batch 256, two steps
+// 1542 us against 1622 with Adam in every epilogue.
+bool simt_wgrad_adam_fits(int R, int N, int K);
+cudaError_t simt_gemm_wgrad_adam(const float* G, int ldg, const float* X, int ldx, int R, const AdamArgs& a,
+                                 cudaStream_t st);
 
 }  // namespace ff
 

@@ -6,7 +6,8 @@ absolute sum, whatever the order)."""
 import numpy as np
 import pytest
 
-from tests.gpu_common import U32, lib_ready, torch_cuda
+from oracle import ff_oracle as fo
+from tests.gpu_common import U32, assert_adam_state, lib_ready, torch_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -46,6 +47,20 @@ def test_fp32_forward_and_weight_gradient_at_tile_edges(M, K, N):
     gref = (ref * ref).sum(1)
     gb = (2 * ref * bound + bound ** 2).sum(1) + (N + 8) * U32 * gref
     assert bool(((good.double() - gref).abs() <= gb).all())
+    # a layer that keeps no gradient ends in the same state (small shapes form
+    # the gradient and the Adam step in one kernel)
+    plain = ff.Layer(K, N, prec="fp32", theta=2.0, lr=1e-3, max_rows=M)
+    plain.set_state(W=st["W"], b=b)
+    plain.train_step(x, row_scale=s, B=M // 2)
+    torch.cuda.synchronize()
+    after, sp = layer.get_state(), plain.get_state()
+    for k in ("W", "b", "mW", "vW", "mb", "vb"):
+        assert np.array_equal(after[k], sp[k]), k
+    # and W, m, v are Adam's on that gradient
+    dw = layer.get_grad()[0].astype(np.float64)
+    zero = np.zeros((N, K))
+    assert_adam_state(after["W"], after["mW"], after["vW"], st["W"].astype(np.float64), zero, zero, 1, dw,
+                      1e-6 * np.abs(dw) + 1e-12, fo.AdamHyper(lr=1e-3), "W")
     # the weight gradient of the GPU's own operand
     G = torch.from_numpy(layer.get_grad_operand(M)).cuda()[:, :N]
     dW = torch.from_numpy(layer.get_grad()[0]).cuda().double()
