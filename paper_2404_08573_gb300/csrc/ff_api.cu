@@ -57,7 +57,7 @@ static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // goodness partials per row: the most either forward GEMM writes
 static int gpart_tiles_max(int N) {
-  const int a = tc_fwd_ntiles_max(N), b = simt_fwd_ntiles_max(N);
+  const int a = tc_fwd_ntiles_max(N), b = f32_fwd_ntiles_max(N);
   return a > b ? a : b;
 }
 
@@ -193,9 +193,9 @@ static ff_status forward_core(ff_layer* L, const void* x, const int* labels, con
               tc_gemm_fwd(static_cast<const bf16*>(X), L->ldK, L->Wb, L->ldK, M, N, K, ep, &L->ds->err, st),
               "forward GEMM (tcgen05)");
   } else {
-    ntiles = simt_fwd_ntiles(M, N, K);
+    ntiles = f32_fwd_ntiles(M, N, K);
     FF_LAUNCH(K_FWD_SIMT, 2.0 * M * N * K, st,
-              simt_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, M, N, K, M, ep, st), "forward GEMM (fp32)");
+              f32_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, M, N, K, M, ep, &L->ds->err, st), "forward GEMM (fp32)");
   }
   r->s = s;
   r->H = H;
@@ -299,9 +299,9 @@ ff_status weight_update(ff_layer* L, const void* X, int M, AdamArgs& aa, cudaStr
   const double flops = 2.0 * M * L->N * L->K;
   const double state = (double)L->N * L->K * 24.0 + (double)L->N * (aa.nrb * 4.0 + 28);
   aa.keep_dW = L->cfg.keep_grad ? L->dW : nullptr;
-  if (!L->is_bf16 && simt_wgrad_adam_fits(M, L->N, L->K)) {
+  if (!L->is_bf16 && f32_wgrad_adam_fits(M, L->N, L->K)) {
     FF_LAUNCH(K_WGRAD_SIMT, flops, st,
-              simt_gemm_wgrad_adam(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(X), L->ldK, M,
+              f32_gemm_wgrad_adam(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(X), L->ldK, M,
                                    aa, st),
               "weight-gradient GEMM and Adam (fp32)");
     return FF_OK;
@@ -313,8 +313,8 @@ ff_status weight_update(ff_layer* L, const void* X, int M, AdamArgs& aa, cudaStr
               "weight-gradient GEMM (tcgen05)");
   } else {
     FF_LAUNCH(K_WGRAD_SIMT, flops, st,
-              simt_gemm_wgrad(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(X), L->ldK, M, L->N,
-                              L->K, L->dW, L->K, st),
+              f32_gemm_wgrad(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(X), L->ldK, M, L->N,
+                              L->K, L->dW, L->K, &L->ds->err, st),
               "weight-gradient GEMM (fp32)");
   }
   // Data nobody reads after this step, so its dirty lines need not reach HBM:
@@ -500,7 +500,7 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
   int ldmax = 0, ntmax = 0;
   for (int k = 0; k < n_layers; ++k) {
     if (layers[k]->ldN > ldmax) ldmax = layers[k]->ldN;
-    const int nt = b16 || f32tc ? tc_fwd_ntiles_max(layers[k]->N) : simt_fwd_ntiles_max(layers[k]->N);
+    const int nt = b16 || f32tc ? tc_fwd_ntiles_max(layers[k]->N) : f32_fwd_ntiles_max(layers[k]->N);
     if (nt > ntmax) ntmax = nt;
   }
   // Samples per chunk: about 40 MB of activations per buffer, so that one
@@ -592,7 +592,7 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
                 "layer-1 base GEMM (fp32, tcgen05 TF32 x 3)");
     } else {
       FF_LAUNCH(K_STORE_SIMT, 2.0 * cn * N1 * L0->K, st,
-                simt_gemm_store(static_cast<const float*>(X0), L0->ldK, L0->W, L0->K, cn, N1, L0->K, base, L0->ldN,
+                f32_gemm_store(static_cast<const float*>(X0), L0->ldK, L0->W, L0->K, cn, N1, L0->K, base, L0->ldN,
                                 st),
                 "layer-1 base GEMM (fp32)");
     }
@@ -631,10 +631,10 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
                                   err, st),
                   "predict forward GEMM (fp32, tcgen05 TF32 x 3)");
       } else {
-        nt = simt_fwd_ntiles(rows, Lk->N, Lk->K);
+        nt = f32_fwd_ntiles(rows, Lk->N, Lk->K);
         FF_LAUNCH(K_FWD_SIMT, 2.0 * rows * Lk->N * Lk->K, st,
-                  simt_gemm_fwd(static_cast<const float*>(Hb[cur]), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, rows, ep,
-                                st),
+                  f32_gemm_fwd(static_cast<const float*>(Hb[cur]), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, rows, ep,
+                               err, st),
                   "predict forward GEMM (fp32)");
       }
       nt_prev = nt;

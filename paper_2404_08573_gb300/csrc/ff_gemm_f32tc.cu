@@ -1,0 +1,310 @@
+// fp32 GEMMs on the tensor cores without loss of precision, for the exact fp32
+// mode's larger training GEMMs (the contracts of ff_gemm_simt.cu).
+//
+// Each fp32 operand value enters as three bf16 parts, hi = rn(x), mid =
+// rn(x - hi), lo = x - hi - mid (exact): 24 bits in all.  Six of the nine
+// part products are formed (lo-hi, mid-mid, mid-hi and hi-hi, both ways); the
+// three dropped ones are below 2^-25 of the term.  Every product is exact in
+// fp32.  The tensor cores' running sum is not rounded to nearest, and a sum of
+// K terms left in it drifts by up to K/16 6 2^-24 of its size (the three-TF32
+// forward of goodness predict shows that drift, 2e-5 at K = 2000): so only 64
+// terms are summed there, the small products first, and each such chunk is
+// added to fp32 registers with ordinary rounded adds.  Measured against 64
+// bits (2-norm), 2000-wide activities over K = 2000: 1.2e-7 with one K slice,
+// 1.0e-7 with four; the CUDA-core GEMM 7.3e-7 and 3.3e-7.
+//
+// Split of the work: a CTA makes a 128 x 128 tile over one slice of K (up to
+// four slices, the CTAs of a cluster, added through distributed shared memory
+// as in ff_gemm_simt.cu), with
+//   warps 0..7   load both operands' 128 x 64 fp32 tiles from L2 into
+//                registers, half a stage ahead, and write the three parts as
+//                128-byte-swizzled tiles into a two-stage ring (96 KB a stage)
+//   warp 8       one lane issues the MMAs of each 64-deep chunk (24 of M = N
+//                = 128, K = 16) into one of four TMEM buffers
+//   warps 8..15  add each finished chunk to their registers (a 32-row quarter
+//                of TMEM and half the columns each), then run the epilogue
+// Bound by shared memory and the splitting: a chunk's 24 MMAs read 192 KB of
+// operands (1536 clocks at 128 bytes a clock, as long as their arithmetic),
+// its 16,384 values are written as 96 KB of parts and cost about 7
+// instructions each; measured 1.7 us a chunk, 136 TFLOP/s of fp32 terms on
+// the 2048-row weight gradient (the CUDA-core GEMM reaches 50).
+// Infinities and values that round to infinity in bf16 come out as NaN
+// (inf - inf), which the non-finite check reports as it does infinities.
+#include "ff_f32_epilogue.cuh"
+#include "ff_internal.cuh"
+#include "ff_ptx.cuh"
+
+namespace ff {
+namespace {
+
+constexpr int T = 128;          // rows and columns of a CTA's tile
+constexpr int KC = 64;          // K per chunk: one 128-byte row of bf16
+constexpr int STAGES = 2;
+constexpr int PART_BYTES = T * KC * 2;      // one part of one operand
+constexpr int OP_BYTES = 3 * PART_BYTES;
+constexpr int STAGE_BYTES = 2 * OP_BYTES;
+constexpr int BUFS = 4;         // TMEM chunk buffers of T columns
+constexpr int LOAD_WARPS = 8, SUM_WARPS = 8;
+constexpr int NTHREADS = 32 * (LOAD_WARPS + SUM_WARPS);
+constexpr int LD = f32_tile_ld(T);
+constexpr int SMEM = STAGES * STAGE_BYTES + 1024 /*alignment*/ + 256 /*barriers*/;
+static_assert(T * LD * 4 <= STAGES * STAGE_BYTES, "the partial tile takes the ring's place");
+static_assert(SMEM > 113 * 1024 && SMEM <= 227 * 1024, "one tensor-core GEMM CTA per SM: no TMEM allocation waits");
+
+// The three bf16 parts of x0 (low halves) and x1 (high halves).
+__device__ __forceinline__ uint32_t cvt2(float x0, float x1) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(x0, x1);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ void split2(float x0, float x1, uint32_t (&p)[3]) {
+  p[0] = cvt2(x0, x1);
+  x0 = __fsub_rn(x0, __uint_as_float(p[0] << 16));
+  x1 = __fsub_rn(x1, __uint_as_float(p[0] & 0xFFFF0000u));
+  p[1] = cvt2(x0, x1);
+  x0 = __fsub_rn(x0, __uint_as_float(p[1] << 16));
+  x1 = __fsub_rn(x1, __uint_as_float(p[1] & 0xFFFF0000u));
+  p[2] = cvt2(x0, x1);
+}
+
+// A loader thread's share of one operand's 128 x 64 fp32 tile: 8 words of 4
+// values.  Tile row i of 128 holds 64 values contiguous in memory: K-major
+// operands, row r0 + i, K k0 ..; MN-major ones, K k0 + i % 64, rows r0 + 64
+// (i / 64) ...  16 lanes take a row, a warp two rows at a time.
+template <bool MN>
+__device__ __forceinline__ void load8(float4 (&v)[8], const float* __restrict__ P, int ld, int rows, int K, int r0,
+                                      int k0, int t) {
+  const int c = 4 * (t & 15), r = t >> 4;
+  if (r0 + T <= rows && k0 + KC <= K) {  // the whole tile exists
+    const float* p = MN ? P + (size_t)(k0 + r) * ld + r0 + c : P + (size_t)(r0 + r) * ld + k0 + c;
+    const size_t step = (size_t)16 * ld;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      v[i] = __ldg(reinterpret_cast<const float4*>(MN ? p + (i & 3) * step + (i >> 2) * 64 : p + i * step));
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int row = r + 16 * i;
+    const int slow = MN ? k0 + (row & 63) : r0 + row;
+    const int fast = MN ? r0 + (row >> 6) * 64 + c : k0 + c;
+    const bool ok = slow < (MN ? K : rows) && fast < (MN ? rows : K);
+    v[i] = ok ? __ldg(reinterpret_cast<const float4*>(P + (size_t)slow * ld + fast)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    // a row's padding is never used
+    const int left = (MN ? rows : K) - fast;
+    if (left < 2) v[i].y = 0.f;
+    if (left < 3) v[i].z = 0.f;
+    if (left < 4) v[i].w = 0.f;
+  }
+}
+// Its three parts into the operand's tiles (128-byte rows, 16-byte words
+// permuted by the row's low three bits, the same for all of a thread's rows).
+__device__ __forceinline__ void store8(uint8_t* op, const float4 (&v)[8], int t) {
+  const int c = t & 15, r = t >> 4;
+  uint8_t* dst = op + r * 128 + (((c >> 1) ^ (r & 7)) << 4) + (c & 1) * 8;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    uint32_t a[3], b[3];
+    split2(v[i].x, v[i].y, a);
+    split2(v[i].z, v[i].w, b);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(dst + i * 16 * 128 + p * PART_BYTES) = make_uint2(a[p], b[p]);
+  }
+}
+
+__device__ __forceinline__ void latch(int* err, volatile int* abort_flag) {
+  *abort_flag = 1;
+  atomicOr(err, DEVERR_TIMEOUT);
+}
+
+template <bool MN, int MODE>
+__global__ void __launch_bounds__(NTHREADS, 1)
+    k_f32tc_gemm(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb, int M, int N, int K,
+                 EpiArgs ep, int* err) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = ptx::smem_u32(smem_raw);
+  uint8_t* smem = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+  uint64_t* empty = full + STAGES;
+  uint64_t* tfull = empty + STAGES;
+  uint64_t* tempty = tfull + BUFS;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(tempty + BUFS);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m0 = blockIdx.x * T, n0 = blockIdx.y * T;
+  const int S = gridDim.z;
+  const int chunks = (K + KC - 1) / KC;
+  const int per = (chunks + S - 1) / S;
+  const int c0 = min(chunks, (int)blockIdx.z * per), nc = min(chunks, c0 + per) - c0;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      ptx::mbar_init(&full[s], LOAD_WARPS);
+      ptx::mbar_init(&empty[s], 1);
+    }
+    for (int b = 0; b < BUFS; ++b) {
+      ptx::mbar_init(&tfull[b], 1);
+      ptx::mbar_init(&tempty[b], SUM_WARPS);
+    }
+    *abort_flag = 0;
+    ptx::fence_mbar_init();
+  }
+  if (warp == 0) {
+    ptx::tmem_alloc(tslot, BUFS * T);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = *tslot;
+  ptx::griddep_wait();  // launched with programmatic stream serialization
+
+  if (warp < LOAD_WARPS) {
+    const int t = threadIdx.x;
+    float4 va[8], vb[8];
+    if (nc > 0) {
+      load8<MN>(va, A, lda, M, K, m0, c0 * KC, t);
+      load8<MN>(vb, B, ldb, N, K, n0, c0 * KC, t);
+    }
+    for (int c = 0; c < nc; ++c) {
+      const int s = c % STAGES;
+      const bool ok = ptx::mbar_wait(&empty[s], ((uint32_t)(c / STAGES) & 1u) ^ 1u, kWaitTimeoutNs, abort_flag);
+      if (!ok) latch(err, abort_flag);
+      if (!__all_sync(0xffffffffu, ok && !*abort_flag)) break;
+      uint8_t* op = smem + s * STAGE_BYTES;
+      store8(op, va, t);
+      if (c + 1 < nc) load8<MN>(va, A, lda, M, K, m0, (c0 + c + 1) * KC, t);
+      store8(op + OP_BYTES, vb, t);
+      if (c + 1 < nc) load8<MN>(vb, B, ldb, N, K, n0, (c0 + c + 1) * KC, t);
+      ptx::fence_async_smem();  // read by the MMAs (async proxy)
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&full[s]);
+    }
+  } else {
+    const bool issuer = warp == LOAD_WARPS && lane == 0;
+    // 32 rows (TMEM lanes 32 q ..) x 64 columns of the tile
+    const int q = warp & 3, half = (warp - LOAD_WARPS) >> 2;
+    float acc[64];
+#pragma unroll
+    for (int j = 0; j < 64; ++j) acc[j] = 0.f;
+    bool good = true;
+    // chunk c's MMAs are issued before chunk c - 1 is added
+    for (int c = 0; c <= nc; ++c) {
+      if (issuer && c < nc) {
+        constexpr uint32_t idesc = ptx::idesc_bf16_f32(T, T, MN ? 1 : 0, MN ? 1 : 0);
+        // (A part, B part), the smallest products first
+        constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+        const int s = c % STAGES, b = c % BUFS;
+        if (ptx::mbar_wait(&full[s], (uint32_t)(c / STAGES) & 1u, kWaitTimeoutNs, abort_flag) &&
+            ptx::mbar_wait(&tempty[b], ((uint32_t)(c / BUFS) & 1u) ^ 1u, kWaitTimeoutNs, abort_flag)) {
+          ptx::tc_fence_after();
+          const uint32_t ab = ptx::smem_u32(smem + s * STAGE_BYTES), bb = ab + OP_BYTES;
+#pragma unroll
+          for (int p = 0; p < 6; ++p)
+#pragma unroll
+            for (int k = 0; k < KC / 16; ++k) {
+              // K-major: 32 bytes along the swizzled rows, 8-row groups 1024
+              // bytes apart; MN-major: 16 K rows further, the 64-element
+              // halves 64 rows apart
+              const uint32_t aa = ab + pa[p] * PART_BYTES, ba = bb + pb[p] * PART_BYTES;
+              const uint64_t ad =
+                  MN ? ptx::sdesc_sw128(aa + k * 2048, 64 * 128, 1024) : ptx::sdesc_sw128(aa + k * 32, 16, 1024);
+              const uint64_t bd =
+                  MN ? ptx::sdesc_sw128(ba + k * 2048, 64 * 128, 1024) : ptx::sdesc_sw128(ba + k * 32, 16, 1024);
+              ptx::umma_f16(tmem + (uint32_t)(b * T), ad, bd, idesc, (p | k) != 0 ? 1u : 0u);
+            }
+          ptx::umma_commit(&empty[s]);
+          ptx::umma_commit(&tfull[b]);
+        } else {
+          latch(err, abort_flag);
+        }
+      }
+      __syncwarp();
+      if (c == 0) continue;
+      const int b = (c - 1) % BUFS;
+      const bool ok = ptx::mbar_wait(&tfull[b], (uint32_t)((c - 1) / BUFS) & 1u, kWaitTimeoutNs, abort_flag);
+      if (!ok) latch(err, abort_flag);
+      good = __all_sync(0xffffffffu, ok && !*abort_flag);
+      if (!good) break;
+      ptx::tc_fence_after();
+      const uint32_t src = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * T + half * 64);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t r[32];
+        ptx::tmem_ld32(src + 32 * h, r);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[32 * h + j] = __fadd_rn(acc[32 * h + j], __uint_as_float(r[j]));
+      }
+      ptx::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&tempty[b]);
+    }
+    if (!good) {
+      // MMAs already issued finish before TMEM is released
+      const uint64_t t0 = ptx::globaltimer();
+      while (ptx::globaltimer() - t0 < 1000000ull) {
+      }
+    }
+    // every chunk is summed, so every MMA has read the ring: the partial tile
+    // takes its place (all warps of this role first)
+    ptx::named_bar(1, 32 * SUM_WARPS);
+    float* row = reinterpret_cast<float*>(smem) + (q * 32 + lane) * LD + half * 64;
+    if (good) {
+#pragma unroll
+      for (int j = 0; j < 64; j += 4)
+        *reinterpret_cast<float4*>(row + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+    }
+  }
+  if (threadIdx.x == 0) ptx::griddep_launch_dependents();
+  ptx::tc_fence_before();
+  if (S > 1)
+    ptx::cluster_sync();  // every partial of the tile is in place
+  else
+    __syncthreads();
+  if (warp >= LOAD_WARPS) {
+    if (!*abort_flag)
+      f32_tile_epilogue<T, MODE>(reinterpret_cast<const float*>(smem), (int)threadIdx.x - 32 * LOAD_WARPS, M, N, m0, n0,
+                                 S, ep, AdamArgs{});
+  } else if (warp == 0) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, BUFS * T);
+  }
+  if (S > 1) ptx::cluster_sync();  // no CTA leaves while another reads its partial tile
+}
+
+template <bool MN, int MODE>
+cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, const EpiArgs& ep,
+                   int* err, cudaStream_t st) {
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(k_f32tc_gemm<MN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+  if (attr != cudaSuccess) return attr;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cdiv(M, T), cdiv(N, T), S);
+  cfg.blockDim = dim3(NTHREADS);
+  cfg.dynamicSmemBytes = SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = 1;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = S;
+  cfg.attrs = at;
+  cfg.numAttrs = S > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, k_f32tc_gemm<MN, MODE>, A, lda, B, ldb, M, N, K, ep, err);
+}
+
+}  // namespace
+
+cudaError_t f32tc_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S,
+                           const EpiArgs& ep, int* err, cudaStream_t st) {
+  return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, S, ep, err, st);
+}
+
+cudaError_t f32tc_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, int S, float* C,
+                             int ldc, int* err, cudaStream_t st) {
+  EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
+  return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, S, ep, err, st);
+}
+
+}  // namespace ff

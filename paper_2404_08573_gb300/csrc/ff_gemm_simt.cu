@@ -20,16 +20,14 @@
 // shared memory and runs the epilogue on them -- no scratch in device memory
 // and no counters.
 #include "ff_adam.cuh"
+#include "ff_f32_epilogue.cuh"
 #include "ff_internal.cuh"
 #include "ff_ptx.cuh"
 
 namespace ff {
 namespace {
 
-constexpr int NT = 256;
 constexpr int TKS = 32;  // K per stage
-constexpr int MODE_FWD = 0, MODE_STORE = 1, MODE_ADAM = 2;
-constexpr int kMaxSplit = 4;  // CTAs per cluster (see plan_of)
 
 // Shape of one instance.  An operand's stage sits in shared memory as TKS
 // rows (one per K) of the tile's T rows or columns, padded by 4 floats.
@@ -37,7 +35,7 @@ template <int T, int KGRP>
 struct Cfg {
   static constexpr int TM = T, TN = T, KG = KGRP;
   static constexpr int TT = T / 8;                 // threads along each side of a K group's tile
-  static constexpr int LD = T + 4;
+  static constexpr int LD = f32_tile_ld(T);
   static constexpr int OP = TKS * LD;              // floats of one operand's stage
   static constexpr int STAGES = T == 128 ? 3 : 4;
   static constexpr int RING = 2 * OP * STAGES;
@@ -55,15 +53,6 @@ __device__ __forceinline__ void cp_async4(float* dst, const float* src, int byte
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ float4 ld_cluster4(const float* local, uint32_t rank) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(ptx::mapa_shared(ptx::smem_u32(local), rank))
-               : "memory");
-  return v;
-}
-
 // Two fp32 FMAs in one instruction, each rounded as fmaf.
 __device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
   unsigned long long v;
@@ -229,147 +218,57 @@ __global__ void __launch_bounds__(NT, 2)
   else
     __syncthreads();
 
-  // the epilogue on this CTA's TM / S rows of the tile
-  const int RS = C::TM / S;
-  const int col = n0 + lc;
-  // four values of row r of the tile: the sum of the S partials in rank order
-  auto tile4 = [&](int r, float (&v)[4]) {
-    if (S > 1) {
-      float4 u[kMaxSplit];
-#pragma unroll
-      for (int z = 0; z < kMaxSplit; ++z)
-        if (z < S) u[z] = ld_cluster4(sm + r * C::LD + lc, (uint32_t)z);
-      v[0] = v[1] = v[2] = v[3] = 0.f;
-#pragma unroll
-      for (int z = 0; z < kMaxSplit; ++z)
-        if (z < S) {
-          v[0] += u[z].x; v[1] += u[z].y; v[2] += u[z].z; v[3] += u[z].w;
-        }
-    } else {
-      const float4 u = *reinterpret_cast<const float4*>(sm + r * C::LD + lc);
-      v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
-    }
-  };
-  if constexpr (MODE == MODE_ADAM) {
-    // Adam on the tile's weights: the state of kBatch rows in flight at a time
-    constexpr int kBatch = 4;
-    const float a1 = ad.lr / ad.ds->bc1, r2 = 1.f / ad.ds->bc2;
-    const bool vec = (ad.K & 3) == 0;
-    for (int p = 0; p < RS; p += kBatch * RPP) {
-      AdamVec st[kBatch];
-#pragma unroll
-      for (int q = 0; q < kBatch; ++q) {
-        const int o = p + q * RPP + lr;
-        const int gi = m0 + (int)blockIdx.z * RS + o;
-        if (vec && o < RS && gi < M && col < N) st[q].load(ad, (size_t)gi * N + col);
-      }
-#pragma unroll
-      for (int q = 0; q < kBatch; ++q) {
-        const int o = p + q * RPP + lr;
-        const int gi = m0 + (int)blockIdx.z * RS + o;
-        if (o >= RS || gi >= M || col >= N) continue;
-        float v[4];
-        tile4((int)blockIdx.z * RS + o, v);
-        const size_t idx = (size_t)gi * N + col;
-        if (vec) {
-          const float4 dw = make_float4(v[0], v[1], v[2], v[3]);
-          if (ad.keep_dW) *reinterpret_cast<float4*>(ad.keep_dW + idx) = dw;
-          st[q].update(ad, dw, a1, r2);
-          st[q].store(ad, idx);
-        } else {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            if (col + e >= N) break;
-            float w = ad.W[idx + e], m = ad.mW[idx + e], vv = ad.vW[idx + e];
-            adam1(w, m, vv, v[e], a1, ad.beta1, ad.beta2, ad.eps, r2);
-            ad.W[idx + e] = w;
-            ad.mW[idx + e] = m;
-            ad.vW[idx + e] = vv;
-            if (ad.keep_dW) ad.keep_dW[idx + e] = v[e];
-          }
-        }
-      }
-    }
-  } else {
-    for (int p = 0; p < RS; p += RPP) {
-      const int r = (int)blockIdx.z * RS + p + lr;
-      const bool row_ok = p + lr < RS && m0 + r < M;
-      const int gi = m0 + r;
-      float v[4] = {0.f, 0.f, 0.f, 0.f};
-      if (row_ok) tile4(r, v);
-      if (MODE == MODE_FWD) {
-        float g = 0.f;
-        if (row_ok) {
-          const float s = __ldg(ep.row_scale + gi);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            float h = 0.f;
-            if (col + e < N) {
-              float z = s * v[e];
-              if (ep.bias) z += __ldg(ep.bias + col + e);
-              h = z != z ? z : fmaxf(z, 0.f);  // ReLU, NaN kept for the non-finite check
-            }
-            g = fmaf(h, h, g);
-            v[e] = h;
-          }
-          // activation rows are padded to multiples of 8: whole 16-byte words
-          if (col < ep.ldo)
-            *reinterpret_cast<float4*>(static_cast<float*>(ep.out) + (size_t)gi * ep.ldo + col) =
-                make_float4(v[0], v[1], v[2], v[3]);
-        }
-        // the LPR lanes sharing this row
-#pragma unroll
-        for (int o = LPR / 2; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-        if (lc == 0 && row_ok) ep.gpart[(size_t)blockIdx.y * M + gi] = g;
-      } else if (row_ok) {
-        float* out = static_cast<float*>(ep.out) + (size_t)gi * ep.ldo + col;
-        if ((ep.ldo & 3) == 0 && col + 4 <= N) {
-          *reinterpret_cast<float4*>(out) = make_float4(v[0], v[1], v[2], v[3]);
-        } else {
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (col + e < N) out[e] = v[e];
-        }
-      }
-    }
-  }
+  f32_tile_epilogue<T, MODE>(sm, tid, M, N, m0, n0, S, ep, ad);
   if (S > 1) ptx::cluster_sync();  // no CTA leaves while another reads its partial tile
 }
 
-// Tile shape and number of K slices for an M x N output over K: the least
-// modelled time.  Measured: a CTA takes 0.95 us per stage of a 64 x 64 tile
-// and 3.3 us of a 128 x 128 one (42 and 48 TFLOP/s over 152 SMs) whether or
-// not it shares its SM -- the shared-memory operand reads and the FMAs fill
-// the SM's time -- so a GEMM takes the stages that the fullest SM runs; a
-// split costs about 1 us more.  Eight slices measured no faster than four at
-// any size (forward of 128 rows, 784 -> 500: 15.2 us with 4, 16.6 with 8;
-// clusters of 8 find fewer places).  That forward took 22 us with one CTA
-// per 128 x 128 tile and slice and partials through device memory; 512 rows
-// of 2000 -> 2000 122 us against 113 now, their weight gradient 118 against
-// 94.
+// How an M x N output over K is computed: on the CUDA cores in 64 x 64 or
+// 128 x 128 tiles, or on the tensor cores (ff_gemm_f32tc.cu) in 128 x 128
+// tiles, and in how many K slices: the least modelled time.  Measured: a CTA
+// takes 0.95 us per 32-deep stage of a 64 x 64 tile and 3.3 us of a 128 x 128
+// one (42 and 48 TFLOP/s over 152 SMs) whether or not it shares its SM -- the
+// shared-memory operand reads and the FMAs fill the SM's time -- and 1.7 us
+// per 64-deep chunk of a tensor-core tile, an SM to itself, with about 9 us
+// before and after its mainloop against 5.  A GEMM takes the stages that the
+// fullest SM runs; a split costs about 1 us more.  Eight slices measured no
+// faster than four at any size (clusters of 8 find fewer places).
+// Rows x K -> N, us: one 128 x 128 tile per CTA and partial tiles through
+// device memory (as before) / CUDA cores / tensor cores:
+//   128 x 784 -> 500    22 / 15 / 20      (CUDA cores chosen)
+//   128 x 2000 -> 2000  -- / 39 / 27      (tensor cores from here on)
+//   512 x 2000 -> 2000  122 / 113 / 44    weight gradient 118 / 94 / 41
+//   2048 x 2000 -> 2000 480 / 367 / 139   weight gradient 416 / 322 / 120
+enum Kind { TILE_64, TILE_128, TENSOR };
 struct Plan {
-  bool large;
+  Kind kind;
   int S;
 };
-Plan plan_of(int M, int N, int K) {
-  const int steps = cdiv(K, TKS);
-  Plan best{true, 1};
+Plan plan_of(int M, int N, int K, bool tensor) {
+  Plan best{TILE_128, 1};
   double bt = 0.0;
-  for (int large = 1; large >= 0; --large) {
-    const int T = large ? 128 : 64;
+  for (int kind = tensor ? TENSOR : TILE_128; kind >= TILE_64; --kind) {
+    const int T = kind == TILE_64 ? 64 : 128;
+    const int steps = cdiv(K, kind == TENSOR ? 64 : TKS);
     const double tiles = (double)cdiv(M, T) * cdiv(N, T);
     for (int S = 1; S <= kMaxSplit; S *= 2) {
       if (S > 1 && steps < 2 * S) break;
       const double per_sm = cdiv((long long)(tiles * S), 152);  // CTAs an SM runs in all
-      const double t = per_sm * cdiv(steps, S) * (large ? 3.3 : 0.95) + (S > 1 ? 1.0 : 0.0);
+      const double step = kind == TILE_64 ? 0.95 : kind == TILE_128 ? 3.3 : 1.7;
+      const double t = (kind == TENSOR ? per_sm * (cdiv(steps, S) * step + 9.0) : per_sm * cdiv(steps, S) * step + 5.0) +
+                       (S > 1 ? 1.0 : 0.0);
       if (bt == 0.0 || t < bt) {
         bt = t;
-        best = Plan{large != 0, S};
+        best = Plan{(Kind)kind, S};
       }
     }
   }
   return best;
 }
+// The tensor-core form needs 16-byte aligned rows of both operands: for the
+// forward and store, of the weights (rows of K).
+Plan plan_kmajor(int M, int N, int K) { return plan_of(M, N, K, (K & 3) == 0); }
+
+bool aligned(const float* p, int ld) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (ld & 3) == 0; }
 
 template <int T, int KGRP, bool MN, int MODE>
 cudaError_t launch_plan(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, const EpiArgs& ep,
@@ -378,7 +277,6 @@ cudaError_t launch_plan(const float* A, int lda, const float* B, int ldb, int M,
   static const cudaError_t attr = cudaFuncSetAttribute(k_simt_gemm<T, KGRP, MN, MODE>,
                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (attr != cudaSuccess) return attr;
-  auto vec = [](const float* p, int ld) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (ld & 3) == 0; };
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cdiv(M, T), cdiv(N, T) + (MODE == MODE_ADAM ? 1 : 0), S);
   cfg.blockDim = dim3(NT);
@@ -394,49 +292,55 @@ cudaError_t launch_plan(const float* A, int lda, const float* B, int ldb, int M,
   cfg.attrs = at;
   cfg.numAttrs = S > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k_simt_gemm<T, KGRP, MN, MODE>, A, lda, B, ldb, M, N, K,
-                            (vec(A, lda) ? 1 : 0) | (vec(B, ldb) ? 2 : 0), ep, ad);
+                            (aligned(A, lda) ? 1 : 0) | (aligned(B, ldb) ? 2 : 0), ep, ad);
 }
 
 template <bool MN, int MODE>
 cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int N, int K, Plan p, const EpiArgs& ep,
                    const AdamArgs& ad, cudaStream_t st) {
-  if (p.large) return launch_plan<128, 1, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, ad, st);
+  if (p.kind != TILE_64) return launch_plan<128, 1, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, ad, st);
   return launch_plan<64, 4, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, ad, st);
 }
 
 }  // namespace
 
-int simt_fwd_ntiles(int M, int N, int K) { return cdiv(N, plan_of(M, N, K).large ? 128 : 64); }
-int simt_fwd_ntiles_max(int N) { return cdiv(N, 64); }
+int f32_fwd_ntiles(int plan_rows, int N, int K) { return cdiv(N, plan_kmajor(plan_rows, N, K).kind == TILE_64 ? 64 : 128); }
+int f32_fwd_ntiles_max(int N) { return cdiv(N, 64); }
 
-cudaError_t simt_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
-                          const EpiArgs& ep, cudaStream_t st) {
-  return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, plan_of(plan_rows, N, K), ep, AdamArgs{}, st);
+cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
+                         const EpiArgs& ep, int* err, cudaStream_t st) {
+  const Plan p = plan_kmajor(plan_rows, N, K);
+  if (p.kind == TENSOR && aligned(A, lda) && aligned(B, ldb))
+    return f32tc_gemm_fwd(A, lda, B, ldb, M, N, K, p.S, ep, err, st);
+  return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, p, ep, AdamArgs{}, st);
 }
 
-cudaError_t simt_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, float* C, int ldc,
-                            cudaStream_t st) {
+cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, float* C, int ldc,
+                           cudaStream_t st) {
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, plan_of(M, N, K), ep, AdamArgs{}, st);
+  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, plan_of(M, N, K, false), ep, AdamArgs{}, st);
 }
 
-cudaError_t simt_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, float* C, int ldc,
-                            cudaStream_t st) {
-  // C[n, k] = sum_r G[r, n] X[r, k]: rows of C index G's columns (MN-major A),
-  // columns of C index X's columns (MN-major B), contraction over R.
+// C[n, k] = sum_r G[r, n] X[r, k]: rows of C index G's columns (MN-major A),
+// columns of C index X's columns (MN-major B), contraction over R.
+cudaError_t f32_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, float* C, int ldc,
+                           int* err, cudaStream_t st) {
+  const Plan p = plan_of(N, K, R, true);
+  if (p.kind == TENSOR && aligned(G, ldg) && aligned(X, ldx))
+    return f32tc_gemm_wgrad(G, ldg, X, ldx, R, N, K, p.S, C, ldc, err, st);
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, plan_of(N, K, R), ep, AdamArgs{}, st);
+  return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, p, ep, AdamArgs{}, st);
 }
 
-bool simt_wgrad_adam_fits(int R, int N, int K) {
-  const Plan p = plan_of(N, K, R);
-  const int T = p.large ? 128 : 64;
-  return (long long)cdiv(N, T) * cdiv(K, T) * p.S <= 2 * 152;
+bool f32_wgrad_adam_fits(int R, int N, int K) {
+  const Plan p = plan_of(N, K, R, true);
+  const int T = p.kind == TILE_64 ? 64 : 128;
+  return p.kind != TENSOR && (long long)cdiv(N, T) * cdiv(K, T) * p.S <= 2 * 152;
 }
 
-cudaError_t simt_gemm_wgrad_adam(const float* G, int ldg, const float* X, int ldx, int R, const AdamArgs& a,
-                                 cudaStream_t st) {
-  return launch<true, MODE_ADAM>(G, ldg, X, ldx, a.N, a.K, R, plan_of(a.N, a.K, R), EpiArgs{}, a, st);
+cudaError_t f32_gemm_wgrad_adam(const float* G, int ldg, const float* X, int ldx, int R, const AdamArgs& a,
+                                cudaStream_t st) {
+  return launch<true, MODE_ADAM>(G, ldg, X, ldx, a.N, a.K, R, plan_of(a.N, a.K, R, true), EpiArgs{}, a, st);
 }
 
 }  // namespace ff

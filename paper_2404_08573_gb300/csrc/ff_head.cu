@@ -1029,7 +1029,7 @@ ff_status head_workspace(ff_head* hd, ff_layer* const* layers, int L, int rows, 
   const size_t es = b16 ? 2 : 4;
   int ntmax = 0;
   for (int k = 0; k < L; ++k) {
-    const int nt = b16 ? tc_fwd_ntiles_max(layers[k]->N) : simt_fwd_ntiles_max(layers[k]->N);
+    const int nt = b16 ? tc_fwd_ntiles_max(layers[k]->N) : f32_fwd_ntiles_max(layers[k]->N);
     if (nt > ntmax) ntmax = nt;
   }
   size_t off = 0;
@@ -1109,10 +1109,10 @@ ff_status head_forward(ff_layer* const* layers, int L, const float* x, int rows,
                 "head forward GEMM (tcgen05)");
     } else {
       const int plan_rows = narrow ? rows : kTrainPlanRows;
-      nt = simt_fwd_ntiles(plan_rows, Lk->N, Lk->K);
+      nt = f32_fwd_ntiles(plan_rows, Lk->N, Lk->K);
       FF_LAUNCH(K_FWD_SIMT, 2.0 * rows * Lk->N * Lk->K, st,
-                simt_gemm_fwd(static_cast<const float*>(in), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, plan_rows, ep,
-                              st),
+                f32_gemm_fwd(static_cast<const float*>(in), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, plan_rows, ep,
+                             err, st),
                 "head forward GEMM (fp32)");
     }
     nt_prev = nt;
@@ -1665,9 +1665,9 @@ ff_status ff_po_train_step(ff_layer* L, ff_head* hd, const void* x, int raw_inpu
               tc_gemm_fwd(static_cast<const bf16*>(X), L->ldK, L->Wb, L->ldK, n, N, K, ep, &L->ds->err, st),
               "forward GEMM (tcgen05)");
   } else {
-    ntiles = simt_fwd_ntiles(n, N, K);
+    ntiles = f32_fwd_ntiles(n, N, K);
     FF_LAUNCH(K_FWD_SIMT, 2.0 * n * N * K, st,
-              simt_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, n, N, K, n, ep, st), "forward GEMM (fp32)");
+              f32_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, n, N, K, n, ep, &L->ds->err, st), "forward GEMM (fp32)");
   }
   if (!b16) {
     // the block on the raw activity: logits, cross-entropy, dz

@@ -207,7 +207,7 @@ struct AdamArgs {
   int ndead;
   char* dead[2];
   long long dead_lines[2];
-  // simt_gemm_wgrad_adam, which forms dW itself: where to keep it
+  // f32_gemm_wgrad_adam, which forms dW itself: where to keep it
   // (ff_layer_get_grad), or null
   float* keep_dW;
 };
@@ -325,29 +325,37 @@ bool make_plain_map(CUtensorMap* m, const void* ptr, int esize, int cols, int ro
 bool make_sw128_map(CUtensorMap* m, const void* ptr, int esize, int cols, int rows, int ld, int box_cols,
                     int box_rows);
 
-// SIMT fp32 GEMMs with the same contracts.  The tile shape and the split of
-// the contraction depend on the output's shape; for the forward, on plan_rows
+// fp32 GEMMs of the exact mode with the same contracts, on the CUDA cores or,
+// where the GEMM is large enough and its rows are 16-byte aligned, on the
+// tensor cores as six products of bf16 parts per term (no precision lost; err
+// then latches a wait that ran out).  The tile shape and the split of the
+// contraction depend on the output's shape; for the forward, on plan_rows
 // rows instead of M, so that a chain whose per-row results must not depend on
-// how many rows share a GEMM passes a constant.  simt_fwd_ntiles(plan_rows,
+// how many rows share a GEMM passes a constant.  f32_fwd_ntiles(plan_rows,
 // ...): goodness partials per row it then writes; _max: the most for any rows.
-int simt_fwd_ntiles(int plan_rows, int N, int K);
-int simt_fwd_ntiles_max(int N);
-cudaError_t simt_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
-                          const EpiArgs& ep, cudaStream_t st);
-cudaError_t simt_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K,
-                            float* C, int ldc, cudaStream_t st);
-cudaError_t simt_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K,
-                            float* C, int ldc, cudaStream_t st);
+int f32_fwd_ntiles(int plan_rows, int N, int K);
+int f32_fwd_ntiles_max(int N);
+cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
+                         const EpiArgs& ep, int* err, cudaStream_t st);
+cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K,
+                           float* C, int ldc, cudaStream_t st);
+cudaError_t f32_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K,
+                           float* C, int ldc, int* err, cudaStream_t st);
+// The tensor-core forms (S: slices of K), ff_gemm_f32tc.cu.
+cudaError_t f32tc_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S,
+                           const EpiArgs& ep, int* err, cudaStream_t st);
+cudaError_t f32tc_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, int S,
+                             float* C, int ldc, int* err, cudaStream_t st);
 // The weight gradient of a.N x a.K outputs over R rows and the Adam step it
 // feeds, in the GEMM's epilogue (dW itself only to a.keep_dW).  Pays where
-// the GEMM's CTAs are all resident at once (simt_wgrad_adam_fits): the step
+// the GEMM's CTAs are all resident at once (f32_wgrad_adam_fits): the step
 // is latency-bound and a launch shorter (784-500-500, batch 64: 9.8 us against
 // 7 + 5).  A larger GEMM fills the FMA pipes, and a separate Adam, bound by
 // HBM, runs beside the other layers' GEMMs: 784-2000x4, batch 256, two steps
 // 1542 us against 1622 with Adam in every epilogue.
-bool simt_wgrad_adam_fits(int R, int N, int K);
-cudaError_t simt_gemm_wgrad_adam(const float* G, int ldg, const float* X, int ldx, int R, const AdamArgs& a,
-                                 cudaStream_t st);
+bool f32_wgrad_adam_fits(int R, int N, int K);
+cudaError_t f32_gemm_wgrad_adam(const float* G, int ldg, const float* X, int ldx, int R, const AdamArgs& a,
+                                cudaStream_t st);
 
 }  // namespace ff
 

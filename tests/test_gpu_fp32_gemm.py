@@ -1,7 +1,7 @@
-"""The fp32 CUDA-core GEMMs at the edges of their tiles, stages and K slices:
-forward and weight gradient of an fp32 layer against float64 products, within
-the bound of a K-term fp32 sum (K + 8 roundings of 2^-24 of the terms'
-absolute sum, whatever the order)."""
+"""The fp32 GEMMs (CUDA cores, and bf16 parts on the tensor cores) at the edges
+of their tiles, stages and K slices: forward and weight gradient of an fp32
+layer against float64 products, within the bound of a K-term fp32 sum (K + 8
+roundings of 2^-24 of the terms' absolute sum, whatever the order)."""
 
 import numpy as np
 import pytest
@@ -15,7 +15,10 @@ pytestmark = pytest.mark.gpu
 # multiple of 4 (unaligned weight rows); one and several K slices, ragged
 # stages; outputs of many large tiles
 SHAPES = [(2, 10, 8), (2, 33, 1), (62, 31, 63), (64, 32, 64), (66, 65, 65), (128, 784, 500), (130, 786, 129),
-          (254, 1001, 127), (256, 256, 2000), (600, 129, 1023), (1538, 300, 1027)]
+          (254, 1001, 127), (256, 256, 2000), (600, 129, 1023), (1538, 300, 1027),
+          # large enough for the tensor cores: whole tiles; every edge ragged;
+          # a last chunk of 4; several K slices, the last one short
+          (512, 768, 2048), (1022, 1004, 1001), (1150, 2052, 643), (258, 2500, 1500)]
 
 
 @pytest.mark.parametrize("M,K,N", SHAPES)
