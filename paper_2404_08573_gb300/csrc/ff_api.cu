@@ -294,12 +294,12 @@ AdamArgs adam_args(ff_layer* L, int M) {
 
 // The weight gradient from the operand in L->dZ and the layer input X (M
 // rows), and the Adam step: one kernel for small fp32 GEMMs, else the GEMM
-// and the Adam kernel.
-ff_status weight_update(ff_layer* L, const void* X, int M, AdamArgs& aa, cudaStream_t st) {
+// and the Adam kernel.  in_order: see kF32InOrder.
+ff_status weight_update(ff_layer* L, const void* X, int M, AdamArgs& aa, cudaStream_t st, bool in_order) {
   const double flops = 2.0 * M * L->N * L->K;
   const double state = (double)L->N * L->K * 24.0 + (double)L->N * (aa.nrb * 4.0 + 28);
   aa.keep_dW = L->cfg.keep_grad ? L->dW : nullptr;
-  if (!L->is_bf16 && f32_wgrad_adam_fits(M, L->N, L->K)) {
+  if (!L->is_bf16 && !in_order && f32_wgrad_adam_fits(M, L->N, L->K)) {
     FF_LAUNCH(K_WGRAD_SIMT, flops, st,
               f32_gemm_wgrad_adam(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(X), L->ldK, M,
                                    aa, st),
@@ -314,7 +314,7 @@ ff_status weight_update(ff_layer* L, const void* X, int M, AdamArgs& aa, cudaStr
   } else {
     FF_LAUNCH(K_WGRAD_SIMT, flops, st,
               f32_gemm_wgrad(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(X), L->ldK, M, L->N,
-                              L->K, L->dW, L->K, &L->ds->err, st),
+                              L->K, L->dW, L->K, in_order, &L->ds->err, st),
               "weight-gradient GEMM (fp32)");
   }
   // Data nobody reads after this step, so its dirty lines need not reach HBM:

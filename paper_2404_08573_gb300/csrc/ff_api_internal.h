@@ -27,7 +27,7 @@ ff_status ensure_capacity(ff_layer* L, int rows);
 // The end of a train step on M rows: Adam arguments of the layer, and the
 // weight gradient (from L->dZ and the layer input X) with the Adam step.
 AdamArgs adam_args(ff_layer* L, int M);
-ff_status weight_update(ff_layer* L, const void* X, int M, AdamArgs& aa, cudaStream_t st);
+ff_status weight_update(ff_layer* L, const void* X, int M, AdamArgs& aa, cudaStream_t st, bool in_order = false);
 
 // One layer-local train step (see ff_layer_train_step).  ev_input_read, if
 // not null, is recorded once the raw input x has been consumed (after the

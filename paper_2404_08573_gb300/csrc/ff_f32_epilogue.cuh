@@ -116,34 +116,40 @@ __device__ __forceinline__ void f32_tile_epilogue(const float* sm, int tid, int 
       for (int q = 0; q < kBatch; ++q) {
         const int o = p + q * RPP + lr;
         const int gi = m0 + (int)blockIdx.z * RS + o;
-        g[q] = 0.f;
-        if (o >= RS || gi >= M) continue;
-        float v[4];
-        tile4((int)blockIdx.z * RS + o, v);
+        const bool row_ok = o < RS && gi < M;
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+        if (row_ok) tile4((int)blockIdx.z * RS + o, v);
+        float own = 0.f;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           float h = 0.f;
-          if (col + e < N) {
-            float z = s[q] * v[e];
-            if (ep.bias) z += bias[e];
+          if (row_ok && col + e < N) {
+            // both roundings spelled out, so that every GEMM form agrees
+            float z = __fmul_rn(s[q], v[e]);
+            if (ep.bias) z = __fadd_rn(z, bias[e]);
             h = z != z ? z : fmaxf(z, 0.f);  // ReLU, NaN kept for the non-finite check
           }
-          g[q] = fmaf(h, h, g[q]);
+          own = fmaf(h, h, own);
           v[e] = h;
         }
+        // the upper half of a row's lanes carries on the lower half's sums
+        // (columns 4 l .. 4 l + 3, then T/2 + 4 l ..): LPR / 2 sums a row
+        g[q] = __shfl_sync(0xffffffffu, own, (int)(threadIdx.x & 31) ^ (LPR / 2));
+#pragma unroll
+        for (int e = 0; e < 4; ++e) g[q] = fmaf(v[e], v[e], g[q]);
         // activation rows are padded to multiples of 8: whole 16-byte words
-        if (col < ep.ldo)
+        if (row_ok && col < ep.ldo)
           *reinterpret_cast<float4*>(static_cast<float*>(ep.out) + (size_t)gi * ep.ldo + col) =
               make_float4(v[0], v[1], v[2], v[3]);
       }
-      // the LPR lanes sharing each row
+      // the upper lanes' sums
 #pragma unroll
       for (int q = 0; q < kBatch; ++q) {
 #pragma unroll
-        for (int o = LPR / 2; o > 0; o >>= 1) g[q] += __shfl_xor_sync(0xffffffffu, g[q], o);
+        for (int o = LPR / 4; o > 0; o >>= 1) g[q] += __shfl_xor_sync(0xffffffffu, g[q], o);
         const int o = p + q * RPP + lr;
         const int gi = m0 + (int)blockIdx.z * RS + o;
-        if (lc == 0 && o < RS && gi < M) ep.gpart[(size_t)blockIdx.y * M + gi] = g[q];
+        if (lc == T / 2 && o < RS && gi < M) ep.gpart[(size_t)blockIdx.y * M + gi] = g[q];
       }
     }
   } else {

@@ -268,6 +268,11 @@ Plan plan_of(int M, int N, int K, bool tensor) {
 // forward and store, of the weights (rows of K).
 Plan plan_kmajor(int M, int N, int K) { return plan_of(M, N, K, (K & 3) == 0); }
 
+// plan_rows = kF32InOrder: each output one ascending chain of FMAs over K.
+Plan plan_fwd(int plan_rows, int N, int K) {
+  return plan_rows == kF32InOrder ? Plan{TILE_128, 1} : plan_kmajor(plan_rows, N, K);
+}
+
 bool aligned(const float* p, int ld) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (ld & 3) == 0; }
 
 template <int T, int KGRP, bool MN, int MODE>
@@ -304,12 +309,12 @@ cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int 
 
 }  // namespace
 
-int f32_fwd_ntiles(int plan_rows, int N, int K) { return cdiv(N, plan_kmajor(plan_rows, N, K).kind == TILE_64 ? 64 : 128); }
+int f32_fwd_ntiles(int plan_rows, int N, int K) { return cdiv(N, plan_fwd(plan_rows, N, K).kind == TILE_64 ? 64 : 128); }
 int f32_fwd_ntiles_max(int N) { return cdiv(N, 64); }
 
 cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
                          const EpiArgs& ep, int* err, cudaStream_t st) {
-  const Plan p = plan_kmajor(plan_rows, N, K);
+  const Plan p = plan_fwd(plan_rows, N, K);
   if (p.kind == TENSOR && aligned(A, lda) && aligned(B, ldb))
     return f32tc_gemm_fwd(A, lda, B, ldb, M, N, K, p.S, ep, err, st);
   return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, p, ep, AdamArgs{}, st);
@@ -324,8 +329,8 @@ cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int
 // C[n, k] = sum_r G[r, n] X[r, k]: rows of C index G's columns (MN-major A),
 // columns of C index X's columns (MN-major B), contraction over R.
 cudaError_t f32_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, float* C, int ldc,
-                           int* err, cudaStream_t st) {
-  const Plan p = plan_of(N, K, R, true);
+                           bool in_order, int* err, cudaStream_t st) {
+  const Plan p = in_order ? Plan{TILE_128, 1} : plan_of(N, K, R, true);
   if (p.kind == TENSOR && aligned(G, ldg) && aligned(X, ldx))
     return f32tc_gemm_wgrad(G, ldg, X, ldx, R, N, K, p.S, C, ldc, err, st);
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};

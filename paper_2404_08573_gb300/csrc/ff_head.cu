@@ -1665,9 +1665,10 @@ ff_status ff_po_train_step(ff_layer* L, ff_head* hd, const void* x, int raw_inpu
               tc_gemm_fwd(static_cast<const bf16*>(X), L->ldK, L->Wb, L->ldK, n, N, K, ep, &L->ds->err, st),
               "forward GEMM (tcgen05)");
   } else {
-    ntiles = f32_fwd_ntiles(n, N, K);
+    ntiles = f32_fwd_ntiles(kF32InOrder, N, K);
     FF_LAUNCH(K_FWD_SIMT, 2.0 * n * N * K, st,
-              f32_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, n, N, K, n, ep, &L->ds->err, st), "forward GEMM (fp32)");
+              f32_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, n, N, K, kF32InOrder, ep,
+                           &L->ds->err, st), "forward GEMM (fp32)");
   }
   if (!b16) {
     // the block on the raw activity: logits, cross-entropy, dz
@@ -1740,7 +1741,7 @@ ff_status ff_po_train_step(ff_layer* L, ff_head* hd, const void* x, int raw_inpu
   FF_TRY(cudaEventRecord(hd->ev_join, hd->side), "event record");
   AdamArgs aa = adam_args(L, n);
   aa.B = n;
-  s = weight_update(L, X, n, aa, st);
+  s = weight_update(L, X, n, aa, st, true);
   if (s != FF_OK) return s;
   FF_TRY(cudaStreamWaitEvent(st, hd->ev_join, 0), "stream wait");
   return FF_OK;

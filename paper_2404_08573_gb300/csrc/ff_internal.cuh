@@ -333,6 +333,11 @@ bool make_sw128_map(CUtensorMap* m, const void* ptr, int esize, int cols, int ro
 // rows instead of M, so that a chain whose per-row results must not depend on
 // how many rows share a GEMM passes a constant.  f32_fwd_ntiles(plan_rows,
 // ...): goodness partials per row it then writes; _max: the most for any rows.
+// plan_rows = kF32InOrder (in_order): CUDA cores, every output one ascending
+// chain of FMAs over K.  The Performance-Optimized step takes it: its
+// gradient jumps where an activity crosses zero, so there another order of
+// the same sums can change single rows' gradients by their whole size.
+constexpr int kF32InOrder = 0;
 int f32_fwd_ntiles(int plan_rows, int N, int K);
 int f32_fwd_ntiles_max(int N);
 cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
@@ -340,7 +345,7 @@ cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M
 cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K,
                            float* C, int ldc, cudaStream_t st);
 cudaError_t f32_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K,
-                           float* C, int ldc, int* err, cudaStream_t st);
+                           float* C, int ldc, bool in_order, int* err, cudaStream_t st);
 // The tensor-core forms (S: slices of K), ff_gemm_f32tc.cu.
 cudaError_t f32tc_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S,
                            const EpiArgs& ep, int* err, cudaStream_t st);
