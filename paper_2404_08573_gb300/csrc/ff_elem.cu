@@ -52,6 +52,7 @@ __device__ __forceinline__ void store4<bf16>(bf16* p, float a, float b, float c,
 template <typename T>
 __global__ void k_overlay(const float* __restrict__ x, const int* __restrict__ labels, int rows, int F,
                           T* __restrict__ out, int ldo, float* __restrict__ s_out, int mode, int src_rows) {
+  ptx::griddep_wait();  // launched with programmatic stream serialization
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = blockIdx.x * 8 + warp;
   if (row >= rows) return;
@@ -88,6 +89,7 @@ __global__ void k_overlay(const float* __restrict__ x, const int* __restrict__ l
 
 template <typename T>
 __global__ void k_row_scale(const T* __restrict__ x, int ldx, int rows, int F, float* __restrict__ s_out) {
+  ptx::griddep_wait();  // launched with programmatic stream serialization
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = blockIdx.x * 8 + warp;
   if (row >= rows) return;
@@ -350,6 +352,7 @@ __global__ void k_to_bf16(const float* __restrict__ W, int N, int K, bf16* __res
 // ------------------------------------------------------------------ predict
 template <typename T>
 __global__ void k_label_columns(const T* __restrict__ W, int ldw, int N, float* __restrict__ cols, int ldc) {
+  ptx::griddep_wait();  // launched with programmatic stream serialization
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= ldc) return;
 #pragma unroll
@@ -368,6 +371,7 @@ __global__ void __launch_bounds__(256) k_expand(const float* __restrict__ base, 
                                                 const float* __restrict__ cols, const float* __restrict__ s1,
                                                 const float* __restrict__ bias, int N, T* __restrict__ H, int ldh,
                                                 float* __restrict__ s_next, float* __restrict__ G_acc, int* err) {
+  ptx::griddep_wait();  // launched with programmatic stream serialization
   __shared__ float red[8][10];
   const int n = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -423,6 +427,7 @@ __global__ void __launch_bounds__(256) k_expand(const float* __restrict__ base, 
 // its strongest wrong label; a label outside 0..9 leaves nothing out.
 __global__ void k_argmax(const float* __restrict__ G, int n, const int* __restrict__ labels,
                          int* __restrict__ pred) {
+  ptx::griddep_wait();  // launched with programmatic stream serialization
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float* g = G + (size_t)i * 10;
@@ -468,22 +473,17 @@ cudaError_t launch_overlay(const float* x, const int* labels, int rows, int F, v
                            float* s_out, int mode, cudaStream_t st, int src_rows) {
   if (rows <= 0) return cudaSuccess;
   if (src_rows <= 0 || src_rows > rows) src_rows = rows;
-  const int grid = cdiv(rows, 8);
+  PdlLaunch l(dim3(cdiv(rows, 8)), dim3(256), st);
   if (out_bf16)
-    k_overlay<bf16><<<grid, 256, 0, st>>>(x, labels, rows, F, (bf16*)out, ldo, s_out, mode, src_rows);
-  else
-    k_overlay<float><<<grid, 256, 0, st>>>(x, labels, rows, F, (float*)out, ldo, s_out, mode, src_rows);
-  return cudaGetLastError();
+    return cudaLaunchKernelEx(&l.cfg, k_overlay<bf16>, x, labels, rows, F, (bf16*)out, ldo, s_out, mode, src_rows);
+  return cudaLaunchKernelEx(&l.cfg, k_overlay<float>, x, labels, rows, F, (float*)out, ldo, s_out, mode, src_rows);
 }
 
 cudaError_t launch_row_scale(const void* x, int ldx, bool x_bf16, int rows, int F, float* s_out, cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
-  const int grid = cdiv(rows, 8);
-  if (x_bf16)
-    k_row_scale<bf16><<<grid, 256, 0, st>>>((const bf16*)x, ldx, rows, F, s_out);
-  else
-    k_row_scale<float><<<grid, 256, 0, st>>>((const float*)x, ldx, rows, F, s_out);
-  return cudaGetLastError();
+  PdlLaunch l(dim3(cdiv(rows, 8)), dim3(256), st);
+  if (x_bf16) return cudaLaunchKernelEx(&l.cfg, k_row_scale<bf16>, (const bf16*)x, ldx, rows, F, s_out);
+  return cudaLaunchKernelEx(&l.cfg, k_row_scale<float>, (const float*)x, ldx, rows, F, s_out);
 }
 
 int finalize_grid(int M) { return cdiv(M, 256); }
@@ -532,28 +532,26 @@ cudaError_t launch_to_bf16(const float* W, int N, int K, bf16* Wb, int ldb, cuda
 }
 
 cudaError_t launch_label_columns(const void* W, int ldw, bool w_bf16, int N, float* cols, int ldc, cudaStream_t st) {
-  if (w_bf16)
-    k_label_columns<bf16><<<cdiv(ldc, 256), 256, 0, st>>>((const bf16*)W, ldw, N, cols, ldc);
-  else
-    k_label_columns<float><<<cdiv(ldc, 256), 256, 0, st>>>((const float*)W, ldw, N, cols, ldc);
-  return cudaGetLastError();
+  PdlLaunch l(dim3(cdiv(ldc, 256)), dim3(256), st);
+  if (w_bf16) return cudaLaunchKernelEx(&l.cfg, k_label_columns<bf16>, (const bf16*)W, ldw, N, cols, ldc);
+  return cudaLaunchKernelEx(&l.cfg, k_label_columns<float>, (const float*)W, ldw, N, cols, ldc);
 }
 
 cudaError_t launch_expand(const float* base, int ldbase, const float* cols, const float* s1, const float* bias, int n,
                           int N, void* H, int ldh, bool h_bf16, float* s_next, float* G_acc, int* err,
                           cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
+  PdlLaunch l(dim3(n), dim3(256), st);
   if (h_bf16)
-    k_expand<bf16><<<n, 256, 0, st>>>(base, ldbase, cols, s1, bias, N, (bf16*)H, ldh, s_next, G_acc, err);
-  else
-    k_expand<float><<<n, 256, 0, st>>>(base, ldbase, cols, s1, bias, N, (float*)H, ldh, s_next, G_acc, err);
-  return cudaGetLastError();
+    return cudaLaunchKernelEx(&l.cfg, k_expand<bf16>, base, ldbase, cols, s1, bias, N, (bf16*)H, ldh, s_next, G_acc,
+                              err);
+  return cudaLaunchKernelEx(&l.cfg, k_expand<float>, base, ldbase, cols, s1, bias, N, (float*)H, ldh, s_next, G_acc, err);
 }
 
 cudaError_t launch_argmax(const float* G, int n, const int* labels, int* pred, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_argmax<<<cdiv(n, 256), 256, 0, st>>>(G, n, labels, pred);
-  return cudaGetLastError();
+  PdlLaunch l(dim3(cdiv(n, 256)), dim3(256), st);
+  return cudaLaunchKernelEx(&l.cfg, k_argmax, G, n, labels, pred);
 }
 
 cudaError_t launch_wait_selftest(int* err, unsigned long long timeout_ns, cudaStream_t st) {
