@@ -493,14 +493,16 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
   if (L0->K < 10) return FF_ERR_INVALID_ARG;
   const bool b16 = L0->is_bf16;
   const size_t es = b16 ? 2 : 4;
-  // fp32 layers: the GEMMs on the tensor cores (three TF32 products) where
-  // every layer's rows allow TMA, else on the CUDA cores
+  // fp32 layers: GEMMs that fill the GPU as three TF32 products where every
+  // layer's rows allow TMA (4600 x 2000 over 2000: 240 TFLOP/s of fp32 terms),
+  // the others as the training GEMMs run (800 x 2000 over 2000, a last chunk:
+  // 93 us before, 78 now; 460 x 2000 over 784: 44 and 23 us)
   bool f32tc = !b16;
   for (int k = 0; k < n_layers && f32tc; ++k) f32tc = tc_f32_supported(layers[k]->K, layers[k]->ldK, layers[k]->K);
   int ldmax = 0, ntmax = 0;
   for (int k = 0; k < n_layers; ++k) {
     if (layers[k]->ldN > ldmax) ldmax = layers[k]->ldN;
-    const int nt = b16 || f32tc ? tc_fwd_ntiles_max(layers[k]->N) : f32_fwd_ntiles_max(layers[k]->N);
+    const int nt = gpart_tiles_max(layers[k]->N);
     if (nt > ntmax) ntmax = nt;
   }
   // Samples per chunk: about 40 MB of activations per buffer, so that one
@@ -585,7 +587,7 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
                 tc_gemm_store(static_cast<const bf16*>(X0), L0->ldK, L0->Wb, L0->ldK, cn, N1, L0->K, base, L0->ldN,
                               err, st),
                 "layer-1 base GEMM (tcgen05)");
-    } else if (f32tc) {
+    } else if (f32tc && tc_full_shape(cn, N1)) {
       FF_LAUNCH(K_STORE_TC, 2.0 * cn * N1 * L0->K, st,
                 tc_gemm_store_f32(static_cast<const float*>(X0), L0->ldK, L0->W, L0->K, cn, N1, L0->K, base,
                                   L0->ldN, err, st),
@@ -593,7 +595,7 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
     } else {
       FF_LAUNCH(K_STORE_SIMT, 2.0 * cn * N1 * L0->K, st,
                 f32_gemm_store(static_cast<const float*>(X0), L0->ldK, L0->W, L0->K, cn, N1, L0->K, base, L0->ldN,
-                                st),
+                               err, st),
                 "layer-1 base GEMM (fp32)");
     }
     float* Gc = G + (size_t)c0 * 10;
@@ -623,7 +625,7 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
                   tc_gemm_fwd(static_cast<const bf16*>(Hb[cur]), Lk->ldK, Lk->Wb, Lk->ldK, rows, Lk->N, Lk->K, ep,
                               err, st),
                   "predict forward GEMM (tcgen05)");
-      } else if (f32tc) {
+      } else if (f32tc && tc_full_shape(rows, Lk->N)) {
         ep.narrow = false;
         nt = tc_fwd_ntiles(rows, Lk->N, false);
         FF_LAUNCH(K_FWD_TC, 2.0 * rows * Lk->N * Lk->K, st,

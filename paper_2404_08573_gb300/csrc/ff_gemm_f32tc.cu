@@ -301,6 +301,12 @@ cudaError_t f32tc_gemm_fwd(const float* A, int lda, const float* B, int ldb, int
   return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, S, ep, err, st);
 }
 
+cudaError_t f32tc_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, float* C,
+                             int ldc, int* err, cudaStream_t st) {
+  EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
+  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, S, ep, err, st);
+}
+
 cudaError_t f32tc_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, int S, float* C,
                              int ldc, int* err, cudaStream_t st) {
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};

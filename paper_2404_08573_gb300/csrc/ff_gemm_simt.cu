@@ -321,9 +321,12 @@ cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M
 }
 
 cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, float* C, int ldc,
-                           cudaStream_t st) {
+                           int* err, cudaStream_t st) {
+  const Plan p = plan_kmajor(M, N, K);
+  if (p.kind == TENSOR && aligned(A, lda) && aligned(B, ldb))
+    return f32tc_gemm_store(A, lda, B, ldb, M, N, K, p.S, C, ldc, err, st);
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, plan_of(M, N, K, false), ep, AdamArgs{}, st);
+  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, p, ep, AdamArgs{}, st);
 }
 
 // C[n, k] = sum_r G[r, n] X[r, k]: rows of C index G's columns (MN-major A),

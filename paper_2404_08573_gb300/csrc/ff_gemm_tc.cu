@@ -316,6 +316,8 @@ int tc_fwd_ntiles(int M, int N, bool narrow) {
 }
 int tc_fwd_ntiles_max(int N) { return cdiv(N, TINY_BN) * (EPI_WARPS / 4); }
 
+bool tc_full_shape(int M, int N) { return shape_of(M, N, FWD_BN) == SHAPE_FULL; }
+
 int tc_gemm_fwd_ctas(int M, int N, bool narrow) {
   switch (shape_of(M, N, FWD_BN)) {
     case SHAPE_FULL: return grid_ctas(M, N, ROW_SUBTILES, FWD_BN);
@@ -443,9 +445,8 @@ cudaError_t tc_gemm_wgrad(const bf16* G, int ldg, const bf16* X, int ldx, int R,
 
 // ------------------------------------------------ fp32 operands (3 x TF32)
 // Stages of fp32 tiles with their lo parts: 96 KB with two 128-row subtiles
-// per CTA (2 fit), 64 KB with one (3 fit).
+// per CTA (2 fit).
 constexpr int NSTAGES_F32 = 2;
-constexpr int NSTAGES_F32_SMALL = 3;
 
 bool tc_f32_supported(int K, int lda, int ldb) {
   // TMA rows of 16-byte multiples: fp32 row strides and K in multiples of 4
@@ -454,30 +455,25 @@ bool tc_f32_supported(int K, int lda, int ldb) {
 
 cudaError_t tc_gemm_fwd_f32(const float* A, int lda, const float* B, int ldb, int M, int N, int K, const EpiArgs& ep,
                             int* err, cudaStream_t st) {
-  if (!tc_f32_supported(K, lda, ldb) || ep.logit_V || ep.gpart_in || (ep.ldo & 3)) return cudaErrorInvalidValue;
+  if (!tc_f32_supported(K, lda, ldb) || !tc_full_shape(M, N) || ep.logit_V || ep.gpart_in || (ep.ldo & 3))
+    return cudaErrorInvalidValue;
   CUtensorMap ta, tb, tc;
   if (!make_map(&ta, A, 4, K, M, lda, 32, BM) || !make_map(&tb, B, 4, K, N, ldb, 32, b_box_rows(FWD_BN)) ||
       !make_map(&tc, ep.out, 4, ep.ldo, M, ep.ldo, 32, 32))
     return cudaErrorInvalidValue;
-  if (shape_of(M, N, FWD_BN) != SHAPE_FULL)
-    return launch_tc<FWD_BN, false, false, MODE_FWD, USE_PAIR, NSTAGES_F32_SMALL, 1, 1, 4>(ta, tb, tc, 1, M, N, K, ep,
-                                                                                          err, st);
   return launch_tc<FWD_BN, false, false, MODE_FWD, USE_PAIR, NSTAGES_F32, ROW_SUBTILES, 1, 4>(ta, tb, tc, 1, M, N, K,
                                                                                               ep, err, st);
 }
 
 cudaError_t tc_gemm_store_f32(const float* A, int lda, const float* B, int ldb, int M, int N, int K, float* Cm,
                               int ldc, int* err, cudaStream_t st) {
-  if (!tc_f32_supported(K, lda, ldb)) return cudaErrorInvalidValue;
+  if (!tc_f32_supported(K, lda, ldb) || !tc_full_shape(M, N)) return cudaErrorInvalidValue;
   CUtensorMap ta, tb, tc;
   if (!make_map(&ta, A, 4, K, M, lda, 32, BM) || !make_map(&tb, B, 4, K, N, ldb, 32, b_box_rows(FWD_BN)))
     return cudaErrorInvalidValue;
   const int tma = store_map(&tc, Cm, ldc, M, N) ? 1 : 0;
   if (!tma) tc = ta;  // unused
   EpiArgs ep{nullptr, nullptr, Cm, ldc, nullptr};
-  if (shape_of(M, N, FWD_BN) != SHAPE_FULL)
-    return launch_tc<FWD_BN, false, false, MODE_STORE, USE_PAIR, NSTAGES_F32_SMALL, 1, 1, 4>(ta, tb, tc, tma, M, N, K,
-                                                                                            ep, err, st);
   return launch_tc<FWD_BN, false, false, MODE_STORE, USE_PAIR, NSTAGES_F32, ROW_SUBTILES, 1, 4>(ta, tb, tc, tma, M, N,
                                                                                                 K, ep, err, st);
 }

@@ -304,7 +304,9 @@ cudaError_t tc_gemm_store(const bf16* A, int lda, const bf16* B, int ldb, int M,
 // The same forward (without gpart_in or block logits) and store GEMMs on fp32
 // operands, as three TF32 tensor-core products per term (Ah Bh + Ah Bl +
 // Al Bh; relative error near 2^-21 per product); H is written in fp32.  For K
-// and both row strides multiples of 4 (tc_f32_supported).
+// and both row strides multiples of 4 (tc_f32_supported) and outputs that
+// fill the GPU's tiles (tc_full_shape: at least 64 CTAs of two row subtiles).
+bool tc_full_shape(int M, int N);
 bool tc_f32_supported(int K, int lda, int ldb);
 cudaError_t tc_gemm_fwd_f32(const float* A, int lda, const float* B, int ldb, int M, int N, int K, const EpiArgs& ep,
                             int* err, cudaStream_t st);
@@ -343,12 +345,14 @@ int f32_fwd_ntiles_max(int N);
 cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
                          const EpiArgs& ep, int* err, cudaStream_t st);
 cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K,
-                           float* C, int ldc, cudaStream_t st);
+                           float* C, int ldc, int* err, cudaStream_t st);
 cudaError_t f32_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K,
                            float* C, int ldc, bool in_order, int* err, cudaStream_t st);
 // The tensor-core forms (S: slices of K), ff_gemm_f32tc.cu.
 cudaError_t f32tc_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S,
                            const EpiArgs& ep, int* err, cudaStream_t st);
+cudaError_t f32tc_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S,
+                             float* C, int ldc, int* err, cudaStream_t st);
 cudaError_t f32tc_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, int S,
                              float* C, int ldc, int* err, cudaStream_t st);
 // The weight gradient of a.N x a.K outputs over R rows and the Adam step it
