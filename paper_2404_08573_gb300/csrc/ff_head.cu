@@ -659,7 +659,7 @@ constexpr int kPoRows = 32;
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_po_grad(PoGradArgs a, const T* __restrict__ H, T* __restrict__ G) {
-  __shared__ float Vsh[kClasses][8][32];  // V[c][c0 + 8 l + e] at [c][e][l]: conflict-free reads
+  __shared__ __align__(16) float Vsh[kClasses][2][32][4];  // V[c][c0 + 8 l + 4 q + e] at [c][q][l][e]
   __shared__ float dzs[kPoRows][kClasses];
   // the block's activity tile in its own type (for the dV partials), then
   // the db reduction in the same memory
@@ -671,12 +671,13 @@ __global__ void __launch_bounds__(256) k_po_grad(PoGradArgs a, const T* __restri
   const int cg = c0 + lane * 8;
   const bool cols_ok = cg < a.ld;
   ptx::griddep_wait();  // launched with programmatic stream serialization
-  // this thread's activity (rows y, y+8, y+16, y+24; 8 columns), loaded first
-  // so that its latency overlaps the logits and softmax below
-  float hv[4][8];
+  // this thread's activity (rows y, y+8, y+16, y+24; 8 columns) and its rows'
+  // scales, loaded first so that their latency overlaps the logits and softmax
+  float hv[4][8], sr[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int i = r0 + threadIdx.y + 8 * k;
+    sr[k] = i < a.n ? __ldg(a.s + i) : 0.f;
     if (cols_ok && i < a.n) {
       Vec8<T>::load(H + (size_t)i * a.ld + cg, hv[k]);
     } else {
@@ -686,15 +687,35 @@ __global__ void __launch_bounds__(256) k_po_grad(PoGradArgs a, const T* __restri
   }
   for (int idx = tid; idx < kClasses * 256; idx += 256) {
     const int c = idx / 256, j = idx % 256;
-    Vsh[c][j % 8][j / 8] = (c0 + j < a.N) ? __ldg(a.V + (size_t)c * a.N + c0 + j) : 0.f;
+    Vsh[c][(j >> 2) & 1][j >> 3][j & 3] = (c0 + j < a.N) ? __ldg(a.V + (size_t)c * a.N + c0 + j) : 0.f;
   }
   if (a.zpart) {
-    // logits of the block's rows: thread per (row, class), partials in tile order
-    for (int idx = tid; idx < kPoRows * kClasses; idx += 256) {
-      const int i = idx / kClasses, c = idx % kClasses;
-      dzs[i][c] = r0 + i < a.n ? __ldg(a.cb + c) + sum_partials(a.zpart, a.zt, a.n * kClasses, (r0 + i) * kClasses + c)
-                               : 0.f;
+    // logits of the block's rows: thread per (row, class), partials in tile
+    // order, both of a thread's sums and 8 partials each in flight together
+    constexpr int NI = (kPoRows * kClasses + 255) / 256;
+    const int items = min(kPoRows, a.n - r0) * kClasses;
+    const float* zp = a.zpart + (size_t)r0 * kClasses + tid;
+    const size_t stride = (size_t)a.n * kClasses;
+    float z[NI] = {};
+    for (int t0 = 0; t0 < a.zt; t0 += 8) {
+      float v[NI][8];
+#pragma unroll
+      for (int i = 0; i < NI; ++i)
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          v[i][u] = t0 + u < a.zt && tid + 256 * i < items ? __ldg(zp + 256 * i + (t0 + u) * stride) : 0.f;
+#pragma unroll
+      for (int i = 0; i < NI; ++i)
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (t0 + u < a.zt) z[i] += v[i][u];
     }
+    const int y = threadIdx.y == 0 && r0 + lane < a.n ? __ldg(a.labels + r0 + lane) : 0;
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+      if (tid + 256 * i < kPoRows * kClasses)
+        (&dzs[0][0])[tid + 256 * i] =
+            tid + 256 * i < items ? __ldg(a.cb + (tid + 256 * i) % kClasses) + z[i] : 0.f;
     __syncthreads();
     if (threadIdx.y == 0) {
       // warp 0: softmax, loss and dz of row r0 + lane, in place
@@ -703,7 +724,7 @@ __global__ void __launch_bounds__(256) k_po_grad(PoGradArgs a, const T* __restri
       for (int c = 0; c < kClasses; ++c) z[c] = dzs[lane][c];
       float loss = 0.f;
       if (r0 + lane < a.n) {
-        loss = finish_row(z, r0 + lane, true, __ldg(a.labels + r0 + lane), a.inv_n, nullptr, nullptr, dzr, &a.hds->err);
+        loss = finish_row(z, r0 + lane, true, y, a.inv_n, nullptr, nullptr, dzr, &a.hds->err);
       } else {
 #pragma unroll
         for (int c = 0; c < kClasses; ++c) dzr[c] = 0.f;
@@ -737,15 +758,16 @@ __global__ void __launch_bounds__(256) k_po_grad(PoGradArgs a, const T* __restri
       dzs[i][c] = (r0 + i < a.n) ? __ldg(a.dz + (size_t)(r0 + i) * kClasses + c) : 0.f;
     }
   }
-  if (blockIdx.x == 0 && tid < kPoRows && r0 + tid < a.n) {
-    const float g = sum_partials(a.gpart, a.ntiles, a.n, r0 + tid);
+  // beside warp 0's softmax: warp 1 the next layer's scales, warp 2 the step
+  if (blockIdx.x == 0 && threadIdx.y == 1 && r0 + lane < a.n) {
+    const float g = sum_partials(a.gpart, a.ntiles, a.n, r0 + lane);
     if (!isfinite(g)) atomicOr(a.err, DEVERR_NONFINITE);
     if (a.s_next) {
       const float r = sqrtf(g);
-      a.s_next[r0 + tid] = r != r ? r : 1.f / fmaxf(r, 1e-12f);
+      a.s_next[r0 + lane] = r != r ? r : 1.f / fmaxf(r, 1e-12f);
     }
   }
-  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 64) {
     a.ds->t += 1;
     a.ds->pow1 *= a.beta1;
     a.ds->pow2 *= a.beta2;
@@ -753,6 +775,26 @@ __global__ void __launch_bounds__(256) k_po_grad(PoGradArgs a, const T* __restri
     a.ds->bc2 = (float)(1.0 - a.ds->pow2);
   }
   __syncthreads();
+  // d_ke = sum over the classes in order: a class's 8 weights are read once
+  // for the thread's 4 rows (with a row's classes innermost the kernel was
+  // bound by its 640 shared-memory reads a thread; now 60)
+  float d[4][8];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int e = 0; e < 8; ++e) d[k][e] = 0.f;
+#pragma unroll
+  for (int c = 0; c < kClasses; ++c) {
+    const float4 v0 = *reinterpret_cast<const float4*>(Vsh[c][0][lane]);
+    const float4 v1 = *reinterpret_cast<const float4*>(Vsh[c][1][lane]);
+    const float v[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float z = dzs[threadIdx.y + 8 * k][c];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) d[k][e] = fmaf(z, v[e], d[k][e]);
+    }
+  }
   float db[8];
 #pragma unroll
   for (int e = 0; e < 8; ++e) db[e] = 0.f;
@@ -760,40 +802,52 @@ __global__ void __launch_bounds__(256) k_po_grad(PoGradArgs a, const T* __restri
   for (int k = 0; k < 4; ++k) {
     const int li = threadIdx.y + 8 * k;
     const int i = r0 + li;
-    const float(&h)[8] = hv[k];
-    float z[8];
-    Vec8<T>::store(&Hs[li][lane * 8], h);
+    Vec8<T>::store(&Hs[li][lane * 8], hv[k]);
     if (!cols_ok || i >= a.n) continue;
-    const float si = __ldg(a.s + i);
+    float z[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      float d = 0.f;
-#pragma unroll
-      for (int c = 0; c < kClasses; ++c) d = fmaf(dzs[li][c], Vsh[c][e][lane], d);
-      d = h[e] > 0.f ? d : 0.f;
-      db[e] += d;
-      z[e] = si * d;
+      const float t = hv[k][e] > 0.f ? d[k][e] : 0.f;
+      db[e] += t;
+      z[e] = sr[k] * t;
     }
     Vec8<T>::store(G + (size_t)i * a.ld + cg, z);
   }
   __syncthreads();
-  // dV partials from the staged tile: thread (x, y) sums classes y and
-  // y + 8 (when below 10) over the block's 32 rows in order, for its 8 columns
-#pragma unroll
-  for (int c = threadIdx.y; c < kClasses; c += 8) {
-    float dv[8];
+  // dV partials from the staged tile, each the block's 32 rows in order:
+  // thread (x, y) sums class y over its 8 columns and, of classes 8 and 9, two
+  // columns (64 (y % 4) + 2 x, + 1 of class 8 + y / 4)
+  {
+    const int y = threadIdx.y, c2 = 8 + (y >> 2), j2 = 64 * (y & 3) + 2 * lane;
+    float dv[8], dw[2] = {0.f, 0.f};
 #pragma unroll
     for (int e = 0; e < 8; ++e) dv[e] = 0.f;
+#pragma unroll 4
     for (int li = 0; li < kPoRows; ++li) {
-      const float d = dzs[li][c];
+      const float d = dzs[li][y], d2 = dzs[li][c2];
       float h[8];
       Vec8<T>::load(&Hs[li][lane * 8], h);
+      float h0, h1;
+      if constexpr (sizeof(T) == 2) {
+        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&Hs[li][j2]));
+        h0 = f.x;
+        h1 = f.y;
+      } else {
+        h0 = Hs[li][j2];
+        h1 = Hs[li][j2 + 1];
+      }
 #pragma unroll
       for (int e = 0; e < 8; ++e) dv[e] = fmaf(d, h[e], dv[e]);
+      dw[0] = fmaf(d2, h0, dw[0]);
+      dw[1] = fmaf(d2, h1, dw[1]);
     }
+    float* out = a.dVpart + (size_t)blockIdx.y * kClasses * a.N;
 #pragma unroll
     for (int e = 0; e < 8; ++e)
-      if (cg + e < a.N) a.dVpart[((size_t)blockIdx.y * kClasses + c) * a.N + cg + e] = dv[e];
+      if (cg + e < a.N) out[(size_t)y * a.N + cg + e] = dv[e];
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      if (c0 + j2 + e < a.N) out[(size_t)c2 * a.N + c0 + j2 + e] = dw[e];
   }
   __syncthreads();
   // db partials: the eight row groups added in order, through the tile's memory
