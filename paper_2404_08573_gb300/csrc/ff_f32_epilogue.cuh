@@ -25,14 +25,16 @@ __device__ __forceinline__ float4 ld_cluster4(const float* local, uint32_t rank)
   return v;
 }
 
-// By threads 0 .. 255 (tid) of a CTA, after its own and its cluster's partials
+// The slices' CTAs have cluster ranks rank0 + rank_step * slice (slice:
+// blockIdx.z).  By threads 0 .. 255 (tid) of a CTA, after its own and its cluster's partials
 // are in place (and before any CTA of the cluster leaves):
 //   MODE_FWD    H = ReLU(s_r z + b), goodness partials per row and T columns
 //   MODE_STORE  C = z
 //   MODE_ADAM   z is the gradient of the weights W[gi, col]: Adam on them
 template <int T, int MODE>
 __device__ __forceinline__ void f32_tile_epilogue(const float* sm, int tid, int M, int N, int m0, int n0, int S,
-                                                  const EpiArgs& ep, const AdamArgs& ad) {
+                                                  const EpiArgs& ep, const AdamArgs& ad, uint32_t rank0 = 0,
+                                                  uint32_t rank_step = 1) {
   constexpr int LD = f32_tile_ld(T);
   constexpr int LPR = T / 4;     // lanes per row, 4 columns each
   constexpr int RPP = NT / LPR;  // rows per pass
@@ -46,7 +48,7 @@ __device__ __forceinline__ void f32_tile_epilogue(const float* sm, int tid, int 
       float4 u[kMaxSplit];
 #pragma unroll
       for (int z = 0; z < kMaxSplit; ++z)
-        if (z < S) u[z] = ld_cluster4(sm + r * LD + lc, (uint32_t)z);
+        if (z < S) u[z] = ld_cluster4(sm + r * LD + lc, rank0 + rank_step * (uint32_t)z);
       v[0] = v[1] = v[2] = v[3] = 0.f;
 #pragma unroll
       for (int z = 0; z < kMaxSplit; ++z)
@@ -149,7 +151,7 @@ __device__ __forceinline__ void f32_tile_epilogue(const float* sm, int tid, int 
         for (int o = LPR / 4; o > 0; o >>= 1) g[q] += __shfl_xor_sync(0xffffffffu, g[q], o);
         const int o = p + q * RPP + lr;
         const int gi = m0 + (int)blockIdx.z * RS + o;
-        if (lc == T / 2 && o < RS && gi < M) ep.gpart[(size_t)blockIdx.y * M + gi] = g[q];
+        if (lc == T / 2 && o < RS && gi < M) ep.gpart[(size_t)(n0 / T) * M + gi] = g[q];
       }
     }
   } else {

@@ -66,25 +66,28 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t (&p)[3]) {
   p[2] = cvt2(x0, x1);
 }
 
-// A loader thread's share of one operand's 128 x 64 fp32 tile: 8 words of 4
-// values.  Tile row i of 128 holds 64 values contiguous in memory: K-major
-// operands, row r0 + i, K k0 ..; MN-major ones, K k0 + i % 64, rows r0 + 64
-// (i / 64) ...  16 lanes take a row, a warp two rows at a time.
-template <bool MN>
-__device__ __forceinline__ void load8(float4 (&v)[8], const float* __restrict__ P, int ld, int rows, int K, int r0,
-                                      int k0, int t) {
+// One of 16 RPP loader threads' share of one operand's 128 x 64 fp32 tile:
+// NV = 128 / RPP words of 4 values, RPP tile rows at a time.  Tile row i of 128
+// holds 64 values contiguous in memory: K-major operands, row r0 + i, K k0 ..;
+// MN-major ones, K k0 + i % 64, rows r0 + 64 (i / 64) ...  16 lanes take a row,
+// a warp two rows at a time.
+template <bool MN, int NV>
+__device__ __forceinline__ void load_part(float4 (&v)[NV], const float* __restrict__ P, int ld, int rows, int K, int r0,
+                                          int k0, int t) {
+  constexpr int RPP = T / NV;
   const int c = 4 * (t & 15), r = t >> 4;
   if (r0 + T <= rows && k0 + KC <= K) {  // the whole tile exists
     const float* p = MN ? P + (size_t)(k0 + r) * ld + r0 + c : P + (size_t)(r0 + r) * ld + k0 + c;
-    const size_t step = (size_t)16 * ld;
+    const size_t step = (size_t)RPP * ld;
+    constexpr int H = 64 / RPP;  // words per 64-row half of an MN-major tile
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      v[i] = __ldg(reinterpret_cast<const float4*>(MN ? p + (i & 3) * step + (i >> 2) * 64 : p + i * step));
+    for (int i = 0; i < NV; ++i)
+      v[i] = __ldg(reinterpret_cast<const float4*>(MN ? p + (i % H) * step + (i / H) * 64 : p + i * step));
     return;
   }
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int row = r + 16 * i;
+  for (int i = 0; i < NV; ++i) {
+    const int row = r + RPP * i;
     const int slow = MN ? k0 + (row & 63) : r0 + row;
     const int fast = MN ? r0 + (row >> 6) * 64 + c : k0 + c;
     const bool ok = slow < (MN ? K : rows) && fast < (MN ? rows : K);
@@ -98,22 +101,47 @@ __device__ __forceinline__ void load8(float4 (&v)[8], const float* __restrict__ 
 }
 // Its three parts into the operand's tiles (128-byte rows, 16-byte words
 // permuted by the row's low three bits, the same for all of a thread's rows).
-__device__ __forceinline__ void store8(uint8_t* op, const float4 (&v)[8], int t) {
+template <int NV>
+__device__ __forceinline__ void store_part(uint8_t* op, const float4 (&v)[NV], int t) {
+  constexpr int RPP = T / NV;
   const int c = t & 15, r = t >> 4;
   uint8_t* dst = op + r * 128 + (((c >> 1) ^ (r & 7)) << 4) + (c & 1) * 8;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < NV; ++i) {
     uint32_t a[3], b[3];
     split2(v[i].x, v[i].y, a);
     split2(v[i].z, v[i].w, b);
 #pragma unroll
-    for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(dst + i * 16 * 128 + p * PART_BYTES) = make_uint2(a[p], b[p]);
+    for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(dst + i * RPP * 128 + p * PART_BYTES) = make_uint2(a[p], b[p]);
   }
 }
 
 __device__ __forceinline__ void latch(int* err, volatile int* abort_flag) {
   *abort_flag = 1;
   atomicOr(err, DEVERR_TIMEOUT);
+}
+
+// The MMAs of one chunk (a stage's parts) into the accumulator at acc: the six
+// part products, the smallest first.  PAIR: M = N = 256 over the CTA pair.
+template <bool MN, bool PAIR>
+__device__ __forceinline__ void issue_chunk(uint32_t acc, const uint8_t* stage) {
+  constexpr uint32_t idesc = ptx::idesc_bf16_f32(PAIR ? 2 * T : T, PAIR ? 2 * T : T, MN ? 1 : 0, MN ? 1 : 0);
+  constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+  const uint32_t ab = ptx::smem_u32(stage), bb = ab + OP_BYTES;
+#pragma unroll
+  for (int p = 0; p < 6; ++p)
+#pragma unroll
+    for (int k = 0; k < KC / 16; ++k) {
+      // K-major: 32 bytes along the swizzled rows, 8-row groups 1024 bytes
+      // apart; MN-major: 16 K rows further, the 64-element halves 64 rows apart
+      const uint32_t aa = ab + pa[p] * PART_BYTES, ba = bb + pb[p] * PART_BYTES;
+      const uint64_t ad = MN ? ptx::sdesc_sw128(aa + k * 2048, 64 * 128, 1024) : ptx::sdesc_sw128(aa + k * 32, 16, 1024);
+      const uint64_t bd = MN ? ptx::sdesc_sw128(ba + k * 2048, 64 * 128, 1024) : ptx::sdesc_sw128(ba + k * 32, 16, 1024);
+      if constexpr (PAIR)
+        ptx::umma_f16_pair(acc, ad, bd, idesc, (p | k) != 0 ? 1u : 0u);
+      else
+        ptx::umma_f16(acc, ad, bd, idesc, (p | k) != 0 ? 1u : 0u);
+    }
 }
 
 template <bool MN, int MODE>
@@ -161,8 +189,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int t = threadIdx.x;
     float4 va[8], vb[8];
     if (nc > 0) {
-      load8<MN>(va, A, lda, M, K, m0, c0 * KC, t);
-      load8<MN>(vb, B, ldb, N, K, n0, c0 * KC, t);
+      load_part<MN>(va, A, lda, M, K, m0, c0 * KC, t);
+      load_part<MN>(vb, B, ldb, N, K, n0, c0 * KC, t);
     }
     for (int c = 0; c < nc; ++c) {
       const int s = c % STAGES;
@@ -170,10 +198,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       if (!ok) latch(err, abort_flag);
       if (!__all_sync(0xffffffffu, ok && !*abort_flag)) break;
       uint8_t* op = smem + s * STAGE_BYTES;
-      store8(op, va, t);
-      if (c + 1 < nc) load8<MN>(va, A, lda, M, K, m0, (c0 + c + 1) * KC, t);
-      store8(op + OP_BYTES, vb, t);
-      if (c + 1 < nc) load8<MN>(vb, B, ldb, N, K, n0, (c0 + c + 1) * KC, t);
+      store_part(op, va, t);
+      if (c + 1 < nc) load_part<MN>(va, A, lda, M, K, m0, (c0 + c + 1) * KC, t);
+      store_part(op + OP_BYTES, vb, t);
+      if (c + 1 < nc) load_part<MN>(vb, B, ldb, N, K, n0, (c0 + c + 1) * KC, t);
       ptx::fence_async_smem();  // read by the MMAs (async proxy)
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&full[s]);
@@ -189,28 +217,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     // chunk c's MMAs are issued before chunk c - 1 is added
     for (int c = 0; c <= nc; ++c) {
       if (issuer && c < nc) {
-        constexpr uint32_t idesc = ptx::idesc_bf16_f32(T, T, MN ? 1 : 0, MN ? 1 : 0);
-        // (A part, B part), the smallest products first
-        constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
         const int s = c % STAGES, b = c % BUFS;
         if (ptx::mbar_wait(&full[s], (uint32_t)(c / STAGES) & 1u, kWaitTimeoutNs, abort_flag) &&
             ptx::mbar_wait(&tempty[b], ((uint32_t)(c / BUFS) & 1u) ^ 1u, kWaitTimeoutNs, abort_flag)) {
           ptx::tc_fence_after();
-          const uint32_t ab = ptx::smem_u32(smem + s * STAGE_BYTES), bb = ab + OP_BYTES;
-#pragma unroll
-          for (int p = 0; p < 6; ++p)
-#pragma unroll
-            for (int k = 0; k < KC / 16; ++k) {
-              // K-major: 32 bytes along the swizzled rows, 8-row groups 1024
-              // bytes apart; MN-major: 16 K rows further, the 64-element
-              // halves 64 rows apart
-              const uint32_t aa = ab + pa[p] * PART_BYTES, ba = bb + pb[p] * PART_BYTES;
-              const uint64_t ad =
-                  MN ? ptx::sdesc_sw128(aa + k * 2048, 64 * 128, 1024) : ptx::sdesc_sw128(aa + k * 32, 16, 1024);
-              const uint64_t bd =
-                  MN ? ptx::sdesc_sw128(ba + k * 2048, 64 * 128, 1024) : ptx::sdesc_sw128(ba + k * 32, 16, 1024);
-              ptx::umma_f16(tmem + (uint32_t)(b * T), ad, bd, idesc, (p | k) != 0 ? 1u : 0u);
-            }
+          issue_chunk<MN, false>(tmem + (uint32_t)(b * T), smem + s * STAGE_BYTES);
           ptx::umma_commit(&empty[s]);
           ptx::umma_commit(&tfull[b]);
         } else {
@@ -271,14 +282,156 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   if (S > 1) ptx::cluster_sync();  // no CTA leaves while another reads its partial tile
 }
 
+// The same by CTA pairs (cta_group::2), for outputs of more than 128 rows and
+// columns: a pair makes a 256 x 256 tile, each CTA its 128 rows, splitting
+// 128 x 64 of A and of B per chunk as above -- half the splitting, half the
+// shared-memory reads and writes per output.  All 16 warps do the same: write
+// chunk c's parts, (one lane of the even CTA issues its MMAs once both CTAs
+// have written,) add chunk c - 1 from TMEM to their registers (a 32-row quarter
+// and 64 columns each), load chunk c + 1.  Measured 2.7 us a chunk (its 24
+// MMAs of M = N = 256 take 3072 clocks; the rest is the chain of barriers,
+// loads and splitting between them): 165 to 188 TFLOP/s of fp32 terms on 2048
+// to 4600 rows of a 2000-wide layer, where 128 x 128 tiles reach 126 to 147.
 template <bool MN, int MODE>
-cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, const EpiArgs& ep,
-                   int* err, cudaStream_t st) {
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(k_f32tc_gemm<MN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+__global__ void __launch_bounds__(NTHREADS, 1)
+    k_f32tc_pair(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb, int M, int N, int K,
+                 EpiArgs ep, int* err) {
+  static_assert(2 * T * LD * 4 <= STAGES * STAGE_BYTES, "both halves of the partial tile take the ring's place");
+  constexpr int WARPS = NTHREADS / 32;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = ptx::smem_u32(smem_raw);
+  uint8_t* smem = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);  // both CTAs have written the stage
+  uint64_t* done = full + STAGES;                                             // the stage's MMAs have finished
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + STAGES);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = ptx::cluster_ctarank(), lead = rank & ~1u;
+  const bool leader = rank == lead;
+  const int m0 = blockIdx.x * T;
+  const int n0 = blockIdx.y * 2 * T;
+  const int nb = n0 + (int)(rank & 1u) * T;  // the columns whose B this CTA supplies
+  const int S = gridDim.z;
+  const int chunks = (K + KC - 1) / KC;
+  const int per = (chunks + S - 1) / S;
+  const int c0 = min(chunks, (int)blockIdx.z * per), nc = min(chunks, c0 + per) - c0;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      ptx::mbar_init(&full[s], 2 * WARPS);
+      ptx::mbar_init(&done[s], 1);
+    }
+    *abort_flag = 0;
+    ptx::fence_mbar_init();
+  }
+  if (warp == 1) {
+    ptx::tmem_alloc_pair(tslot, STAGES * 2 * T);
+    ptx::tmem_relinquish_pair();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::cluster_sync();  // every CTA's barriers and TMEM exist before any cross-CTA use
+  ptx::tc_fence_after();
+  const uint32_t tmem = *tslot;
+  ptx::griddep_wait();  // launched with programmatic stream serialization
+
+  const int q = warp & 3, cg = warp >> 2;
+  float acc[64];
+#pragma unroll
+  for (int j = 0; j < 64; ++j) acc[j] = 0.f;
+  float4 va[4], vb[4];
+  if (nc > 0) {
+    load_part<MN>(va, A, lda, M, K, m0, c0 * KC, threadIdx.x);
+    load_part<MN>(vb, B, ldb, N, K, nb, c0 * KC, threadIdx.x);
+  }
+  bool good = true;
+  for (int c = 0; c <= nc; ++c) {
+    const int s = c % STAGES;
+    if (c < nc) {
+      // stage s and its TMEM buffer are free: this warp added chunk c - STAGES,
+      // whose MMAs had then finished, and the MMAs wait for every warp
+      uint8_t* op = smem + s * STAGE_BYTES;
+      store_part(op, va, threadIdx.x);
+      store_part(op + OP_BYTES, vb, threadIdx.x);
+      ptx::fence_async_smem();  // read by the MMAs (async proxy)
+      ptx::tc_fence_before();   // this warp's TMEM reads come before the buffer's next MMAs
+      __syncwarp();
+      if (lane == 0) {
+        if (leader)
+          ptx::mbar_arrive(&full[s]);
+        else
+          ptx::mbar_arrive_remote(&full[s], lead);
+      }
+      if (leader && threadIdx.x == 0) {
+        if (ptx::mbar_wait_cluster(&full[s], (uint32_t)(c / STAGES) & 1u, kWaitTimeoutNs, abort_flag)) {
+          ptx::tc_fence_after();
+          issue_chunk<MN, true>(tmem + (uint32_t)(s * 2 * T), op);
+          ptx::umma_commit_pair(&done[s], (uint16_t)(3u << lead));
+        } else {
+          latch(err, abort_flag);
+        }
+      }
+      __syncwarp();
+    }
+    if (c > 0) {
+      const int sp = (c - 1) % STAGES;
+      const bool ok = ptx::mbar_wait(&done[sp], (uint32_t)((c - 1) / STAGES) & 1u, kWaitTimeoutNs, abort_flag);
+      if (!ok) latch(err, abort_flag);
+      good = __all_sync(0xffffffffu, ok && !*abort_flag);
+      if (!good) break;
+      ptx::tc_fence_after();
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t r[32];
+        ptx::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(sp * 2 * T + cg * 64 + h * 32), r);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[32 * h + j] = __fadd_rn(acc[32 * h + j], __uint_as_float(r[j]));
+      }
+    }
+    if (c + 1 < nc) {
+      load_part<MN>(va, A, lda, M, K, m0, (c0 + c + 1) * KC, threadIdx.x);
+      load_part<MN>(vb, B, ldb, N, K, nb, (c0 + c + 1) * KC, threadIdx.x);
+    }
+  }
+  if (!good) {
+    // MMAs already issued finish before shared memory and TMEM are released
+    const uint64_t t0 = ptx::globaltimer();
+    while (ptx::globaltimer() - t0 < 1000000ull) {
+    }
+  }
+  // every warp has seen the last chunk's MMAs finish, so nothing reads the
+  // ring any more: the partial tile takes its place, as two 128-column halves
+  __syncthreads();
+  if (good) {
+    float* row = reinterpret_cast<float*>(smem) + ((cg >> 1) * T + q * 32 + lane) * LD + (cg & 1) * 64;
+#pragma unroll
+    for (int j = 0; j < 64; j += 4)
+      *reinterpret_cast<float4*>(row + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+  }
+  if (threadIdx.x == 0) ptx::griddep_launch_dependents();
+  ptx::tc_fence_before();
+  ptx::cluster_sync();  // every partial of the tile is in place; the pair is done with TMEM
+  ptx::tc_fence_after();
+  if (warp == 1) ptx::tmem_dealloc_pair(tmem, STAGES * 2 * T);
+  const int half = threadIdx.x / NT;
+  if (!*abort_flag && n0 + half * T < N)
+    f32_tile_epilogue<T, MODE>(reinterpret_cast<const float*>(smem) + half * T * LD, threadIdx.x % NT, M, N, m0,
+                               n0 + half * T, S, ep, AdamArgs{}, rank & 1u, 2u);
+  ptx::cluster_sync();  // no CTA leaves while another reads its partial tile
+}
+
+template <bool MN, int MODE>
+cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, bool pair,
+                   const EpiArgs& ep, int* err, cudaStream_t st) {
+  static const cudaError_t attr = [] {
+    cudaError_t e = cudaFuncSetAttribute(k_f32tc_gemm<MN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_f32tc_pair<MN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    return e;
+  }();
   if (attr != cudaSuccess) return attr;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cdiv(M, T), cdiv(N, T), S);
+  cfg.gridDim = pair ? dim3(2 * cdiv(M, 2 * T), cdiv(N, 2 * T), S) : dim3(cdiv(M, T), cdiv(N, T), S);
   cfg.blockDim = dim3(NTHREADS);
   cfg.dynamicSmemBytes = SMEM;
   cfg.stream = st;
@@ -286,31 +439,32 @@ cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int 
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   at[1].id = cudaLaunchAttributeClusterDimension;
-  at[1].val.clusterDim.x = 1;
+  at[1].val.clusterDim.x = pair ? 2 : 1;
   at[1].val.clusterDim.y = 1;
   at[1].val.clusterDim.z = S;
   cfg.attrs = at;
-  cfg.numAttrs = S > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, k_f32tc_gemm<MN, MODE>, A, lda, B, ldb, M, N, K, ep, err);
+  cfg.numAttrs = pair || S > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, pair ? k_f32tc_pair<MN, MODE> : k_f32tc_gemm<MN, MODE>, A, lda, B, ldb, M, N, K, ep,
+                            err);
 }
 
 }  // namespace
 
-cudaError_t f32tc_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S,
+cudaError_t f32tc_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, bool pair,
                            const EpiArgs& ep, int* err, cudaStream_t st) {
-  return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, S, ep, err, st);
+  return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, S, pair, ep, err, st);
 }
 
-cudaError_t f32tc_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, float* C,
-                             int ldc, int* err, cudaStream_t st) {
+cudaError_t f32tc_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, bool pair,
+                             float* C, int ldc, int* err, cudaStream_t st) {
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, S, ep, err, st);
+  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, S, pair, ep, err, st);
 }
 
-cudaError_t f32tc_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, int S, float* C,
-                             int ldc, int* err, cudaStream_t st) {
+cudaError_t f32tc_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, int S, bool pair,
+                             float* C, int ldc, int* err, cudaStream_t st) {
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, S, ep, err, st);
+  return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, S, pair, ep, err, st);
 }
 
 }  // namespace ff

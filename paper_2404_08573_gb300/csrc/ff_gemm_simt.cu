@@ -224,21 +224,23 @@ __global__ void __launch_bounds__(NT, 2)
 
 // How an M x N output over K is computed: on the CUDA cores in 64 x 64 or
 // 128 x 128 tiles, or on the tensor cores (ff_gemm_f32tc.cu) in 128 x 128
-// tiles, and in how many K slices: the least modelled time.  Measured: a CTA
+// tiles or, by CTA pairs, 256 x 256 ones, and in how many K slices: the least
+// modelled time.  Measured: a CTA
 // takes 0.95 us per 32-deep stage of a 64 x 64 tile and 3.3 us of a 128 x 128
 // one (42 and 48 TFLOP/s over 152 SMs) whether or not it shares its SM -- the
 // shared-memory operand reads and the FMAs fill the SM's time -- and 1.7 us
-// per 64-deep chunk of a tensor-core tile, an SM to itself, with about 9 us
-// before and after its mainloop against 5.  A GEMM takes the stages that the
+// per 64-deep chunk of a tensor-core tile, an SM to itself (a pair's, of four
+// times the output, 2.7 us), with about 9 us before and after its mainloop
+// against 5.  A GEMM takes the stages that the
 // fullest SM runs; a split costs about 1 us more.  Eight slices measured no
 // faster than four at any size (clusters of 8 find fewer places).
 // Rows x K -> N, us: one 128 x 128 tile per CTA and partial tiles through
-// device memory (as before) / CUDA cores / tensor cores:
-//   128 x 784 -> 500    22 / 15 / 20      (CUDA cores chosen)
-//   128 x 2000 -> 2000  -- / 39 / 27      (tensor cores from here on)
-//   512 x 2000 -> 2000  122 / 113 / 44    weight gradient 118 / 94 / 41
-//   2048 x 2000 -> 2000 480 / 367 / 139   weight gradient 416 / 322 / 120
-enum Kind { TILE_64, TILE_128, TENSOR };
+// device memory (as before) / CUDA cores / tensor cores / by pairs:
+//   128 x 784 -> 500    22 / 15 / 20 / --     (CUDA cores chosen)
+//   128 x 2000 -> 2000  -- / 39 / 27 / 35     (tensor cores from here on)
+//   512 x 2000 -> 2000  122 / 113 / 43 / 57   weight gradient 118 / 94 / 42 / 33
+//   2048 x 2000 -> 2000 480 / 367 / 130 / 99  weight gradient 416 / 322 / 121 / 97
+enum Kind { TILE_64, TILE_128, TENSOR, TENSOR_PAIR };
 struct Plan {
   Kind kind;
   int S;
@@ -246,15 +248,16 @@ struct Plan {
 Plan plan_of(int M, int N, int K, bool tensor) {
   Plan best{TILE_128, 1};
   double bt = 0.0;
-  for (int kind = tensor ? TENSOR : TILE_128; kind >= TILE_64; --kind) {
-    const int T = kind == TILE_64 ? 64 : 128;
-    const int steps = cdiv(K, kind == TENSOR ? 64 : TKS);
+  for (int kind = tensor ? TENSOR_PAIR : TILE_128; kind >= TILE_64; --kind) {
+    const int T = kind == TILE_64 ? 64 : kind == TENSOR_PAIR ? 256 : 128;
+    const int steps = cdiv(K, kind >= TENSOR ? 64 : TKS);
     const double tiles = (double)cdiv(M, T) * cdiv(N, T);
     for (int S = 1; S <= kMaxSplit; S *= 2) {
       if (S > 1 && steps < 2 * S) break;
-      const double per_sm = cdiv((long long)(tiles * S), 152);  // CTAs an SM runs in all
-      const double step = kind == TILE_64 ? 0.95 : kind == TILE_128 ? 3.3 : 1.7;
-      const double t = (kind == TENSOR ? per_sm * (cdiv(steps, S) * step + 9.0) : per_sm * cdiv(steps, S) * step + 5.0) +
+      // CTAs (pairs) an SM (two SMs) runs in all
+      const double per_sm = cdiv((long long)(tiles * S), kind == TENSOR_PAIR ? 76 : 152);
+      const double step = kind == TILE_64 ? 0.95 : kind == TILE_128 ? 3.3 : kind == TENSOR ? 1.7 : 2.7;
+      const double t = (kind >= TENSOR ? per_sm * (cdiv(steps, S) * step + 9.0) : per_sm * cdiv(steps, S) * step + 5.0) +
                        (S > 1 ? 1.0 : 0.0);
       if (bt == 0.0 || t < bt) {
         bt = t;
@@ -315,16 +318,16 @@ int f32_fwd_ntiles_max(int N) { return cdiv(N, 64); }
 cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
                          const EpiArgs& ep, int* err, cudaStream_t st) {
   const Plan p = plan_fwd(plan_rows, N, K);
-  if (p.kind == TENSOR && aligned(A, lda) && aligned(B, ldb))
-    return f32tc_gemm_fwd(A, lda, B, ldb, M, N, K, p.S, ep, err, st);
+  if (p.kind >= TENSOR && aligned(A, lda) && aligned(B, ldb))
+    return f32tc_gemm_fwd(A, lda, B, ldb, M, N, K, p.S, p.kind == TENSOR_PAIR, ep, err, st);
   return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, p, ep, AdamArgs{}, st);
 }
 
 cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, float* C, int ldc,
                            int* err, cudaStream_t st) {
   const Plan p = plan_kmajor(M, N, K);
-  if (p.kind == TENSOR && aligned(A, lda) && aligned(B, ldb))
-    return f32tc_gemm_store(A, lda, B, ldb, M, N, K, p.S, C, ldc, err, st);
+  if (p.kind >= TENSOR && aligned(A, lda) && aligned(B, ldb))
+    return f32tc_gemm_store(A, lda, B, ldb, M, N, K, p.S, p.kind == TENSOR_PAIR, C, ldc, err, st);
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
   return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, p, ep, AdamArgs{}, st);
 }
@@ -334,8 +337,8 @@ cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int
 cudaError_t f32_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, float* C, int ldc,
                            bool in_order, int* err, cudaStream_t st) {
   const Plan p = in_order ? Plan{TILE_128, 1} : plan_of(N, K, R, true);
-  if (p.kind == TENSOR && aligned(G, ldg) && aligned(X, ldx))
-    return f32tc_gemm_wgrad(G, ldg, X, ldx, R, N, K, p.S, C, ldc, err, st);
+  if (p.kind >= TENSOR && aligned(G, ldg) && aligned(X, ldx))
+    return f32tc_gemm_wgrad(G, ldg, X, ldx, R, N, K, p.S, p.kind == TENSOR_PAIR, C, ldc, err, st);
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
   return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, p, ep, AdamArgs{}, st);
 }
@@ -343,7 +346,7 @@ cudaError_t f32_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int
 bool f32_wgrad_adam_fits(int R, int N, int K) {
   const Plan p = plan_of(N, K, R, true);
   const int T = p.kind == TILE_64 ? 64 : 128;
-  return p.kind != TENSOR && (long long)cdiv(N, T) * cdiv(K, T) * p.S <= 2 * 152;
+  return p.kind < TENSOR && (long long)cdiv(N, T) * cdiv(K, T) * p.S <= 2 * 152;
 }
 
 cudaError_t f32_gemm_wgrad_adam(const float* G, int ldg, const float* X, int ldx, int R, const AdamArgs& a,

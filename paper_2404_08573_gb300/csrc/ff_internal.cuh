@@ -348,12 +348,13 @@ cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int
                            float* C, int ldc, int* err, cudaStream_t st);
 cudaError_t f32_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K,
                            float* C, int ldc, bool in_order, int* err, cudaStream_t st);
-// The tensor-core forms (S: slices of K), ff_gemm_f32tc.cu.
-cudaError_t f32tc_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S,
+// The tensor-core forms (S: slices of K; pair: 256 x 256 tiles by CTA pairs),
+// ff_gemm_f32tc.cu.
+cudaError_t f32tc_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, bool pair,
                            const EpiArgs& ep, int* err, cudaStream_t st);
-cudaError_t f32tc_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S,
+cudaError_t f32tc_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, bool pair,
                              float* C, int ldc, int* err, cudaStream_t st);
-cudaError_t f32tc_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, int S,
+cudaError_t f32tc_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, int S, bool pair,
                              float* C, int ldc, int* err, cudaStream_t st);
 // The weight gradient of a.N x a.K outputs over R rows and the Adam step it
 // feeds, in the GEMM's epilogue (dW itself only to a.keep_dW).  Pays where
