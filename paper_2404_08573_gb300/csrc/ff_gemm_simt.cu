@@ -254,6 +254,7 @@ Plan plan_of(int M, int N, int K, bool tensor) {
     const double tiles = (double)cdiv(M, T) * cdiv(N, T);
     for (int S = 1; S <= kMaxSplit; S *= 2) {
       if (S > 1 && steps < 2 * S) break;
+      if (kind == TENSOR_PAIR && S > 2) break;  // no clusters of 8
       // CTAs (pairs) an SM (two SMs) runs in all
       const double per_sm = cdiv((long long)(tiles * S), kind == TENSOR_PAIR ? 76 : 152);
       const double step = kind == TILE_64 ? 0.95 : kind == TILE_128 ? 3.3 : kind == TENSOR ? 1.7 : 2.7;
