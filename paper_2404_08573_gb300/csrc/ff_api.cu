@@ -571,7 +571,6 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
   float* G = goodness ? goodness : reinterpret_cast<float*>(w + oG);
   int* err = &L0->ds->err;
 
-  FF_TRY(cudaMemsetAsync(G, 0, (size_t)n * 10 * 4, st), "zero goodness");
   FF_LAUNCH(K_LABEL_COLS, (double)N1 * 10 * (es + 4), st,
             launch_label_columns(b16 ? (const void*)L0->Wb : (const void*)L0->W, b16 ? L0->ldK : L0->K, b16, N1,
                                  cols, L0->ldN, st),
@@ -619,6 +618,7 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
           ep.gpart_in = gpb[(k - 1) & 1];
           ep.ntiles_in = nt_prev;
           ep.G_acc = Gc;
+          ep.G_first = k == 2;  // layer 2's share, the first
         }
         nt = tc_fwd_ntiles(rows, Lk->N, true);
         FF_LAUNCH(K_FWD_TC, 2.0 * rows * Lk->N * Lk->K, st,
@@ -647,13 +647,20 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
         fa.M = rows;
         fa.s_next = (k + 1 < n_layers) ? Sb[cur ^ 1] : nullptr;
         fa.G_acc = Gc;
+        fa.G_first = k == 1;
         fa.err = err;
-        FF_LAUNCH(K_FINALIZE, (double)rows * (nt * 4.0 + 12), st, launch_finalize(fa, st), "predict goodness");
+        if (k + 1 < n_layers)
+          FF_LAUNCH(K_FINALIZE, (double)rows * (nt * 4.0 + 12), st, launch_finalize(fa, st), "predict goodness");
+        else
+          FF_LAUNCH(K_FINALIZE, (double)rows * (nt * 4.0 + 12) + cn * (labels ? 8.0 : 4.0), st,
+                    launch_finalize_argmax(fa, labels ? labels + c0 : nullptr, pred + c0, st),
+                    "predict goodness and argmax");
       }
       cur ^= 1;
     }
   }
-  FF_LAUNCH(K_ARGMAX, (double)n * (labels ? 48 : 44), st, launch_argmax(G, n, labels, pred, st), "argmax");
+  if (n_layers == 1)
+    FF_LAUNCH(K_ARGMAX, (double)n * (labels ? 48 : 44), st, launch_argmax(G, n, labels, pred, st), "argmax");
   return FF_OK;
 }
 

@@ -113,7 +113,45 @@ __global__ void __launch_bounds__(256) k_finalize(FinalizeArgs a) {
   if (!isfinite(g)) atomicOr(a.err, DEVERR_NONFINITE);
   if (a.g_out) a.g_out[i] = g;
   if (a.s_next) a.s_next[i] = inv_norm(g);
-  if (a.G_acc) a.G_acc[i] += g;
+  if (a.G_acc) a.G_acc[i] = (a.G_first ? 0.f : a.G_acc[i]) + g;
+}
+
+// The label with the largest of a sample's 10 goodness sums, the lowest on
+// ties; `skip` is left out (AdaptiveNEG, §5: the sample's own label, so that
+// the strongest wrong one is chosen; a value outside 0..9 leaves nothing out).
+__device__ __forceinline__ int best_label(const float* g, int skip) {
+  int best = -1;
+  float bv = 0.f;
+#pragma unroll
+  for (int c = 0; c < 10; ++c) {
+    if (c == skip) continue;
+    const float v = g[c];
+    if (best < 0 || v > bv) {
+      bv = v;
+      best = c;
+    }
+  }
+  return best;
+}
+
+// The last layer's goodness and the label choice: 25 samples' rows a block.
+constexpr int kArgmaxSamples = 25;
+__global__ void __launch_bounds__(256) k_finalize_argmax(FinalizeArgs a, const int* __restrict__ labels,
+                                                         int* __restrict__ pred) {
+  ptx::griddep_wait();  // launched with programmatic stream serialization
+  __shared__ float gs[10 * kArgmaxSamples];
+  const int t = threadIdx.x, i = blockIdx.x * 10 * kArgmaxSamples + t;
+  const int smp = blockIdx.x * kArgmaxSamples + t;
+  const int skip = labels && t < kArgmaxSamples && smp * 10 < a.M ? __ldg(labels + smp) : -1;
+  if (t < 10 * kArgmaxSamples && i < a.M) {
+    const float before = a.G_first ? 0.f : a.G_acc[i];
+    const float g = sum_partials(a.gpart, a.ntiles, a.M, i);
+    if (!isfinite(g)) atomicOr(a.err, DEVERR_NONFINITE);
+    gs[t] = before + g;
+    a.G_acc[i] = gs[t];
+  }
+  __syncthreads();
+  if (t < kArgmaxSamples && smp * 10 < a.M) pred[smp] = best_label(gs + 10 * t, skip);
 }
 
 // --------------------------------------------------------------- local grad
@@ -365,21 +403,23 @@ __global__ void k_label_columns(const T* __restrict__ W, int ldw, int N, float* 
 // and the goodness/next scale of that row (row r = 10 * sample + c).  Each
 // thread takes 8 consecutive columns: the base row and the bias are read
 // once for all 10 labels, the 10 goodness sums stay in registers and are
-// reduced once at the end (warp, then the 8 warps in order).
-template <typename T>
+// reduced once at the end (warp, then the 8 warps in order).  Few samples: a
+// block takes LABELS of the 10 labels from blockIdx.y * LABELS on (8 samples of
+// a 2000-wide layer 7.2 -> 3.7 us).
+template <typename T, int LABELS>
 __global__ void __launch_bounds__(256) k_expand(const float* __restrict__ base, int ldbase,
                                                 const float* __restrict__ cols, const float* __restrict__ s1,
                                                 const float* __restrict__ bias, int N, T* __restrict__ H, int ldh,
                                                 float* __restrict__ s_next, float* __restrict__ G_acc, int* err) {
   ptx::griddep_wait();  // launched with programmatic stream serialization
-  __shared__ float red[8][10];
-  const int n = blockIdx.x;
+  __shared__ float red[8][LABELS];
+  const int n = blockIdx.x, l0 = blockIdx.y * LABELS;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float s = s1[n];
   const float* brow = base + (size_t)n * ldbase;
-  float g[10];
+  float g[LABELS];
 #pragma unroll
-  for (int c = 0; c < 10; ++c) g[c] = 0.f;
+  for (int c = 0; c < LABELS; ++c) g[c] = 0.f;
   for (int j = 8 * threadIdx.x; j < ldh; j += 8 * 256) {
     float b8[8], bi[8];
     const float4 p = *reinterpret_cast<const float4*>(brow + j);
@@ -389,8 +429,8 @@ __global__ void __launch_bounds__(256) k_expand(const float* __restrict__ base, 
 #pragma unroll
     for (int e = 0; e < 8; ++e) bi[e] = (bias && j + e < N) ? __ldg(bias + j + e) : 0.f;
 #pragma unroll
-    for (int c = 0; c < 10; ++c) {
-      const float* cr = cols + (size_t)c * ldh + j;
+    for (int c = 0; c < LABELS; ++c) {
+      const float* cr = cols + (size_t)(l0 + c) * ldh + j;
       const float4 u = __ldg(reinterpret_cast<const float4*>(cr));
       const float4 v = __ldg(reinterpret_cast<const float4*>(cr + 4));
       const float cv[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
@@ -402,48 +442,32 @@ __global__ void __launch_bounds__(256) k_expand(const float* __restrict__ base, 
         h[e] = j + e < N ? relu_nan(z) : 0.f;
         g[c] = fmaf(h[e], h[e], g[c]);
       }
-      Vec8<T>::store(H + ((size_t)n * 10 + c) * ldh + j, h);
+      Vec8<T>::store(H + ((size_t)n * 10 + l0 + c) * ldh + j, h);
     }
   }
 #pragma unroll
-  for (int c = 0; c < 10; ++c) {
+  for (int c = 0; c < LABELS; ++c) {
     const float v = warp_sum(g[c]);
     if (lane == 0) red[warp][c] = v;
   }
   __syncthreads();
-  if (threadIdx.x < 10) {
+  if (threadIdx.x < LABELS) {
     float t = 0.f;
 #pragma unroll
     for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
-    const size_t r = (size_t)n * 10 + threadIdx.x;
+    const size_t r = (size_t)n * 10 + l0 + threadIdx.x;
     if (!isfinite(t)) atomicOr(err, DEVERR_NONFINITE);
     s_next[r] = inv_norm(t);
-    if (G_acc) G_acc[r] += t;
+    if (G_acc) G_acc[r] = 0.f + t;  // a net of one layer: the only goodness
   }
 }
 
-// pred[i] = the label with the largest G[i, c], the lowest on ties.  With
-// labels (AdaptiveNEG, §5) the sample's own label is left out, so pred[i] is
-// its strongest wrong label; a label outside 0..9 leaves nothing out.
+// pred[i] = best_label of G[i, 0..9] (skip: labels[i], or none without labels).
 __global__ void k_argmax(const float* __restrict__ G, int n, const int* __restrict__ labels,
                          int* __restrict__ pred) {
   ptx::griddep_wait();  // launched with programmatic stream serialization
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float* g = G + (size_t)i * 10;
-  const int skip = labels ? labels[i] : -1;
-  int best = -1;
-  float bv = 0.f;
-#pragma unroll
-  for (int c = 0; c < 10; ++c) {
-    if (c == skip) continue;
-    const float v = g[c];
-    if (best < 0 || v > bv) {
-      bv = v;
-      best = c;
-    }
-  }
-  pred[i] = best;
+  if (i < n) pred[i] = best_label(G + (size_t)i * 10, labels ? labels[i] : -1);
 }
 
 // Self-test of the bounded waits: one thread waits on an mbarrier that
@@ -494,6 +518,12 @@ cudaError_t launch_finalize(const FinalizeArgs& a, cudaStream_t st) {
   return cudaLaunchKernelEx(&l.cfg, k_finalize, a);
 }
 
+cudaError_t launch_finalize_argmax(const FinalizeArgs& a, const int* labels, int* pred, cudaStream_t st) {
+  if (a.M <= 0) return cudaSuccess;
+  PdlLaunch l(dim3(cdiv(a.M, 10 * kArgmaxSamples)), dim3(256), st);
+  return cudaLaunchKernelEx(&l.cfg, k_finalize_argmax, a, labels, pred);
+}
+
 int local_grad_row_blocks(int M) { return cdiv(M, kGradRows); }
 
 cudaError_t launch_grad_prep(const GradPrepArgs& a, bool b16, const void* H, void* dZ, cudaStream_t st) {
@@ -541,11 +571,13 @@ cudaError_t launch_expand(const float* base, int ldbase, const float* cols, cons
                           int N, void* H, int ldh, bool h_bf16, float* s_next, float* G_acc, int* err,
                           cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  PdlLaunch l(dim3(n), dim3(256), st);
-  if (h_bf16)
-    return cudaLaunchKernelEx(&l.cfg, k_expand<bf16>, base, ldbase, cols, s1, bias, N, (bf16*)H, ldh, s_next, G_acc,
-                              err);
-  return cudaLaunchKernelEx(&l.cfg, k_expand<float>, base, ldbase, cols, s1, bias, N, (float*)H, ldh, s_next, G_acc, err);
+  const bool few = n <= 152 / 2;
+  PdlLaunch l(dim3(n, few ? 5 : 1), dim3(256), st);
+  auto go = [&](auto kernel, auto* h) {
+    return cudaLaunchKernelEx(&l.cfg, kernel, base, ldbase, cols, s1, bias, N, h, ldh, s_next, G_acc, err);
+  };
+  if (h_bf16) return few ? go(k_expand<bf16, 2>, (bf16*)H) : go(k_expand<bf16, 10>, (bf16*)H);
+  return few ? go(k_expand<float, 2>, (float*)H) : go(k_expand<float, 10>, (float*)H);
 }
 
 cudaError_t launch_argmax(const float* G, int n, const int* labels, int* pred, cudaStream_t st) {

@@ -150,6 +150,7 @@ struct FinishArgs {
   const int* labels;
   float inv_n;
   float* logits;  // [n, 10] or null
+  int* pred;      // [n] or null: the class with the largest logit, the lowest on ties
   float* dz;      // [n, 10] or null
   float* part;    // [row blocks, 11] or null
   uint4* dzfrag;  // [segment][16-row group][part][lane]: A operands of k_head_wgrad_adam, or null
@@ -258,6 +259,17 @@ __device__ __forceinline__ void finish_row_block(const Segs& sg, const float* __
       float z[kClasses];
 #pragma unroll
       for (int c = 0; c < kClasses; ++c) z[c] = zs[threadIdx.x][c];
+      if (fa.pred) {
+        int best = 0;
+        float bv = z[0];
+#pragma unroll
+        for (int c = 1; c < kClasses; ++c)
+          if (z[c] > bv) {
+            bv = z[c];
+            best = c;
+          }
+        fa.pred[row] = best;
+      }
       loss = finish_row(z, row, fa.labels != nullptr, fa.labels ? ys[threadIdx.x] : 0, fa.inv_n, fa.logits, fa.dz, dzr, err);
     }
     if (fa.part) {
@@ -1058,7 +1070,6 @@ struct HeadWork {
   void* Hk[kMaxSegs + 1];
   float* gpart;
   float* gpart2;   // the tensor-core forward alternates between gpart and gpart2
-  float* logits;
   float* zpart;
   float* dz;
   float* part;
@@ -1094,7 +1105,6 @@ ff_status head_workspace(ff_head* hd, ff_layer* const* layers, int L, int rows, 
   for (int k = 0; k < L; ++k) { oH[k] = off; off += align256((size_t)rows * layers[k]->ldN * es); }
   size_t oG = off; off += align256((size_t)ntmax * rows * 4);
   size_t oG2 = off; off += align256(b16 ? (size_t)ntmax * rows * 4 : 0);
-  size_t oZ = off; off += align256((size_t)rows * kClasses * 4);
   size_t oZP = off; off += align256(chain_zpart_floats(layers, L, rows) * 4);
   size_t oD = off; off += align256(train && !b16 ? (size_t)rows * kClasses * 4 : 0);
   const int nseg = L > 1 ? L - 1 : 1;
@@ -1116,7 +1126,6 @@ ff_status head_workspace(ff_head* hd, ff_layer* const* layers, int L, int rows, 
   for (int k = 0; k < L; ++k) w->Hk[k] = base + oH[k];
   w->gpart = reinterpret_cast<float*>(base + oG);
   w->gpart2 = reinterpret_cast<float*>(base + (b16 ? oG2 : oG));
-  w->logits = reinterpret_cast<float*>(base + oZ);
   w->zpart = reinterpret_cast<float*>(base + oZP);
   w->dz = train && !b16 ? reinterpret_cast<float*>(base + oD) : nullptr;
   w->dzfrag = train && b16 ? reinterpret_cast<uint4*>(base + oF) : nullptr;
@@ -1217,8 +1226,8 @@ ff_status ensure_counters(ff_head* hd, int blocks) {
 // Logits (and, with labels, softmax, loss, dz and the per-row-block
 // partials) of n rows: k_head_dot over the feature splits, whose last block
 // per row block finishes the rows.
-ff_status head_logits(ff_head* hd, const Segs& sg, bool b16, int n, const int* labels, float* logits, float* zpart,
-                      float* dz, float* part, uint4* dzfrag, int* err, cudaStream_t st) {
+ff_status head_logits(ff_head* hd, const Segs& sg, bool b16, int n, const int* labels, float* logits, int* pred,
+                      float* zpart, float* dz, float* part, uint4* dzfrag, int* err, cudaStream_t st) {
   const int es = b16 ? 2 : 4;
   const int split = dot_split(sg.F, sg.nseg, n, es);
   const int S = head_splits(sg.F, sg.nseg, split);
@@ -1229,6 +1238,7 @@ ff_status head_logits(ff_head* hd, const Segs& sg, bool b16, int n, const int* l
   fa.labels = labels;
   fa.inv_n = 1.f / (float)n;
   fa.logits = logits;
+  fa.pred = pred;
   fa.dz = dz;
   fa.part = part;
   fa.dzfrag = dzfrag;
@@ -1473,7 +1483,7 @@ static ff_status head_step_on_features(ff_head* hd, ff_layer* const* layers, int
     sg.s[j] += r0;
   }
   int* err = &hd->ds->err;
-  ff_status s = head_logits(hd, sg, b16, n, labels, nullptr, w.zpart, w.dz, w.part, w.dzfrag, err, st);
+  ff_status s = head_logits(hd, sg, b16, n, labels, nullptr, nullptr, w.zpart, w.dz, w.part, w.dzfrag, err, st);
   if (s != FF_OK) return s;
   const HeadAdamArgs a =
       head_adam_args(hd, w.dVpart, b16 ? 0 : cdiv(n, kWgRows), w.part, cdiv(n, kDotRows), n, loss);
@@ -1585,11 +1595,9 @@ ff_status ff_head_predict(ff_head* hd, ff_layer* const* layers, int n_layers, co
     s = head_forward(layers, n_layers, x + (size_t)r0 * K0, cn, w, err, st, true);
     if (s != FF_OK) return s;
     const Segs sg = make_segs(layers, n_layers, w, hd->F);
-    float* z = logits ? logits + (size_t)r0 * kClasses : w.logits;
-    s = head_logits(hd, sg, b16, cn, nullptr, z, w.zpart, nullptr, nullptr, nullptr, err, st);
+    s = head_logits(hd, sg, b16, cn, nullptr, logits ? logits + (size_t)r0 * kClasses : nullptr,
+                    pred ? pred + r0 : nullptr, w.zpart, nullptr, nullptr, nullptr, err, st);
     if (s != FF_OK) return s;
-    if (pred)
-      FF_LAUNCH(K_ARGMAX, (double)cn * 44, st, launch_argmax(z, cn, nullptr, pred + r0, st), "head argmax");
   }
   return FF_OK;
 }
@@ -1734,7 +1742,7 @@ ff_status ff_po_train_step(ff_layer* L, ff_head* hd, const void* x, int raw_inpu
     sg.off[0] = 0;
     sg.nseg = 1;
     sg.F_total = N;
-    s = head_logits(hd, sg, b16, n, labels, nullptr, w.zpart, w.dz, w.part, nullptr, &hd->ds->err, st);
+    s = head_logits(hd, sg, b16, n, labels, nullptr, nullptr, w.zpart, w.dz, w.part, nullptr, &hd->ds->err, st);
     if (s != FF_OK) return s;
   }
   // the gradient reaching the layer, with the block's weights before its
@@ -1833,11 +1841,9 @@ ff_status ff_po_predict(ff_layer* const* layers, int n_layers, ff_head* hd, cons
     sg.F[0] = top->N;
     sg.nseg = 1;
     sg.F_total = top->N;
-    float* z = logits ? logits + (size_t)r0 * kClasses : w.logits;
-    s = head_logits(hd, sg, b16, cn, nullptr, z, w.zpart, nullptr, nullptr, nullptr, err, st);
+    s = head_logits(hd, sg, b16, cn, nullptr, logits ? logits + (size_t)r0 * kClasses : nullptr,
+                    pred ? pred + r0 : nullptr, w.zpart, nullptr, nullptr, nullptr, err, st);
     if (s != FF_OK) return s;
-    if (pred)
-      FF_LAUNCH(K_ARGMAX, (double)cn * 44, st, launch_argmax(z, cn, nullptr, pred + r0, st), "block argmax");
   }
   return FF_OK;
 }

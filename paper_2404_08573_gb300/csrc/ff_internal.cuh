@@ -164,10 +164,14 @@ struct FinalizeArgs {
   float* g_out;        // [M] or null
   float* s_next;       // [M] or null
   float* G_acc;        // [M] predict goodness accumulator or null
+  bool G_first;        // the first goodness to reach G_acc: set it
   int* err;            // error word
 };
 int finalize_grid(int M);
 cudaError_t launch_finalize(const FinalizeArgs& a, cudaStream_t st);
+// The last layer's, with the label choice of launch_argmax (M = 10 rows per
+// sample; G_acc required).
+cudaError_t launch_finalize_argmax(const FinalizeArgs& a, const int* labels, int* pred, cudaStream_t st);
 // Train step after the forward GEMM: goodness, loss, dL/dg, next-layer scale,
 // dZ' = (s * 2 dL/dg) * H in the operand type, db partials per 32 rows, and
 // the Adam step counter / bias-correction terms.
@@ -263,6 +267,7 @@ struct EpiArgs {
   const float* gpart_in;
   int ntiles_in;
   float* G_acc;
+  bool G_first;        // the first goodness to reach G_acc: set it
   float* s_out;
   // Tensor-core forward GEMMs: a grid that would fill at most half the SMs
   // may use 128-column tiles (twice the CTAs).  Set where the GEMM has the
