@@ -6,6 +6,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <algorithm>
 #include <chrono>
 #include <new>
 #include <thread>
@@ -495,8 +496,8 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
   const size_t es = b16 ? 2 : 4;
   // fp32 layers: GEMMs that fill the GPU as three TF32 products where every
   // layer's rows allow TMA (4600 x 2000 over 2000: 240 TFLOP/s of fp32 terms),
-  // the others as the training GEMMs run (800 x 2000 over 2000, a last chunk:
-  // 93 us before, 78 now; 460 x 2000 over 784: 44 and 23 us)
+  // the others and layer 1 as the training GEMMs run (800 x 2000 over 2000, a
+  // last chunk: 93 us with TF32 products, 57 so; 460 x 2000 over 784: 44 and 23)
   bool f32tc = !b16;
   for (int k = 0; k < n_layers && f32tc; ++k) f32tc = tc_f32_supported(layers[k]->K, layers[k]->ldK, layers[k]->K);
   int ldmax = 0, ntmax = 0;
@@ -537,10 +538,18 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
   if (C > n) C = n;
   const int R = 10 * C;
   const int N1 = L0->N;
+  // Layer 1 up to the expansion (overlay, base GEMM) runs once for a group of
+  // whole chunks, as many as kPredictGroupBytes of operand and base rows hold:
+  // a chunk's share is a small GEMM that leaves most of the GPU idle (972
+  // samples of 784 -> 2000: 11.5 + 5.9 us each; 9720 at once 23 + 10).
+  constexpr size_t kPredictGroupBytes = size_t(96) << 20;
+  const size_t chunk_bytes = (size_t)C * (L0->ldK * es + L0->ldN * 4);
+  const long long group_chunks = chunk_bytes < kPredictGroupBytes ? (long long)(kPredictGroupBytes / chunk_bytes) : 1;
+  const int GR = (int)std::min<long long>(n, group_chunks * C);  // samples per group
   size_t off = 0;
-  const size_t oX = off; off += align256((size_t)C * L0->ldK * es);
-  const size_t oS1 = off; off += align256((size_t)C * 4);
-  const size_t oBase = off; off += align256((size_t)C * L0->ldN * 4);
+  const size_t oX = off; off += align256((size_t)GR * L0->ldK * es);
+  const size_t oS1 = off; off += align256((size_t)GR * 4);
+  const size_t oBase = off; off += align256((size_t)GR * L0->ldN * 4);
   const size_t oCols = off; off += align256((size_t)10 * L0->ldN * 4);
   const size_t oH0 = off; off += align256((size_t)R * ldmax * es);
   const size_t oH1 = off; off += align256((size_t)R * ldmax * es);
@@ -578,28 +587,28 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
   for (int c0 = 0; c0 < n; c0 += C) {
     const int cn = (n - c0) < C ? (n - c0) : C;
     const int rows = 10 * cn;
-    FF_LAUNCH(K_OVERLAY, (double)cn * (L0->K * 4.0 + L0->ldK * es + 4), st,
-              launch_overlay(x + (size_t)c0 * L0->K, nullptr, cn, L0->K, X0, L0->ldK, b16, s1, 1, st),
-              "zero label area");
-    if (b16) {
-      FF_LAUNCH(K_STORE_TC, 2.0 * cn * N1 * L0->K, st,
-                tc_gemm_store(static_cast<const bf16*>(X0), L0->ldK, L0->Wb, L0->ldK, cn, N1, L0->K, base, L0->ldN,
-                              err, st),
-                "layer-1 base GEMM (tcgen05)");
-    } else if (f32tc && tc_full_shape(cn, N1)) {
-      FF_LAUNCH(K_STORE_TC, 2.0 * cn * N1 * L0->K, st,
-                tc_gemm_store_f32(static_cast<const float*>(X0), L0->ldK, L0->W, L0->K, cn, N1, L0->K, base,
-                                  L0->ldN, err, st),
-                "layer-1 base GEMM (fp32, tcgen05 TF32 x 3)");
-    } else {
-      FF_LAUNCH(K_STORE_SIMT, 2.0 * cn * N1 * L0->K, st,
-                f32_gemm_store(static_cast<const float*>(X0), L0->ldK, L0->W, L0->K, cn, N1, L0->K, base, L0->ldN,
-                               err, st),
-                "layer-1 base GEMM (fp32)");
+    const int g0 = c0 % GR;  // the chunk's first row of its group
+    if (g0 == 0) {
+      const int gn = std::min(n - c0, GR);
+      FF_LAUNCH(K_OVERLAY, (double)gn * (L0->K * 4.0 + L0->ldK * es + 4), st,
+                launch_overlay(x + (size_t)c0 * L0->K, nullptr, gn, L0->K, X0, L0->ldK, b16, s1, 1, st),
+                "zero label area");
+      if (b16) {
+        FF_LAUNCH(K_STORE_TC, 2.0 * gn * N1 * L0->K, st,
+                  tc_gemm_store(static_cast<const bf16*>(X0), L0->ldK, L0->Wb, L0->ldK, gn, N1, L0->K, base, L0->ldN,
+                                err, st),
+                  "layer-1 base GEMM (tcgen05)");
+      } else {
+        FF_LAUNCH(K_STORE_SIMT, 2.0 * gn * N1 * L0->K, st,
+                  f32_gemm_store(static_cast<const float*>(X0), L0->ldK, L0->W, L0->K, gn, N1, L0->K, base, L0->ldN,
+                                 err, st),
+                  "layer-1 base GEMM (fp32)");
+      }
     }
     float* Gc = G + (size_t)c0 * 10;
     FF_LAUNCH(K_EXPAND, (double)cn * (L0->ldN * 4.0 + 10.0 * L0->ldN * es + 40), st,
-              launch_expand(base, L0->ldN, cols, s1, L0->cfg.has_bias ? L0->b : nullptr, cn, N1, Hb[0], L0->ldN, b16,
+              launch_expand(base + (size_t)g0 * L0->ldN, L0->ldN, cols, s1 + g0,
+                            L0->cfg.has_bias ? L0->b : nullptr, cn, N1, Hb[0], L0->ldN, b16,
                             Sb[0], n_layers == 1 ? Gc : nullptr, err, st),
               "layer-1 expansion");
     int cur = 0;

@@ -465,17 +465,4 @@ cudaError_t tc_gemm_fwd_f32(const float* A, int lda, const float* B, int ldb, in
                                                                                               ep, err, st);
 }
 
-cudaError_t tc_gemm_store_f32(const float* A, int lda, const float* B, int ldb, int M, int N, int K, float* Cm,
-                              int ldc, int* err, cudaStream_t st) {
-  if (!tc_f32_supported(K, lda, ldb) || !tc_full_shape(M, N)) return cudaErrorInvalidValue;
-  CUtensorMap ta, tb, tc;
-  if (!make_map(&ta, A, 4, K, M, lda, 32, BM) || !make_map(&tb, B, 4, K, N, ldb, 32, b_box_rows(FWD_BN)))
-    return cudaErrorInvalidValue;
-  const int tma = store_map(&tc, Cm, ldc, M, N) ? 1 : 0;
-  if (!tma) tc = ta;  // unused
-  EpiArgs ep{nullptr, nullptr, Cm, ldc, nullptr};
-  return launch_tc<FWD_BN, false, false, MODE_STORE, USE_PAIR, NSTAGES_F32, ROW_SUBTILES, 1, 4>(ta, tb, tc, tma, M, N,
-                                                                                                K, ep, err, st);
-}
-
 }  // namespace ff
