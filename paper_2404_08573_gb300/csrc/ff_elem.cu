@@ -15,6 +15,8 @@
 //                the 9 wrong labels for AdaptiveNEG negatives (§5)
 // Reductions use fixed orders (no floating-point atomics), so results do not
 // depend on scheduling.
+#include <type_traits>
+
 #include "ff_adam.cuh"
 #include "ff_internal.cuh"
 #include "ff_ptx.cuh"
@@ -403,11 +405,14 @@ __global__ void k_label_columns(const T* __restrict__ W, int ldw, int N, float* 
 // and the goodness/next scale of that row (row r = 10 * sample + c).  Each
 // thread takes 8 consecutive columns: the base row and the bias are read
 // once for all 10 labels, the 10 goodness sums stay in registers and are
-// reduced once at the end (warp, then the 8 warps in order).  Few samples: a
-// block takes LABELS of the 10 labels from blockIdx.y * LABELS on (8 samples of
-// a 2000-wide layer 7.2 -> 3.7 us).
+// reduced once at the end (warp, then the 8 warps in order).  Bound by the
+// latency of its loads: five blocks an SM (48 registers) take 972 samples of
+// a 2000-wide layer in 18.2 us, four in 22; six and more spill.  Few samples:
+// a block takes LABELS of the 10 labels from blockIdx.y * LABELS on (8
+// samples: 7.2 us with 10 labels a block, 3.7 with 2; 280: 10.4, 7.8 with 5;
+// 972: 18.2, 18.6 with 5, 28 with 2).
 template <typename T, int LABELS>
-__global__ void __launch_bounds__(256) k_expand(const float* __restrict__ base, int ldbase,
+__global__ void __launch_bounds__(256, 5) k_expand(const float* __restrict__ base, int ldbase,
                                                 const float* __restrict__ cols, const float* __restrict__ s1,
                                                 const float* __restrict__ bias, int N, T* __restrict__ H, int ldh,
                                                 float* __restrict__ s_next, float* __restrict__ G_acc, int* err) {
@@ -571,13 +576,16 @@ cudaError_t launch_expand(const float* base, int ldbase, const float* cols, cons
                           int N, void* H, int ldh, bool h_bf16, float* s_next, float* G_acc, int* err,
                           cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  const bool few = n <= 152 / 2;
-  PdlLaunch l(dim3(n, few ? 5 : 1), dim3(256), st);
+  const int labels = n <= 152 / 2 ? 2 : n <= 2 * 152 ? 5 : 10;  // per block
+  PdlLaunch l(dim3(n, 10 / labels), dim3(256), st);
   auto go = [&](auto kernel, auto* h) {
     return cudaLaunchKernelEx(&l.cfg, kernel, base, ldbase, cols, s1, bias, N, h, ldh, s_next, G_acc, err);
   };
-  if (h_bf16) return few ? go(k_expand<bf16, 2>, (bf16*)H) : go(k_expand<bf16, 10>, (bf16*)H);
-  return few ? go(k_expand<float, 2>, (float*)H) : go(k_expand<float, 10>, (float*)H);
+  auto pick = [&](auto* h) {
+    using T = std::remove_pointer_t<decltype(h)>;
+    return labels == 2 ? go(k_expand<T, 2>, h) : labels == 5 ? go(k_expand<T, 5>, h) : go(k_expand<T, 10>, h);
+  };
+  return h_bf16 ? pick((bf16*)H) : pick((float*)H);
 }
 
 cudaError_t launch_argmax(const float* G, int n, const int* labels, int* pred, cudaStream_t st) {
