@@ -169,12 +169,17 @@ __global__ void __launch_bounds__(256) k_finalize_argmax(FinalizeArgs a, const i
 // 1/max(sqrt g, 1e-12) and the block's loss partial (reduced by the Adam
 // kernel that follows on the same stream); block (0, 0) advances the Adam
 // step t and its bias-correction terms.
+// Bound by the load round trip and the block's tail for few rows, by memory
+// for many.  The tail sums one column per thread of the whole block
+// (conflict-free, coalesced partials); one warp summing 8 columns a lane
+// costs 6.9 us for 128 x 2000 against 4.6, 73 us for 8192 x 8192 against 64
+// (268 MB, 4.2 TB/s).  H kept packed in 48 registers, five blocks an SM: 67.
 constexpr int kGradRows = 32;
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_grad_prep(GradPrepArgs a, const T* __restrict__ H, T* __restrict__ dZ) {
   ptx::griddep_wait();  // launched with programmatic stream serialization
-  __shared__ float red[8][256 + 8];
+  __shared__ alignas(16) float red[8][256];
   __shared__ float lred[8], gpred[8], gnred[8], ared[8];
   const int r0 = blockIdx.y * kGradRows;
   const bool lead = blockIdx.x == 0;
@@ -265,18 +270,17 @@ __global__ void __launch_bounds__(256) k_grad_prep(GradPrepArgs a, const T* __re
     act = warp_sum(act);
     if (lane == 0) ared[threadIdx.y] = act;
   }
-#pragma unroll
-  for (int e = 0; e < 8; ++e) red[threadIdx.y][lane * 8 + e] = db[e];
+  *reinterpret_cast<float4*>(&red[threadIdx.y][lane * 8]) = make_float4(db[0], db[1], db[2], db[3]);
+  *reinterpret_cast<float4*>(&red[threadIdx.y][lane * 8 + 4]) = make_float4(db[4], db[5], db[6], db[7]);
   __syncthreads();
+  {
+    const int c = threadIdx.y * 32 + lane, j = blockIdx.x * 256 + c;
+    float t = 0.f;
+#pragma unroll
+    for (int y = 0; y < 8; ++y) t += red[y][c];
+    if (j < a.N) a.dbpart[(size_t)blockIdx.y * a.N + j] = t;
+  }
   if (threadIdx.y == 0) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int j = cg + e;
-      float t = 0.f;
-#pragma unroll
-      for (int y = 0; y < 8; ++y) t += red[y][lane * 8 + e];
-      if (j < a.N) a.dbpart[(size_t)blockIdx.y * a.N + j] = t;
-    }
     if (a.stat_part && lane == 0) {
       float t = 0.f;
 #pragma unroll
