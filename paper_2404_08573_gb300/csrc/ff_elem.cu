@@ -172,8 +172,9 @@ __global__ void __launch_bounds__(256) k_finalize_argmax(FinalizeArgs a, const i
 // Bound by the load round trip and the block's tail for few rows, by memory
 // for many.  The tail sums one column per thread of the whole block
 // (conflict-free, coalesced partials); one warp summing 8 columns a lane
-// costs 6.9 us for 128 x 2000 against 4.6, 73 us for 8192 x 8192 against 64
-// (268 MB, 4.2 TB/s).  H kept packed in 48 registers, five blocks an SM: 67.
+// costs 6.9 us for 128 x 2000 against 4.6, 73 us for 8192 x 8192 against 61
+// (268 MB, 4.4 TB/s; 64 with the row scale a round trip later).  H kept
+// packed in 48 registers, five blocks an SM, costs 67.
 constexpr int kGradRows = 32;
 
 template <typename T>
@@ -205,9 +206,10 @@ __global__ void __launch_bounds__(256) k_grad_prep(GradPrepArgs a, const T* __re
   {
     const int k = lane >> 3, p = lane & 7;
     const int i = r0 + threadIdx.y + 8 * k;
-    float g = 0.f;
+    float g = 0.f, si = 0.f;
     if (i < a.M) {
       float v[8];
+      si = a.s[i];  // beside the partials, not a round trip after them
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int t = p + 8 * u;
@@ -225,7 +227,7 @@ __global__ void __launch_bounds__(256) k_grad_prep(GradPrepArgs a, const T* __re
       const float tt = pos ? a.theta - g : g - a.theta;  // the pair member's margin error
       const float sg = sigmoid_f(tt);
       cc = 2.f * (pos ? -sg : sg) / (float)a.B;
-      sc = a.s[i] * cc;
+      sc = si * cc;
       if (lead) {
         if (!isfinite(g)) atomicOr(a.err, DEVERR_NONFINITE);
         if (a.g_out) a.g_out[i] = g;
