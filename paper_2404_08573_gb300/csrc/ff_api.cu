@@ -591,7 +591,7 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
     if (g0 == 0) {
       const int gn = std::min(n - c0, GR);
       FF_LAUNCH(K_OVERLAY, (double)gn * (L0->K * 4.0 + L0->ldK * es + 4), st,
-                launch_overlay(x + (size_t)c0 * L0->K, nullptr, gn, L0->K, X0, L0->ldK, b16, s1, 1, st),
+                launch_overlay(x + (size_t)c0 * L0->K, nullptr, gn, L0->K, X0, L0->ldK, b16, s1, 1, st, 0, true),
                 "zero label area");
       if (b16) {
         FF_LAUNCH(K_STORE_TC, 2.0 * gn * N1 * L0->K, st,

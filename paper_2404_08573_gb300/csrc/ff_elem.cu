@@ -54,7 +54,7 @@ __device__ __forceinline__ void store4<bf16>(bf16* p, float a, float b, float c,
 template <typename T>
 __global__ void k_overlay(const float* __restrict__ x, const int* __restrict__ labels, int rows, int F,
                           T* __restrict__ out, int ldo, float* __restrict__ s_out, int mode, int src_rows) {
-  ptx::griddep_wait();  // launched with programmatic stream serialization
+  ptx::griddep_wait();  // predict launches it with programmatic stream serialization
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = blockIdx.x * 8 + warp;
   if (row >= rows) return;
@@ -91,7 +91,6 @@ __global__ void k_overlay(const float* __restrict__ x, const int* __restrict__ l
 
 template <typename T>
 __global__ void k_row_scale(const T* __restrict__ x, int ldx, int rows, int F, float* __restrict__ s_out) {
-  ptx::griddep_wait();  // launched with programmatic stream serialization
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = blockIdx.x * 8 + warp;
   if (row >= rows) return;
@@ -505,10 +504,10 @@ int grid_for(long long work, int per_block, int cap) {
 }  // namespace
 
 cudaError_t launch_overlay(const float* x, const int* labels, int rows, int F, void* out, int ldo, bool out_bf16,
-                           float* s_out, int mode, cudaStream_t st, int src_rows) {
+                           float* s_out, int mode, cudaStream_t st, int src_rows, bool dependent) {
   if (rows <= 0) return cudaSuccess;
   if (src_rows <= 0 || src_rows > rows) src_rows = rows;
-  PdlLaunch l(dim3(cdiv(rows, 8)), dim3(256), st);
+  PdlLaunch l(dim3(cdiv(rows, 8)), dim3(256), st, 0, dependent);
   if (out_bf16)
     return cudaLaunchKernelEx(&l.cfg, k_overlay<bf16>, x, labels, rows, F, (bf16*)out, ldo, s_out, mode, src_rows);
   return cudaLaunchKernelEx(&l.cfg, k_overlay<float>, x, labels, rows, F, (float*)out, ldo, s_out, mode, src_rows);
@@ -516,7 +515,7 @@ cudaError_t launch_overlay(const float* x, const int* labels, int rows, int F, v
 
 cudaError_t launch_row_scale(const void* x, int ldx, bool x_bf16, int rows, int F, float* s_out, cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
-  PdlLaunch l(dim3(cdiv(rows, 8)), dim3(256), st);
+  PdlLaunch l(dim3(cdiv(rows, 8)), dim3(256), st, 0, false);
   if (x_bf16) return cudaLaunchKernelEx(&l.cfg, k_row_scale<bf16>, (const bf16*)x, ldx, rows, F, s_out);
   return cudaLaunchKernelEx(&l.cfg, k_row_scale<float>, (const float*)x, ldx, rows, F, s_out);
 }

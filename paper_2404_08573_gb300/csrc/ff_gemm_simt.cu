@@ -1,8 +1,9 @@
-// fp32 GEMMs of the FF layer step on the CUDA cores (FFMA), for the exact
-// fp32 mode: the same contracts as the tensor-core GEMMs (forward with the
+// fp32 GEMMs of the FF layer step: the choice among the paths (plan_of), and
+// the CUDA-core (FFMA) kernels, which run the outputs too small for the
+// tensor-core ones (k_f32tc_gemm, k_f32tc_pair) and operands that these do
+// not take.  The same contracts as the bf16 GEMMs (forward with the
 // scale/bias/ReLU/goodness epilogue, plain fp32 store, weight gradient over
-// the batch rows), so the fp32 path is the full-precision statement of §3/§4
-// on the GPU.
+// the batch rows); either way fp32 operands and sums.
 //
 // Bound by the SM's shared-memory reads and FMA issue together (large
 // outputs reach 45 to 50 TFLOP/s), small ones by latency.  FMAs are issued in

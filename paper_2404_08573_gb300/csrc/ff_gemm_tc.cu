@@ -33,8 +33,8 @@
 //   warps 2..9  epilogue: tcgen05.ld of TMEM lanes 32*(warp%4).., one half of
 //               the columns each -> registers, fused scale/bias/ReLU/goodness
 //               (partials per 128-column half) or plain store
-// fp32 operands (OPB = 4, the exact-precision mode's forward and store
-// GEMMs): the tensor cores' TF32 products in three terms, A B ~ Ah Bh + Ah Bl +
+// fp32 operands (OPB = 4, the forward GEMMs of fp32 predictions that fill the
+// GPU): the tensor cores' TF32 products in three terms, A B ~ Ah Bh + Ah Bl +
 // Al Bh, where xh is x with the 13 low mantissa bits cleared (exactly a TF32
 // value) and xl = x - xh (exact in fp32); the dropped Al Bl and the TF32
 // truncation of xl leave a relative error near 2^-21 per product.  The

@@ -152,9 +152,12 @@ inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
 //   mode 2: out[:,0..9] = 0.1, the neutral label of the softmax head (§3).
 // Output row r reads input row r % src_rows (src_rows 0: rows): with
 // src_rows = B the B images of a pair batch are read once each for both
-// their positive and their negative row.
+// their positive and their negative row.  Launched plainly -- a layer's step
+// starts after waits on other streams' events -- except with `dependent`
+// (predict: one stream), with programmatic stream serialization.
 cudaError_t launch_overlay(const float* x, const int* labels, int rows, int F, void* out,
-                           int ldo, bool out_bf16, float* s_out, int mode, cudaStream_t st, int src_rows = 0);
+                           int ldo, bool out_bf16, float* s_out, int mode, cudaStream_t st, int src_rows = 0,
+                           bool dependent = false);
 // s_r = 1 / max(||x_r||, 1e-12) of an activation buffer.
 cudaError_t launch_row_scale(const void* x, int ldx, bool x_bf16, int rows, int F,
                              float* s_out, cudaStream_t st);
@@ -225,7 +228,7 @@ void add_dead(AdamArgs& a, void* p, size_t bytes);
 struct PdlLaunch {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  PdlLaunch(dim3 grid, dim3 block, cudaStream_t st, size_t smem = 0) {
+  PdlLaunch(dim3 grid, dim3 block, cudaStream_t st, size_t smem = 0, bool dependent = true) {
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
@@ -233,7 +236,7 @@ struct PdlLaunch {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = dependent ? 1 : 0;
   }
 };
 
