@@ -397,7 +397,6 @@ __global__ void k_to_bf16(const float* __restrict__ W, int N, int K, bf16* __res
 // ------------------------------------------------------------------ predict
 template <typename T>
 __global__ void k_label_columns(const T* __restrict__ W, int ldw, int N, float* __restrict__ cols, int ldc) {
-  ptx::griddep_wait();  // launched with programmatic stream serialization
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= ldc) return;
 #pragma unroll
@@ -572,7 +571,8 @@ cudaError_t launch_to_bf16(const float* W, int N, int K, bf16* Wb, int ldb, cuda
 }
 
 cudaError_t launch_label_columns(const void* W, int ldw, bool w_bf16, int N, float* cols, int ldc, cudaStream_t st) {
-  PdlLaunch l(dim3(cdiv(ldc, 256)), dim3(256), st);
+  // the first kernel of a prediction: plainly, like a layer step's overlay
+  PdlLaunch l(dim3(cdiv(ldc, 256)), dim3(256), st, 0, false);
   if (w_bf16) return cudaLaunchKernelEx(&l.cfg, k_label_columns<bf16>, (const bf16*)W, ldw, N, cols, ldc);
   return cudaLaunchKernelEx(&l.cfg, k_label_columns<float>, (const float*)W, ldw, N, cols, ldc);
 }
