@@ -208,40 +208,45 @@ __device__ __forceinline__ void finish_row_block(const Segs& sg, const float* __
     }
   }
   // z = c + the splits' partials in split order, a thread per row and class
-  // (read past L1: other blocks wrote them during this launch), eight splits'
+  // (read past L1: other blocks wrote them during this launch), sixteen splits'
   // loads in flight at a time
   __shared__ float zs[kDotRows][kClasses];
   // the segments' row scales and the labels, loaded beside the partials
   __shared__ float ss[kMaxSegs][kDotRows];
   __shared__ int ys[kDotRows];
-  if (fa.dzfrag)
-    for (int u = threadIdx.x; u < sg.nseg * kDotRows; u += 256) {
-      const int k = u / kDotRows, r = u % kDotRows;
-      ss[k][r] = rblk + r < n ? (sg.s[k] ? __ldg(sg.s[k] + rblk + r) : 1.f) : 0.f;
-    }
-  if (fa.labels && threadIdx.x < kDotRows && rblk + (int)threadIdx.x < n)
-    ys[threadIdx.x] = __ldg(fa.labels + rblk + threadIdx.x);
   {
-    constexpr int NI = (kDotRows * kClasses + 255) / 256;
+    constexpr int NI = (kDotRows * kClasses + 255) / 256, SP = 16;
     const int items = min(kDotRows, n - rblk) * kClasses;
     const float* zp = zpart + (size_t)rblk * kClasses + threadIdx.x;
     const size_t zs_stride = (size_t)n * kClasses;
-    float z[NI];
-#pragma unroll
-    for (int i = 0; i < NI; ++i) z[i] = __ldg(fa.cb + (threadIdx.x + i * 256) % kClasses);
-    for (int sp0 = 0; sp0 < fa.S; sp0 += 8) {
-      float v[NI][8];
+    float z[NI], v[NI][SP];
+    auto load = [&](int sp0) {
 #pragma unroll
       for (int i = 0; i < NI; ++i)
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
+        for (int u = 0; u < SP; ++u)
           v[i][u] = sp0 + u < fa.S && (int)threadIdx.x + i * 256 < items ? __ldcg(zp + i * 256 + (sp0 + u) * zs_stride)
                                                                          : 0.f;
+    };
+    load(0);
+#pragma unroll
+    for (int i = 0; i < NI; ++i) z[i] = __ldg(fa.cb + (threadIdx.x + i * 256) % kClasses);
+    if (fa.dzfrag)
+      for (int u = threadIdx.x; u < sg.nseg * kDotRows; u += 256) {
+        const int k = u / kDotRows, r = u % kDotRows;
+        ss[k][r] = rblk + r < n ? (sg.s[k] ? __ldg(sg.s[k] + rblk + r) : 1.f) : 0.f;
+      }
+    if (fa.labels && threadIdx.x < kDotRows && rblk + (int)threadIdx.x < n)
+      ys[threadIdx.x] = __ldg(fa.labels + rblk + threadIdx.x);
+    for (int sp0 = 0;;) {
 #pragma unroll
       for (int i = 0; i < NI; ++i)
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
+        for (int u = 0; u < SP; ++u)
           if (sp0 + u < fa.S) z[i] += v[i][u];
+      sp0 += SP;
+      if (sp0 >= fa.S) break;
+      load(sp0);
     }
 #pragma unroll
     for (int i = 0; i < NI; ++i)
@@ -296,22 +301,27 @@ __device__ __forceinline__ void finish_row_block(const Segs& sg, const float* __
   }
   if (!fa.dzfrag) return;
   // dz times each segment's row scale as the weight gradient's A operands
-  // (k_head_wgrad_adam): a class and a pair of rows at a time; rows past n
-  // and classes past 9 are zero
+  // (k_head_wgrad_adam): a lane's four words at a time; rows past n and
+  // classes past 9 are zero
   const int groups = (n + 15) / 16;
-  for (int u = threadIdx.x; u < sg.nseg * (kDotRows / 2) * 16; u += 256) {
-    const int c = u & 15, p = (u >> 4) % (kDotRows / 2), k = (u >> 4) / (kDotRows / 2);
-    const int group = rblk / 16 + (p >> 3);
+  for (int u = threadIdx.x; u < sg.nseg * (kDotRows / 16) * 32; u += 256) {
+    const int l = u & 31, gl = (u >> 5) % (kDotRows / 16), k = (u >> 5) / (kDotRows / 16);
+    const int group = rblk / 16 + gl;
     if (group >= groups) continue;
-    bf16 x[2][3];
+    uint32_t w[3][4];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) split3(c < kClasses ? zs[2 * p + e][c] * ss[k][2 * p + e] : 0.f, x[e]);
-    // a0: class < 8, slots 2t, 2t+1; a1: class >= 8; a2, a3: slots 8 further
-    const int word = (c >> 3) + ((p & 4) ? 2 : 0);
+    for (int a = 0; a < 4; ++a) {
+      // a0: class < 8, slots 2t, 2t+1; a1: class >= 8; a2, a3: slots 8 further
+      const int c = (l >> 2) + 8 * (a & 1), r = 16 * gl + 2 * (l & 3) + 8 * (a >> 1);
+      bf16 x[2][3];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) split3(c < kClasses ? zs[r + e][c] * ss[k][r + e] : 0.f, x[e]);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) w[q][a] = pack_bf16(x[0][q], x[1][q]);
+    }
 #pragma unroll
     for (int q = 0; q < 3; ++q)
-      reinterpret_cast<uint32_t*>(fa.dzfrag)[((((size_t)k * groups + group) * 3 + q) * 32 + (c & 7) * 4 + (p & 3)) * 4 + word] =
-          pack_bf16(x[0][q], x[1][q]);
+      fa.dzfrag[(((size_t)k * groups + group) * 3 + q) * 32 + l] = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
   }
 }
 
@@ -471,11 +481,20 @@ __global__ void __launch_bounds__(256, 1) k_head_dot(const __grid_constant__ Hea
 // x one split of at most 512 features: warp w the 16 rows 16 (w % 4) .. and
 // half w / 4 of the split.  A lane's 16-byte load of a row (8 features) feeds
 // the K slots of two MMAs, so K runs in a permuted order that the staged V
-// parts follow.  1024 rows x 6000 features: 192 blocks; see dot_split.
+// parts follow.  The three parts of the 10 classes are 30 of 32 columns: four
+// MMA tiles a K step (six, with a part's classes padded to 16, took a third
+// longer: the MMAs' own rate counts here).  Bound by a chain of round trips
+// (loads, partials, arrival, the finishing block's loads), so each phase
+// issues all of its loads before it uses one.
+// 1024 rows x 6000 features: 192 blocks (see dot_split), 12.1 us with labels,
+// 9.0 without; 14.1 and 11.2 with padded parts and V loaded a unit at a time.
+constexpr int kMmaLd = 40;  // floats of a row of the halves' sums: no bank conflicts
+int mma_smem(int split) { return std::max(split / 16 * 2 * 32 * 16, 2 * kDotRows * kMmaLd * 4); }
+
 __global__ void __launch_bounds__(256, 2) k_head_dot_mma(Segs sg, int split, int n, const float* __restrict__ V,
                                                       float* __restrict__ zpart, FinishArgs fa, int* err) {
-  extern __shared__ __align__(16) uint4 vfrag[];  // [K step of 16][part][lane]: b0, b1 of classes 0-7, of 8-15
-  __shared__ float red[kDotRows][kClasses];
+  extern __shared__ __align__(16) uint4 vfrag[];  // [K step of 16][column tiles 0-1, 2-3][lane]: b0, b1 of either tile
+  __shared__ float rs[kDotRows];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   int k = 0, sp = blockIdx.x;
@@ -488,6 +507,32 @@ __global__ void __launch_bounds__(256, 2) k_head_dot_mma(Segs sg, int split, int
   const int fs = sp * split, fe = min(fs + split, sg.F[k]);
   const int rblk = blockIdx.y * kDotRows;
   ptx::griddep_wait();  // launched with programmatic stream serialization
+  // The split's V: unit u (block of 32 features, class, quarter) is 8 features
+  // of one class.  All of a thread's loads are issued first, without branches
+  // between them, then its rows' activities; V is split while those arrive.
+  constexpr int NU = (kMmaSplit / 32 * 4 * kClasses + 255) / 256;
+  const int units = split / 32 * 4 * kClasses;
+  const float* Vk = V + sg.off[k];
+  const bool vec = ((sg.F_total | sg.off[k] | sg.F[k]) & 3) == 0;  // V itself is 256-byte aligned
+  float v[NU][8];
+#pragma unroll
+  for (int i = 0; i < NU; ++i) {
+    const int u = threadIdx.x + 256 * i, r = u >> 2;
+    const int c = r % kClasses, f = fs + 32 * (r / kClasses) + 8 * (u & 3);
+    const float* vp = Vk + (size_t)c * sg.F_total + f;
+    if (vec) {
+      const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+      const float4 lo = u < units && f < fe ? __ldg(reinterpret_cast<const float4*>(vp)) : z;
+      const float4 hi = u < units && f + 4 < fe ? __ldg(reinterpret_cast<const float4*>(vp) + 1) : z;
+      v[i][0] = lo.x; v[i][1] = lo.y; v[i][2] = lo.z; v[i][3] = lo.w;
+      v[i][4] = hi.x; v[i][5] = hi.y; v[i][6] = hi.z; v[i][7] = hi.w;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[i][e] = u < units && f + e < fe ? __ldg(vp + e) : 0.f;
+    }
+  }
+  const float scale = threadIdx.x < kDotRows && rblk + (int)threadIdx.x < n && sg.s[k]
+                          ? __ldg(sg.s[k] + rblk + threadIdx.x) : 1.f;
   // this warp's rows over its half of the split, 8 features a lane and row
   constexpr int NB = kMmaSplit / 2 / 32;  // blocks of 32 features per warp
   const int half = split / 2;             // a multiple of 32
@@ -502,71 +547,57 @@ __global__ void __launch_bounds__(256, 2) k_head_dot_mma(Segs sg, int split, int
     ha[i] = ok && ra < n ? __ldg(reinterpret_cast<const uint4*>(H + (size_t)ra * ld + f0 + 32 * i)) : z;
     hb[i] = ok && rb < n ? __ldg(reinterpret_cast<const uint4*>(H + (size_t)rb * ld + f0 + 32 * i)) : z;
   }
-  // the split's V as B operands: unit (block of 32 features, class, t) holds
-  // features 8t .. 8t+7 of the block, zero past the segment and class 9
-  const float* Vk = V + sg.off[k];
-  const bool vec = ((sg.F_total | sg.off[k]) & 3) == 0;  // V itself is 256-byte aligned
-#pragma unroll 4
-  for (int u = threadIdx.x; u < split / 32 * 64; u += 256) {
-    const int ut = u & 3, c = (u >> 2) & 15, b = u >> 6;
-    const int f = fs + 32 * b + 8 * ut;
-    const float* vp = Vk + (size_t)c * sg.F_total + f;
-    float v[8];
-    if (vec && c < kClasses && f + 8 <= fe) {
-      const float4 lo = __ldg(reinterpret_cast<const float4*>(vp)), hi = __ldg(reinterpret_cast<const float4*>(vp) + 1);
-      v[0] = lo.x; v[1] = lo.y; v[2] = lo.z; v[3] = lo.w;
-      v[4] = hi.x; v[5] = hi.y; v[6] = hi.z; v[7] = hi.w;
-    } else {
+  // V as B operands: part q of class c is column 10 q + c of 32 (30 and 31 are
+  // never read)
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = c < kClasses && f + e < fe ? __ldg(vp + e) : 0.f;
-    }
+  for (int i = 0; i < NU; ++i) {
+    const int u = threadIdx.x + 256 * i, ut = u & 3, r = u >> 2, c = r % kClasses, b = r / kClasses;
+    if (u >= units) break;
     bf16 p[8][3];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) split3(v[e], p[e]);
+    for (int e = 0; e < 8; ++e) split3(v[i][e], p[e]);
 #pragma unroll
-    for (int q = 0; q < 3; ++q)
+    for (int q = 0; q < 3; ++q) {
+      const int col = kClasses * q + c;
 #pragma unroll
       for (int s = 0; s < 2; ++s) {
-        uint2* dst = reinterpret_cast<uint2*>(&vfrag[((2 * b + s) * 3 + q) * 32 + (c & 7) * 4 + ut]) + (c >> 3);
+        uint2* dst = reinterpret_cast<uint2*>(&vfrag[((2 * b + s) * 2 + (col >> 4)) * 32 + (col & 7) * 4 + ut]) + ((col >> 3) & 1);
         *dst = make_uint2(pack_bf16(p[4 * s][q], p[4 * s + 1][q]), pack_bf16(p[4 * s + 2][q], p[4 * s + 3][q]));
       }
+    }
   }
+  if (threadIdx.x < kDotRows) rs[threadIdx.x] = scale;
   __syncthreads();
-  float d[2][4] = {};
-  const uint4* vf = vfrag + (warp >> 2) * (half / 16) * 3 * 32 + lane;
+  float d[4][4] = {};  // column tile
+  const uint4* vf = vfrag + (warp >> 2) * (half / 16) * 2 * 32 + lane;
 #pragma unroll
   for (int i = 0; i < NB; ++i) {
     if (32 * i >= half) break;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const uint4 v0 = vf[(2 * i * 3 + q) * 32], v1 = vf[((2 * i + 1) * 3 + q) * 32];
-      mma16816(d[0], ha[i].x, hb[i].x, ha[i].y, hb[i].y, v0.x, v0.y);
-      mma16816(d[1], ha[i].x, hb[i].x, ha[i].y, hb[i].y, v0.z, v0.w);
-      mma16816(d[0], ha[i].z, hb[i].z, ha[i].w, hb[i].w, v1.x, v1.y);
-      mma16816(d[1], ha[i].z, hb[i].z, ha[i].w, hb[i].w, v1.z, v1.w);
+    for (int j = 0; j < 2; ++j) {
+      const uint4 v0 = vf[(2 * i * 2 + j) * 32], v1 = vf[((2 * i + 1) * 2 + j) * 32];
+      mma16816(d[2 * j], ha[i].x, hb[i].x, ha[i].y, hb[i].y, v0.x, v0.y);
+      mma16816(d[2 * j + 1], ha[i].x, hb[i].x, ha[i].y, hb[i].y, v0.z, v0.w);
+      mma16816(d[2 * j], ha[i].z, hb[i].z, ha[i].w, hb[i].w, v1.x, v1.y);
+      mma16816(d[2 * j + 1], ha[i].z, hb[i].z, ha[i].w, hb[i].w, v1.z, v1.w);
     }
   }
-  // the two halves' sums, times the row scale
+  __syncthreads();  // the operands' memory takes the sums
+  float* red = reinterpret_cast<float*>(vfrag);  // [half][row][column], rows of kMmaLd floats
   const int lr = (warp & 3) * 16 + g;
-  if (warp >= 4) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      red[lr + (e >> 1) * 8][2 * t + (e & 1)] = d[0][e];
-      if (t == 0) red[lr + (e >> 1) * 8][8 + (e & 1)] = d[1][e];
-    }
-  }
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      *reinterpret_cast<float2*>(&red[((warp >> 2) * kDotRows + lr + 8 * r) * kMmaLd + 8 * j + 2 * t]) =
+          make_float2(d[j][2 * r], d[j][2 * r + 1]);
   __syncthreads();
-  if (warp < 4) {
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int row = rblk + lr + 8 * r;
-      if (row >= n) continue;
-      const float s = sg.s[k] ? __ldg(sg.s[k] + row) : 1.f;
-      float2* z = reinterpret_cast<float2*>(zpart + ((size_t)blockIdx.x * n + row) * kClasses);
-      const float* o = red[lr + 8 * r];
-      z[t] = make_float2(s * (d[0][2 * r] + o[2 * t]), s * (d[0][2 * r + 1] + o[2 * t + 1]));
-      if (t == 0) z[4] = make_float2(s * (d[1][2 * r] + o[8]), s * (d[1][2 * r + 1] + o[9]));
-    }
+  // a thread per row and class: the small parts first, times the row scale
+  for (int i = threadIdx.x; i < kDotRows * kClasses; i += 256) {
+    const int row = i / kClasses, c = i % kClasses;
+    const float *a = red + row * kMmaLd + c, *b = a + kDotRows * kMmaLd;
+    const float lo = a[2 * kClasses] + b[2 * kClasses], mid = a[kClasses] + b[kClasses], hi = a[0] + b[0];
+    if (rblk + row < n) zpart[((size_t)blockIdx.x * n + rblk) * kClasses + i] = rs[row] * (lo + mid + hi);
   }
   finish_row_block(sg, zpart, n, rblk, fa, err);
 }

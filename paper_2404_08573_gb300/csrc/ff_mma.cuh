@@ -19,6 +19,4 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-constexpr int mma_smem(int split) { return split / 16 * 3 * 32 * 16; }
-
 }  // namespace ff
