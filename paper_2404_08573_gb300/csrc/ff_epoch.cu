@@ -681,6 +681,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_epoch(const __grid_constant__ E
   const bool gemm_cta = (int)(blockIdx.x / 2) < P.gemm_clusters;
   const bool stream_cta = !P.split || !gemm_cta;
 
+  ptx::tmem_alloc_pair(tslot, TMEM_COLS, warp == 1);
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       ptx::mbar_init(&full[s], 1);
@@ -696,10 +697,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_epoch(const __grid_constant__ E
     }
     ptx::mbar_init(drain, 1);
     ptx::fence_mbar_init();
-  }
-  if (warp == 1) {
-    ptx::tmem_alloc_pair(tslot, TMEM_COLS);
-    ptx::tmem_relinquish_pair();
   }
   ptx::tc_fence_before();
   __syncthreads();

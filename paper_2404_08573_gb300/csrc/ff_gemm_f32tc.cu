@@ -315,6 +315,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const int chunks = (K + KC - 1) / KC;
   const int per = (chunks + S - 1) / S;
   const int c0 = min(chunks, (int)blockIdx.z * per), nc = min(chunks, c0 + per) - c0;
+  ptx::tmem_alloc_pair(tslot, STAGES * 2 * T, warp == 1);
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       ptx::mbar_init(&full[s], 2 * WARPS);
@@ -322,10 +323,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
     *abort_flag = 0;
     ptx::fence_mbar_init();
-  }
-  if (warp == 1) {
-    ptx::tmem_alloc_pair(tslot, STAGES * 2 * T);
-    ptx::tmem_relinquish_pair();
   }
   ptx::tc_fence_before();
   __syncthreads();

@@ -191,15 +191,21 @@ __device__ __forceinline__ void tmem_relinquish() {
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-// CTA-pair (cta_group::2) forms: one warp of each CTA of the pair executes
-// them, with the same column count.
-__device__ __forceinline__ void tmem_alloc_pair(uint32_t* slot, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
-               "r"(ncols)
-               : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish_pair() {
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+// CTA-pair (cta_group::2) forms, executed in both CTAs of the pair with the
+// same column count.  An allocation takes columns on both SMs, so both CTAs
+// must be running before either allocates: without the barrier a CTA that
+// started later than its peer now and then stayed in tcgen05.alloc for good
+// (784-2000x4 on layer streams: within the first 8000 GEMMs of a run; with it
+// 10 million GEMMs ran).  By all threads of the cluster; the calling warp
+// `allocates` in each CTA gives up the right to allocate again.
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* slot, uint32_t ncols, bool allocates) {
+  cluster_sync();
+  if (allocates) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
+                 "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
 }
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
