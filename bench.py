@@ -63,6 +63,59 @@ def peaks():
         return dict(hbm=6800.0, bf16=1900.0, bf16_sus=1700.0, src="fallback")
 
 
+# ------------------------------------------------------------------ stages
+class StageTimeout(RuntimeError):
+    pass
+
+
+class Stages:
+    """Where a run is: names each stage on stderr as it starts, keeps what has
+    been measured, and waits for the device with a limit, so that a stream
+    that stops ends the run with the stage's name instead of hanging it."""
+
+    def __init__(self, limit_s=60.0):
+        self.limit_s = limit_s
+        self.name = None
+        self.measured = {}
+        self.children = []  # processes that must not outlive the run
+
+    def start(self, name):
+        self.name = name
+        print(f"[bench] {name}", file=sys.stderr, flush=True)
+
+    def wait(self, query):
+        """Until query() (an event's) is true, at most limit_s seconds."""
+        end = time.monotonic() + self.limit_s
+        while not query():
+            if time.monotonic() > end:
+                raise StageTimeout(f"stage '{self.name}': the device did not finish within {self.limit_s:g} s; "
+                                   f"measured so far: {json.dumps(self.measured)}")
+            time.sleep(50e-6)
+
+
+STAGES = Stages()
+
+
+def device_wait(torch, stream, dev=None):
+    """The device idle (every stage's work ends joined to `stream`)."""
+    e = torch.cuda.Event()
+    e.record(stream)
+    STAGES.wait(e.query)
+    torch.cuda.synchronize(dev)
+
+
+def guarded(run):
+    """run(); a stage that ran out of time ends the process at once with
+    status 3 (its streams could block an orderly end)."""
+    try:
+        run()
+    except StageTimeout as e:
+        print(f"[bench] {e}", file=sys.stderr, flush=True)
+        for p in STAGES.children:
+            p.terminate()
+        os._exit(3)
+
+
 # ------------------------------------------------------------------ inputs
 def epoch_inputs(seed=0):
     """The epoch's concatenated pair batches: x [2*60000, 784] float32 and
@@ -98,6 +151,7 @@ class ClockSampler:
             self.p = subprocess.Popen(["nvidia-smi", "-i", str(self.index), f"--query-gpu={self.FIELDS}",
                                        "--format=csv,noheader,nounits", "-lms", "200"], stdout=self.f,
                                       stderr=subprocess.DEVNULL)
+            STAGES.children.append(self.p)
         except Exception:
             self.p = None
 
@@ -275,7 +329,7 @@ def run_ours(args):
             n.sync(stream)
 
     def barrier():
-        torch.cuda.synchronize(dev)
+        device_wait(torch, stream, dev)
         if dist is not None:
             dist.barrier()
 
@@ -319,13 +373,14 @@ def run_ours(args):
                 r0 = 2 * start
                 tr.net.train_step(X[r0:r0 + 2 * b], Lb[r0:r0 + 2 * b], B=b, loss=loss[t], stream=stream)
                 tr.net.sync(stream)
-                stream.synchronize()
+                device_wait(torch, stream, dev)
                 for k, a in enumerate(tr.active()):
                     lo[k] = min(lo[k], a)
                     if a == 0.0 and dead_at[k] is None:
                         dead_at[k] = t
         return lo, dead_at
 
+    STAGES.start("eager epochs")
     live.restore()
     with torch.cuda.stream(stream):
         for _ in range(args.warmup):
@@ -336,25 +391,31 @@ def run_ours(args):
     clk.start()
     # eager: one host call into libff per batch
     ms_eager, act_eager, launches_eager = timed_epochs(live, lambda: epoch(net), args.steps)
+    STAGES.measured["ms_per_step_eager"] = round(ms_eager / args.steps, 4)
     final_loss = loss[-1].cpu().numpy().tolist()
     # one epoch captured as a CUDA graph (the 4 layer streams as branches), replayed per step
     ms_graph, launches_graph = None, 0
     if not args.no_graph:
+        STAGES.start("epochs as one CUDA graph")
         live.restore()
         l0 = lib.ff_kernel_launches()
         graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(graph, stream=stream):
             epoch(net)
         launches_per_epoch = lib.ff_kernel_launches() - l0
-        for _ in range(args.warmup):
-            graph.replay()
+        with torch.cuda.stream(stream):
+            for _ in range(args.warmup):
+                graph.replay()
+        barrier()
         ms_graph, _, _ = timed_epochs(live, graph.replay, args.steps)
+        STAGES.measured["ms_per_step_graph"] = round(ms_graph / args.steps, 4)
         launches_graph = launches_per_epoch * args.steps
         del graph
     # the whole epoch in one persistent kernel (ff_net_train_epoch; the last,
     # partial batch through the per-step path)
     ms_epoch, launches_epoch = None, 0
     if not args.no_epoch_kernel:
+        STAGES.start("persistent epoch kernel")
         run_epoch = lambda: net.train_epoch(X, Lb, PAIRS_PER_EPOCH, BATCH, loss=loss, stream=stream)
         live.restore()
         with torch.cuda.stream(stream):
@@ -362,6 +423,7 @@ def run_ours(args):
                 run_epoch()
         barrier()
         ms_epoch, act_epoch, launches_epoch = timed_epochs(live, run_epoch, args.steps)
+        STAGES.measured["ms_per_step_epoch_kernel"] = round(ms_epoch / args.steps, 4)
     # the headline is the fastest of the ways of launching the same work
     modes = [(ms_eager, "eager (one ff_net_train_step call per batch)", launches_eager)]
     if ms_graph is not None:
@@ -374,6 +436,7 @@ def run_ours(args):
     # the workload's own learning rate, timed the same way
     at_cfg = None
     if not args.no_cfg_lr:
+        STAGES.start("epochs at the workload's learning rate")
         cfg_tr = _Trainer(ff, torch, dev, LR, BATCH)
         cfg_tr.restore()
         with torch.cuda.stream(stream):
@@ -396,6 +459,7 @@ def run_ours(args):
     # true and the wrong labels; each epoch from the restored initial state
     e2e = None
     if not args.no_e2e:
+        STAGES.start("end to end, eager")
         X_img = np.concatenate([X_h[2 * start:2 * start + b] for start, b in bl])   # positive halves
         Xp = torch.from_numpy(X_img).pin_memory()
         Lp = torch.from_numpy(L_h).pin_memory()
@@ -449,6 +513,8 @@ def run_ours(args):
         if not args.no_graph:
             # the same epoch -- its host-to-device copies, steps and loss read
             # back -- captured once as a CUDA graph and replayed per epoch
+            STAGES.measured["e2e_ms_per_step_eager"] = round(ems / args.steps, 4)
+            STAGES.start("end to end as one CUDA graph")
             live.restore()
             egraph = torch.cuda.CUDAGraph()
             with torch.cuda.graph(egraph, stream=stream):
@@ -471,6 +537,7 @@ def run_ours(args):
     # bracketed by CUDA events on that stream by libff's profiler.
     kernels, roof = [], None
     if not args.no_profile:
+        STAGES.start("kernel profile")
         import ctypes
         hs = [layers[k].new_activation(2 * BATCH) for k in range(len(layers) - 1)]
         ss = [torch.empty(2 * BATCH, device=dev) for _ in range(len(layers) - 1)]
@@ -531,9 +598,11 @@ def run_ours(args):
                     "peak": peak, "unit": top["unit"], "frac": round(top["achieved"] / peak, 4),
                     "peak_source": pk["src"] + (" bf16 burst (kernel timed alone)" if is_gemm else " HBM copy"),
                     "traffic": traffic, "share": top["share"]}
+    STAGES.start("active fractions over an epoch")
     lo_live, dead_live = alive_pass(live)
     clocks = clk.stop()
 
+    STAGES.start("CPU baseline and report")
     if rank == 0:
         pk = peaks()
         tflops = value * train_flops_per_pair() / 1e12
@@ -592,7 +661,7 @@ def _traffic(workload, kernel):
 TF32_PER_BF16 = 1.1 / 2.25
 
 
-def _kernel_profile(lib, torch, fn, pk, workload=None, tf32x3=False):
+def _kernel_profile(lib, torch, stream, fn, pk, workload=None, tf32x3=False):
     """Per-kernel device time of one more call of `fn`, every launch bracketed
     by CUDA events on its own stream by libff's profiler: the kernel table and
     the roofline of the kernel with the most device time (tensor-core GEMMs
@@ -601,10 +670,11 @@ def _kernel_profile(lib, torch, fn, pk, workload=None, tf32x3=False):
     GEMMs against the fp32 FMA peak, the rest against the measured HBM copy
     bandwidth)."""
     import ctypes
-    torch.cuda.synchronize()
+    STAGES.start("kernel profile")
+    device_wait(torch, stream)
     lib.ff_profile_enable(1)
     fn()
-    torch.cuda.synchronize()
+    device_wait(torch, stream)
     lib.ff_profile_enable(0)
     cap = 32
     names = (ctypes.c_char_p * cap)()
@@ -642,13 +712,13 @@ def _kernel_profile(lib, torch, fn, pk, workload=None, tf32x3=False):
 
 def _timed_loop(torch, stream, fn, k):
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    torch.cuda.synchronize()
+    device_wait(torch, stream)
     with torch.cuda.stream(stream):
         e0.record(stream)
         for _ in range(k):
             fn()
         e1.record(stream)
-    torch.cuda.synchronize()
+    device_wait(torch, stream)
     return e0.elapsed_time(e1)
 
 
@@ -667,6 +737,7 @@ def run_other(args):
     out = {"n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "data": "synthetic",
            "scaling": "weak", "vs_baseline": None, "higher_is_better": True}
     w = args.workload
+    STAGES.start(w)
     prof = None  # the workload's call, profiled once more after the timed calls
     tf32x3 = False  # its tensor-core GEMMs take fp32 operands (three TF32 products per term)
     if w.startswith("predict"):
@@ -813,11 +884,13 @@ def run_other(args):
                                max_rows=2 * BATCH) for k in range(len(NET) - 1)]
             pff = ff.Pff(layers, P, BATCH, 1, S, mode=mode, nodes=nodes)
             pff.run(x, labs, 0, S, stream=stream)          # warm-up run (same work)
-            torch.cuda.synchronize()
+            device_wait(torch, stream)
             ms = _timed_loop(torch, stream, lambda: pff.run(x, labs, 0, S, stream=stream), 1)
             pff.close()
             return ms
+        STAGES.start("chapters, a stream per layer")
         ms_par = min(one("single_layer", 1) for _ in range(max(1, args.steps // 5)))
+        STAGES.start("chapters on one stream")
         ms_seq = min(one("all_layers", 1) for _ in range(max(1, args.steps // 5)))
         pair_epochs = S * P
         flops = pair_epochs * (train_flops_per_pair() + 2.0 * 2 * sum(NET[k] * NET[k + 1] for k in range(3)))
@@ -869,7 +942,8 @@ def run_other(args):
                     "dtype": "bf16", "tflops": round(flops / (ms_p / 1e3) / 1e12, 2),
                     "single_stream_ms_per_step": round(ms_s, 4), "speedup_vs_single_stream": round(ms_s / ms_p, 3),
                     "config": {"workload": "ff_train_784-2000x5_bf16_5streams_60x1000"}})
-        out["kernels"], out["roofline"] = _kernel_profile(lib, torch, lambda: _timed_loop(torch, stream, prof, 1), pk)
+        out["kernels"], out["roofline"] = _kernel_profile(lib, torch, stream,
+                                                          lambda: _timed_loop(torch, stream, prof, 1), pk)
         prof = None
         net.close()
     elif w == "wide_4x8192":
@@ -897,7 +971,8 @@ def run_other(args):
         ms_single = _timed_loop(torch, stream, fn, args.steps) / args.steps  # each step synced: no overlap
         flops = 4.0 * 2 * B * sum(netw[i] * netw[i + 1] for i in range(4))
         tf = flops / (ms / 1e3) / 1e12
-        out["kernels"], out["roofline"] = _kernel_profile(lib, torch, lambda: _timed_loop(torch, stream, fn, 1), pk)
+        out["kernels"], out["roofline"] = _kernel_profile(lib, torch, stream,
+                                                          lambda: _timed_loop(torch, stream, fn, 1), pk)
         prof = None
         out.update({"metric": "FF train pairs/s on 3072-8192x4 (B=4096 pairs)", "value": round(B / (ms / 1e3), 1),
                     "unit": "pairs/s", "ms_per_step": round(ms, 4), "dtype": "bf16", "tflops": round(tf, 2),
@@ -996,7 +1071,8 @@ def run_other(args):
                     "config": {"workload": "ff_train_784-500-500_fp32_B64_16steps"}})
     if prof is not None:
         # one more call, each launch timed on its own stream (not the timed calls above)
-        out["kernels"], out["roofline"] = _kernel_profile(lib, torch, lambda: _timed_loop(torch, stream, prof, 1), pk,
+        out["kernels"], out["roofline"] = _kernel_profile(lib, torch, stream,
+                                                          lambda: _timed_loop(torch, stream, prof, 1), pk,
                                                           out.get("config", {}).get("workload"), tf32x3)
     print(json.dumps(out), flush=True)
 
@@ -1065,9 +1141,9 @@ def main():
     if args.impl == "reference":
         run_reference(args)
     elif args.workload != "train_4x2000":
-        run_other(args)
+        guarded(lambda: run_other(args))
     else:
-        run_ours(args)
+        guarded(lambda: run_ours(args))
 
 
 if __name__ == "__main__":
