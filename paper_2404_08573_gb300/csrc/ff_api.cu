@@ -157,7 +157,6 @@ static ff_status forward_core(ff_layer* L, const void* x, const int* labels, con
   const double es = L->is_bf16 ? 2.0 : 4.0;
   const float* s;
   const void* X;
-  const bool dependent = labels || !row_scale;  // the GEMM follows a kernel of this call (see PdlLaunch)
   if (labels) {
     FF_LAUNCH(K_OVERLAY, (double)M * (K * 4.0 + L->ldK * es + 8), st,
               launch_overlay(static_cast<const float*>(x), labels, M, K, L->X, L->ldK, L->is_bf16, L->s_in, 0, st,
@@ -186,21 +185,18 @@ static ff_status forward_core(ff_layer* L, const void* x, const int* labels, con
     ep.gpart = nullptr;
     FF_LAUNCH(K_FWD_TC, 2.0 * M * N * K, st,
               tc_gemm_fwd_lg(static_cast<const bf16*>(X), L->ldK, L->Wb, L->ldK, M, N, K, ep, *lg,
-                             static_cast<bf16*>(L->dZ), &L->ds->err, st, dependent),
+                             static_cast<bf16*>(L->dZ), &L->ds->err, st),
               "forward GEMM with the local gradient (tcgen05)");
     r->local_grad_done = true;
   } else if (L->is_bf16) {
     ntiles = tc_fwd_ntiles(M, N, false);
     FF_LAUNCH(K_FWD_TC, 2.0 * M * N * K, st,
-              tc_gemm_fwd(static_cast<const bf16*>(X), L->ldK, L->Wb, L->ldK, M, N, K, ep, &L->ds->err, st,
-                          dependent),
+              tc_gemm_fwd(static_cast<const bf16*>(X), L->ldK, L->Wb, L->ldK, M, N, K, ep, &L->ds->err, st),
               "forward GEMM (tcgen05)");
   } else {
     ntiles = f32_fwd_ntiles(M, N, K);
     FF_LAUNCH(K_FWD_SIMT, 2.0 * M * N * K, st,
-              f32_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, M, N, K, M, ep, &L->ds->err, st,
-                           dependent),
-              "forward GEMM (fp32)");
+              f32_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, M, N, K, M, ep, &L->ds->err, st), "forward GEMM (fp32)");
   }
   r->s = s;
   r->H = H;
@@ -600,12 +596,12 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
       if (b16) {
         FF_LAUNCH(K_STORE_TC, 2.0 * gn * N1 * L0->K, st,
                   tc_gemm_store(static_cast<const bf16*>(X0), L0->ldK, L0->Wb, L0->ldK, gn, N1, L0->K, base, L0->ldN,
-                                err, st, true),
+                                err, st),
                   "layer-1 base GEMM (tcgen05)");
       } else {
         FF_LAUNCH(K_STORE_SIMT, 2.0 * gn * N1 * L0->K, st,
                   f32_gemm_store(static_cast<const float*>(X0), L0->ldK, L0->W, L0->K, gn, N1, L0->K, base, L0->ldN,
-                                 err, st, true),
+                                 err, st),
                   "layer-1 base GEMM (fp32)");
       }
     }
@@ -636,20 +632,20 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
         nt = tc_fwd_ntiles(rows, Lk->N, true);
         FF_LAUNCH(K_FWD_TC, 2.0 * rows * Lk->N * Lk->K, st,
                   tc_gemm_fwd(static_cast<const bf16*>(Hb[cur]), Lk->ldK, Lk->Wb, Lk->ldK, rows, Lk->N, Lk->K, ep,
-                              err, st, true),
+                              err, st),
                   "predict forward GEMM (tcgen05)");
       } else if (f32tc && tc_full_shape(rows, Lk->N)) {
         ep.narrow = false;
         nt = tc_fwd_ntiles(rows, Lk->N, false);
         FF_LAUNCH(K_FWD_TC, 2.0 * rows * Lk->N * Lk->K, st,
                   tc_gemm_fwd_f32(static_cast<const float*>(Hb[cur]), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, ep,
-                                  err, st, true),
+                                  err, st),
                   "predict forward GEMM (fp32, tcgen05 TF32 x 3)");
       } else {
         nt = f32_fwd_ntiles(rows, Lk->N, Lk->K);
         FF_LAUNCH(K_FWD_SIMT, 2.0 * rows * Lk->N * Lk->K, st,
                   f32_gemm_fwd(static_cast<const float*>(Hb[cur]), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, rows, ep,
-                               err, st, true),
+                               err, st),
                   "predict forward GEMM (fp32)");
       }
       nt_prev = nt;

@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 
 template <bool MN, int MODE>
 cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, bool pair,
-                   const EpiArgs& ep, int* err, cudaStream_t st, bool dependent) {
+                   const EpiArgs& ep, int* err, cudaStream_t st) {
   static const cudaError_t attr = [] {
     cudaError_t e = cudaFuncSetAttribute(k_f32tc_gemm<MN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     if (e == cudaSuccess)
@@ -433,19 +433,14 @@ cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int 
   cfg.dynamicSmemBytes = SMEM;
   cfg.stream = st;
   cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = pair ? 2 : 1;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = S;
   cfg.attrs = at;
-  if (pair || S > 1) {
-    cudaLaunchAttribute& c = at[cfg.numAttrs++];
-    c.id = cudaLaunchAttributeClusterDimension;
-    c.val.clusterDim.x = pair ? 2 : 1;
-    c.val.clusterDim.y = 1;
-    c.val.clusterDim.z = S;
-  }
-  if (dependent) {
-    cudaLaunchAttribute& p = at[cfg.numAttrs++];
-    p.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    p.val.programmaticStreamSerializationAllowed = 1;
-  }
+  cfg.numAttrs = pair || S > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, pair ? k_f32tc_pair<MN, MODE> : k_f32tc_gemm<MN, MODE>, A, lda, B, ldb, M, N, K, ep,
                             err);
 }
@@ -453,20 +448,20 @@ cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int 
 }  // namespace
 
 cudaError_t f32tc_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, bool pair,
-                           const EpiArgs& ep, int* err, cudaStream_t st, bool dependent) {
-  return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, S, pair, ep, err, st, dependent);
+                           const EpiArgs& ep, int* err, cudaStream_t st) {
+  return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, S, pair, ep, err, st);
 }
 
 cudaError_t f32tc_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, bool pair,
-                             float* C, int ldc, int* err, cudaStream_t st, bool dependent) {
+                             float* C, int ldc, int* err, cudaStream_t st) {
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, S, pair, ep, err, st, dependent);
+  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, S, pair, ep, err, st);
 }
 
 cudaError_t f32tc_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, int S, bool pair,
                              float* C, int ldc, int* err, cudaStream_t st) {
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, S, pair, ep, err, st, true);
+  return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, S, pair, ep, err, st);
 }
 
 }  // namespace ff

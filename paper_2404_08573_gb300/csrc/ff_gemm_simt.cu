@@ -282,7 +282,7 @@ bool aligned(const float* p, int ld) { return (reinterpret_cast<uintptr_t>(p) & 
 
 template <int T, int KGRP, bool MN, int MODE>
 cudaError_t launch_plan(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, const EpiArgs& ep,
-                        const AdamArgs& ad, cudaStream_t st, bool dependent) {
+                        const AdamArgs& ad, cudaStream_t st) {
   using C = Cfg<T, KGRP>;
   static const cudaError_t attr = cudaFuncSetAttribute(k_simt_gemm<T, KGRP, MN, MODE>,
                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
@@ -293,28 +293,23 @@ cudaError_t launch_plan(const float* A, int lda, const float* B, int ldb, int M,
   cfg.dynamicSmemBytes = C::SMEM;
   cfg.stream = st;
   cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = 1;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = S;
   cfg.attrs = at;
-  if (S > 1) {
-    cudaLaunchAttribute& c = at[cfg.numAttrs++];
-    c.id = cudaLaunchAttributeClusterDimension;
-    c.val.clusterDim.x = 1;
-    c.val.clusterDim.y = 1;
-    c.val.clusterDim.z = S;
-  }
-  if (dependent) {
-    cudaLaunchAttribute& p = at[cfg.numAttrs++];
-    p.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    p.val.programmaticStreamSerializationAllowed = 1;
-  }
+  cfg.numAttrs = S > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k_simt_gemm<T, KGRP, MN, MODE>, A, lda, B, ldb, M, N, K,
                             (aligned(A, lda) ? 1 : 0) | (aligned(B, ldb) ? 2 : 0), ep, ad);
 }
 
 template <bool MN, int MODE>
 cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int N, int K, Plan p, const EpiArgs& ep,
-                   const AdamArgs& ad, cudaStream_t st, bool dependent) {
-  if (p.kind != TILE_64) return launch_plan<128, 1, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, ad, st, dependent);
-  return launch_plan<64, 4, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, ad, st, dependent);
+                   const AdamArgs& ad, cudaStream_t st) {
+  if (p.kind != TILE_64) return launch_plan<128, 1, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, ad, st);
+  return launch_plan<64, 4, MN, MODE>(A, lda, B, ldb, M, N, K, p.S, ep, ad, st);
 }
 
 }  // namespace
@@ -323,20 +318,20 @@ int f32_fwd_ntiles(int plan_rows, int N, int K) { return cdiv(N, plan_fwd(plan_r
 int f32_fwd_ntiles_max(int N) { return cdiv(N, 64); }
 
 cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
-                         const EpiArgs& ep, int* err, cudaStream_t st, bool dependent) {
+                         const EpiArgs& ep, int* err, cudaStream_t st) {
   const Plan p = plan_fwd(plan_rows, N, K);
   if (p.kind >= TENSOR && aligned(A, lda) && aligned(B, ldb))
-    return f32tc_gemm_fwd(A, lda, B, ldb, M, N, K, p.S, p.kind == TENSOR_PAIR, ep, err, st, dependent);
-  return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, p, ep, AdamArgs{}, st, dependent);
+    return f32tc_gemm_fwd(A, lda, B, ldb, M, N, K, p.S, p.kind == TENSOR_PAIR, ep, err, st);
+  return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, p, ep, AdamArgs{}, st);
 }
 
 cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, float* C, int ldc,
-                           int* err, cudaStream_t st, bool dependent) {
+                           int* err, cudaStream_t st) {
   const Plan p = plan_kmajor(M, N, K);
   if (p.kind >= TENSOR && aligned(A, lda) && aligned(B, ldb))
-    return f32tc_gemm_store(A, lda, B, ldb, M, N, K, p.S, p.kind == TENSOR_PAIR, C, ldc, err, st, dependent);
+    return f32tc_gemm_store(A, lda, B, ldb, M, N, K, p.S, p.kind == TENSOR_PAIR, C, ldc, err, st);
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, p, ep, AdamArgs{}, st, dependent);
+  return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, p, ep, AdamArgs{}, st);
 }
 
 // C[n, k] = sum_r G[r, n] X[r, k]: rows of C index G's columns (MN-major A),
@@ -347,7 +342,7 @@ cudaError_t f32_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int
   if (p.kind >= TENSOR && aligned(G, ldg) && aligned(X, ldx))
     return f32tc_gemm_wgrad(G, ldg, X, ldx, R, N, K, p.S, p.kind == TENSOR_PAIR, C, ldc, err, st);
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
-  return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, p, ep, AdamArgs{}, st, true);
+  return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, p, ep, AdamArgs{}, st);
 }
 
 bool f32_wgrad_adam_fits(int R, int N, int K) {
@@ -358,7 +353,7 @@ bool f32_wgrad_adam_fits(int R, int N, int K) {
 
 cudaError_t f32_gemm_wgrad_adam(const float* G, int ldg, const float* X, int ldx, int R, const AdamArgs& a,
                                 cudaStream_t st) {
-  return launch<true, MODE_ADAM>(G, ldg, X, ldx, a.N, a.K, R, plan_of(a.N, a.K, R, true), EpiArgs{}, a, st, true);
+  return launch<true, MODE_ADAM>(G, ldg, X, ldx, a.N, a.K, R, plan_of(a.N, a.K, R, true), EpiArgs{}, a, st);
 }
 
 }  // namespace ff

@@ -186,7 +186,7 @@ constexpr int tc_smem() {
 // Launch configuration of one instance: the grid (tile rows padded to whole
 // pairs; a padding CTA loads zeros, supplies its half of B and writes
 // nothing), clusters of the pair (LG: of the pair and every column tile),
-// and programmatic stream serialization where `dependent` allows it.
+// and programmatic stream serialization.
 template <int BN, bool A_MN, bool B_MN, int MODE, bool PAIR, int NSTAGE, int MT, int NT, int OPB = 2, int KB = 128>
 struct TcLaunch {
   static constexpr int SMEM = tc_smem<BN, NSTAGE, MT, PAIR, NT, MODE, OPB, KB>();
@@ -199,7 +199,7 @@ struct TcLaunch {
   static constexpr int CM = PAIR ? 2 : 1;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[2];
-  TcLaunch(int M, int N, cudaStream_t st, bool dependent) {
+  TcLaunch(int M, int N, cudaStream_t st) {
     cfg.gridDim = dim3(cdiv(cdiv(M, BM * MT), CM) * CM, cdiv(N, NT * BN), 1);
     cfg.blockDim = dim3(NTHREADS, 1, 1);
     cfg.dynamicSmemBytes = SMEM;
@@ -212,7 +212,7 @@ struct TcLaunch {
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = dependent ? 2 : 1;
+    cfg.numAttrs = 2;
   }
   static auto kernel() {
     if constexpr (KB == 64)
@@ -229,12 +229,12 @@ struct TcLaunch {
 template <int BN, bool A_MN, bool B_MN, int MODE, bool PAIR, int NSTAGE, int MT, int NT = 1, int OPB = 2,
           int KB = 128>
 cudaError_t launch_tc(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, int tma_store, int M, int N,
-                      int K, const EpiArgs& ep, int* err, cudaStream_t st, bool dependent,
-                      const CUtensorMap* td = nullptr, const GradPrepArgs* lg = nullptr) {
+                      int K, const EpiArgs& ep, int* err, cudaStream_t st, const CUtensorMap* td = nullptr,
+                      const GradPrepArgs* lg = nullptr) {
   using Lc = TcLaunch<BN, A_MN, B_MN, MODE, PAIR, NSTAGE, MT, NT, OPB, KB>;
   const cudaError_t attr = Lc::set_attrs();
   if (attr != cudaSuccess) return attr;
-  Lc l(M, N, st, dependent);
+  Lc l(M, N, st);
   const GradPrepArgs none{};
   return cudaLaunchKernelEx(&l.cfg, Lc::kernel(), ta, tb, tc, td ? *td : tc, tma_store, M, N, K, ep, lg ? *lg : none,
                             err);
@@ -347,7 +347,8 @@ bool tc_fwd_lg_supported(int M, int N) {
     cudaError_t e = FwdLg::set_attrs();
     if (e == cudaSuccess) {
       // the occupancy query takes the cluster shape alone (no other launch attributes)
-      FwdLg l(2 * BM, ct * 2 * FWD_BN, nullptr, false);
+      FwdLg l(2 * BM, ct * 2 * FWD_BN, nullptr);
+      l.cfg.numAttrs = 1;
       e = cudaOccupancyMaxActiveClusters(&clusters, FwdLg::kernel(), &l.cfg);
     }
     if (e != cudaSuccess) cudaGetLastError();  // leave no sticky launch-configuration error behind
@@ -360,19 +361,19 @@ bool tc_fwd_lg_supported(int M, int N) {
 }
 
 cudaError_t tc_gemm_fwd_lg(const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K, const EpiArgs& ep,
-                           const GradPrepArgs& lg, bf16* dZ, int* err, cudaStream_t st, bool dependent) {
+                           const GradPrepArgs& lg, bf16* dZ, int* err, cudaStream_t st) {
   if (!tc_fwd_lg_supported(M, N) || ep.gpart_in || ep.logit_V || !lg.loss_part || !lg.dbpart)
     return cudaErrorInvalidValue;
   CUtensorMap ta, tb, tc, td;
   if (!make_map(&ta, A, 2, K, M, lda, BK, BM) || !make_map(&tb, B, 2, K, N, ldb, BK, b_box_rows(FWD_BN)) ||
       !make_map(&tc, ep.out, 2, ep.ldo, M, ep.ldo, 64, 32) || !make_map(&td, dZ, 2, ep.ldo, M, ep.ldo, 64, 32))
     return cudaErrorInvalidValue;
-  return launch_tc<FWD_BN, false, false, MODE_FWD_LG, true, NSTAGES, 1, 2>(ta, tb, tc, 1, M, N, K, ep, err, st,
-                                                                           dependent, &td, &lg);
+  return launch_tc<FWD_BN, false, false, MODE_FWD_LG, true, NSTAGES, 1, 2>(ta, tb, tc, 1, M, N, K, ep, err, st, &td,
+                                                                            &lg);
 }
 
 cudaError_t tc_gemm_fwd(const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K, const EpiArgs& ep,
-                        int* err, cudaStream_t st, bool dependent) {
+                        int* err, cudaStream_t st) {
   Shape sh = shape_of(M, N, FWD_BN);
   if (sh == SHAPE_TINY && !ep.narrow) sh = SHAPE_SMALL;
   const int bn = sh == SHAPE_TINY ? TINY_BN : FWD_BN;
@@ -385,19 +386,17 @@ cudaError_t tc_gemm_fwd(const bf16* A, int lda, const bf16* B, int ldb, int M, i
     // the Performance-Optimized step's forward (never narrowed)
     if (!ep.zpart || ep.logit_ldV < N || ep.narrow) return cudaErrorInvalidValue;
     if (sh == SHAPE_FULL)
-      return launch_tc<FWD_BN, false, false, MODE_FWD_LOGITS, USE_PAIR, NSTAGES, ROW_SUBTILES>(
-          ta, tb, tc, 1, M, N, K, ep, err, st, dependent);
+      return launch_tc<FWD_BN, false, false, MODE_FWD_LOGITS, USE_PAIR, NSTAGES, ROW_SUBTILES>(ta, tb, tc, 1, M, N, K,
+                                                                                               ep, err, st);
     return launch_tc<FWD_BN, false, false, MODE_FWD_LOGITS, USE_PAIR, NSTAGES_SMALL, 1>(ta, tb, tc, 1, M, N, K, ep, err,
-                                                                                        st, dependent);
+                                                                                        st);
   }
   if (sh == SHAPE_TINY)
-    return launch_tc<TINY_BN, false, false, MODE_FWD, USE_PAIR, NSTAGES_TINY, 1>(ta, tb, tc, 1, M, N, K, ep, err, st,
-                                                                                 dependent);
+    return launch_tc<TINY_BN, false, false, MODE_FWD, USE_PAIR, NSTAGES_TINY, 1>(ta, tb, tc, 1, M, N, K, ep, err, st);
   if (sh == SHAPE_SMALL)
-    return launch_tc<FWD_BN, false, false, MODE_FWD, USE_PAIR, NSTAGES_SMALL, 1>(ta, tb, tc, 1, M, N, K, ep, err, st,
-                                                                                 dependent);
-  return launch_tc<FWD_BN, false, false, MODE_FWD, USE_PAIR, NSTAGES_FULL, ROW_SUBTILES, 1, 2, KB_FULL>(
-      ta, tb, tc, 1, M, N, K, ep, err, st, dependent);
+    return launch_tc<FWD_BN, false, false, MODE_FWD, USE_PAIR, NSTAGES_SMALL, 1>(ta, tb, tc, 1, M, N, K, ep, err, st);
+  return launch_tc<FWD_BN, false, false, MODE_FWD, USE_PAIR, NSTAGES_FULL, ROW_SUBTILES, 1, 2, KB_FULL>(ta, tb, tc, 1, M,
+                                                                                                     N, K, ep, err, st);
 }
 
 // fp32 C written through shared memory and TMA when its rows are 16-byte
@@ -407,7 +406,7 @@ static bool store_map(CUtensorMap* tc, float* C, int ldc, int rows, int cols) {
 }
 
 cudaError_t tc_gemm_store(const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K, float* Cm,
-                          int ldc, int* err, cudaStream_t st, bool dependent) {
+                          int ldc, int* err, cudaStream_t st) {
   const bool full = shape_of(M, N, FWD_BN) == SHAPE_FULL;
   const int kb = full ? KB_FULL : 128;
   CUtensorMap ta, tb, tc;
@@ -418,9 +417,9 @@ cudaError_t tc_gemm_store(const bf16* A, int lda, const bf16* B, int ldb, int M,
   EpiArgs ep{nullptr, nullptr, Cm, ldc, nullptr};
   if (!full)
     return launch_tc<FWD_BN, false, false, MODE_STORE, USE_PAIR, NSTAGES_SMALL, 1>(ta, tb, tc, tma, M, N, K, ep, err,
-                                                                                   st, dependent);
+                                                                                   st);
   return launch_tc<FWD_BN, false, false, MODE_STORE, USE_PAIR, NSTAGES_FULL, ROW_SUBTILES, 1, 2, KB_FULL>(
-      ta, tb, tc, tma, M, N, K, ep, err, st, dependent);
+      ta, tb, tc, tma, M, N, K, ep, err, st);
 }
 
 cudaError_t tc_gemm_wgrad(const bf16* G, int ldg, const bf16* X, int ldx, int R, int N, int K, float* Cm, int ldc,
@@ -439,9 +438,9 @@ cudaError_t tc_gemm_wgrad(const bf16* G, int ldg, const bf16* X, int ldx, int R,
   EpiArgs ep{nullptr, nullptr, Cm, ldc, nullptr};
   if (!full)
     return launch_tc<WGRAD_BN, true, true, MODE_STORE, USE_PAIR, NSTAGES_SMALL, 1>(ta, tb, tc, tma, N, K, R, ep, err,
-                                                                                   st, true);
+                                                                                   st);
   return launch_tc<WGRAD_BN, true, true, MODE_STORE, USE_PAIR, NSTAGES_FULL, ROW_SUBTILES, 1, 2, KB_FULL>(
-      ta, tb, tc, tma, N, K, R, ep, err, st, true);
+      ta, tb, tc, tma, N, K, R, ep, err, st);
 }
 
 // ------------------------------------------------ fp32 operands (3 x TF32)
@@ -455,15 +454,15 @@ bool tc_f32_supported(int K, int lda, int ldb) {
 }
 
 cudaError_t tc_gemm_fwd_f32(const float* A, int lda, const float* B, int ldb, int M, int N, int K, const EpiArgs& ep,
-                            int* err, cudaStream_t st, bool dependent) {
+                            int* err, cudaStream_t st) {
   if (!tc_f32_supported(K, lda, ldb) || !tc_full_shape(M, N) || ep.logit_V || ep.gpart_in || (ep.ldo & 3))
     return cudaErrorInvalidValue;
   CUtensorMap ta, tb, tc;
   if (!make_map(&ta, A, 4, K, M, lda, 32, BM) || !make_map(&tb, B, 4, K, N, ldb, 32, b_box_rows(FWD_BN)) ||
       !make_map(&tc, ep.out, 4, ep.ldo, M, ep.ldo, 32, 32))
     return cudaErrorInvalidValue;
-  return launch_tc<FWD_BN, false, false, MODE_FWD, USE_PAIR, NSTAGES_F32, ROW_SUBTILES, 1, 4>(
-      ta, tb, tc, 1, M, N, K, ep, err, st, dependent);
+  return launch_tc<FWD_BN, false, false, MODE_FWD, USE_PAIR, NSTAGES_F32, ROW_SUBTILES, 1, 4>(ta, tb, tc, 1, M, N, K,
+                                                                                              ep, err, st);
 }
 
 }  // namespace ff

@@ -1203,15 +1203,14 @@ ff_status head_forward(ff_layer* const* layers, int L, const float* x, int rows,
       }
       nt = tc_fwd_ntiles(rows, Lk->N, narrow);
       FF_LAUNCH(K_FWD_TC, 2.0 * rows * Lk->N * Lk->K, st,
-                tc_gemm_fwd(static_cast<const bf16*>(in), Lk->ldK, Lk->Wb, Lk->ldK, rows, Lk->N, Lk->K, ep, err, st,
-                            true),
+                tc_gemm_fwd(static_cast<const bf16*>(in), Lk->ldK, Lk->Wb, Lk->ldK, rows, Lk->N, Lk->K, ep, err, st),
                 "head forward GEMM (tcgen05)");
     } else {
       const int plan_rows = narrow ? rows : kTrainPlanRows;
       nt = f32_fwd_ntiles(plan_rows, Lk->N, Lk->K);
       FF_LAUNCH(K_FWD_SIMT, 2.0 * rows * Lk->N * Lk->K, st,
                 f32_gemm_fwd(static_cast<const float*>(in), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, plan_rows, ep,
-                             err, st, true),
+                             err, st),
                 "head forward GEMM (fp32)");
     }
     nt_prev = nt;
@@ -1261,10 +1260,9 @@ ff_status ensure_counters(ff_head* hd, int blocks) {
 
 // Logits (and, with labels, softmax, loss, dz and the per-row-block
 // partials) of n rows: k_head_dot over the feature splits, whose last block
-// per row block finishes the rows.  dependent: see PdlLaunch.
+// per row block finishes the rows.
 ff_status head_logits(ff_head* hd, const Segs& sg, bool b16, int n, const int* labels, float* logits, int* pred,
-                      float* zpart, float* dz, float* part, uint4* dzfrag, int* err, cudaStream_t st,
-                      bool dependent = true) {
+                      float* zpart, float* dz, float* part, uint4* dzfrag, int* err, cudaStream_t st) {
   const int es = b16 ? 2 : 4;
   const int split = dot_split(sg.F, sg.nseg, n, es);
   const int S = head_splits(sg.F, sg.nseg, split);
@@ -1291,7 +1289,7 @@ ff_status head_logits(ff_head* hd, const Segs& sg, bool b16, int n, const int* l
     static const cudaError_t attr = cudaFuncSetAttribute(k_head_dot_mma, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                          mma_smem(kMmaSplit));
     FF_TRY(attr, "head kernel attributes");
-    PdlLaunch l(grid, dim3(256), st, mma_smem(split), dependent);
+    PdlLaunch l(grid, dim3(256), st, mma_smem(split));
     FF_LAUNCH(K_HEAD_LOGITS, work, st, cudaLaunchKernelEx(&l.cfg, k_head_dot_mma, sg, split, n, V, zpart, fa, err),
               "head logits, softmax and cross-entropy");
     return FF_OK;
@@ -1304,7 +1302,7 @@ ff_status head_logits(ff_head* hd, const Segs& sg, bool b16, int n, const int* l
   static const cudaError_t attr_f = cudaFuncSetAttribute(k_head_dot, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                          kDotSmem);
   FF_TRY(attr_f, "head kernel attributes");
-  PdlLaunch l(grid, dim3(256), st, kDotSmem, dependent);
+  PdlLaunch l(grid, dim3(256), st, kDotSmem);
   FF_LAUNCH(K_HEAD_LOGITS, work, st, cudaLaunchKernelEx(&l.cfg, k_head_dot, maps, sg, split, n, V, zpart, fa, err),
             "head logits, softmax and cross-entropy");
   return FF_OK;
@@ -1509,10 +1507,9 @@ static ff_status ensure_side(ff_head* hd) {
 
 // The head's part of one train step on n rows of the features in w, starting
 // at row r0 of the stored activities: logits, softmax, loss and dz
-// (k_head_dot), dV partials (k_head_wgrad), Adam on V and c (k_head_adam); or
-// k_head_dot_mma and k_head_wgrad_adam.  dependent: see PdlLaunch.
+// (k_head_dot), dV partials (k_head_wgrad), Adam on V and c (k_head_adam).
 static ff_status head_step_on_features(ff_head* hd, ff_layer* const* layers, int n_layers, const HeadWork& w, int r0,
-                                       const int* labels, int n, float* loss, cudaStream_t st, bool dependent) {
+                                       const int* labels, int n, float* loss, cudaStream_t st) {
   Segs sg = make_segs(layers, n_layers, w, hd->F);
   const bool b16 = layers[0]->is_bf16;
   const double es = b16 ? 2.0 : 4.0;
@@ -1521,8 +1518,7 @@ static ff_status head_step_on_features(ff_head* hd, ff_layer* const* layers, int
     sg.s[j] += r0;
   }
   int* err = &hd->ds->err;
-  ff_status s = head_logits(hd, sg, b16, n, labels, nullptr, nullptr, w.zpart, w.dz, w.part, w.dzfrag, err, st,
-                            dependent);
+  ff_status s = head_logits(hd, sg, b16, n, labels, nullptr, nullptr, w.zpart, w.dz, w.part, w.dzfrag, err, st);
   if (s != FF_OK) return s;
   const HeadAdamArgs a =
       head_adam_args(hd, w.dVpart, b16 ? 0 : cdiv(n, kWgRows), w.part, cdiv(n, kDotRows), n, loss);
@@ -1556,7 +1552,7 @@ ff_status ff_head_train_step(ff_head* hd, ff_layer* const* layers, int n_layers,
   int* err = &hd->ds->err;
   s = head_forward(layers, n_layers, x, n, w, err, st, false);
   if (s != FF_OK) return s;
-  return head_step_on_features(hd, layers, n_layers, w, 0, labels, n, loss, st, true);
+  return head_step_on_features(hd, layers, n_layers, w, 0, labels, n, loss, st);
 }
 
 ff_status ff_head_train_epoch(ff_head* hd, ff_layer* const* layers, int n_layers, const float* x, const int* labels,
@@ -1604,8 +1600,7 @@ ff_status ff_head_train_epoch(ff_head* hd, ff_layer* const* layers, int n_layers
     }
     for (int q = 0; q < rows; q += B, ++t) {
       const int b = rows - q < B ? rows - q : B;
-      s = head_step_on_features(hd, layers, n_layers, w[buf], q, labels + r0 + q, b, loss ? loss + t : nullptr, st,
-                                npass == 1 || q > 0);
+      s = head_step_on_features(hd, layers, n_layers, w[buf], q, labels + r0 + q, b, loss ? loss + t : nullptr, st);
       if (s != FF_OK) return s;
     }
     if (npass > 1) FF_TRY(cudaEventRecord(hd->ev_use[buf], st), "event record");
@@ -1738,7 +1733,6 @@ ff_status ff_po_train_step(ff_layer* L, ff_head* hd, const void* x, int raw_inpu
   // the layer's forward pass (layer 1: the neutral-labelled raw input)
   const void* X;
   const float* sc;
-  const bool dependent = raw_input || !row_scale;  // the GEMM follows a kernel of this call
   if (raw_input) {
     FF_LAUNCH(K_OVERLAY, (double)n * (K * 4.0 + L->ldK * es + 4), st,
               launch_overlay(static_cast<const float*>(x), nullptr, n, K, L->X, L->ldK, b16, L->s_in, 2, st),
@@ -1765,15 +1759,13 @@ ff_status ff_po_train_step(ff_layer* L, ff_head* hd, const void* x, int raw_inpu
     ep.zpart = w.zpart;
     ntiles = tc_fwd_ntiles(n, N, false);
     FF_LAUNCH(K_FWD_TC, 2.0 * n * N * K, st,
-              tc_gemm_fwd(static_cast<const bf16*>(X), L->ldK, L->Wb, L->ldK, n, N, K, ep, &L->ds->err, st,
-                          dependent),
+              tc_gemm_fwd(static_cast<const bf16*>(X), L->ldK, L->Wb, L->ldK, n, N, K, ep, &L->ds->err, st),
               "forward GEMM (tcgen05)");
   } else {
     ntiles = f32_fwd_ntiles(kF32InOrder, N, K);
     FF_LAUNCH(K_FWD_SIMT, 2.0 * n * N * K, st,
               f32_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, n, N, K, kF32InOrder, ep,
-                           &L->ds->err, st, dependent),
-              "forward GEMM (fp32)");
+                           &L->ds->err, st), "forward GEMM (fp32)");
   }
   if (!b16) {
     // the block on the raw activity: logits, cross-entropy, dz
@@ -1838,7 +1830,8 @@ ff_status ff_po_train_step(ff_layer* L, ff_head* hd, const void* x, int raw_inpu
     const HeadAdamArgs ha =
         head_adam_args(hd, w.dVpart, cdiv(n, kPoRows), w.part, cdiv(n, b16 ? kPoRows : kDotRows), n, loss);
     const int vblocks = cdiv((long long)kClasses * hd->F, 256);
-    // a plain launch, after the wait (see PdlLaunch)
+    // a plain launch: after an event wait, programmatic serialization has
+    // nothing to overlap (griddepcontrol.wait is then a no-op)
     FF_LAUNCH(K_HEAD_ADAM, (double)kClasses * hd->F * (ha.nrb * 4.0 + 28), hd->side,
               (k_head_adam<<<vblocks + 1, 256, 0, hd->side>>>(ha), cudaGetLastError()), "block Adam");
   }

@@ -152,12 +152,13 @@ inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
 //   mode 2: out[:,0..9] = 0.1, the neutral label of the softmax head (§3).
 // Output row r reads input row r % src_rows (src_rows 0: rows): with
 // src_rows = B the B images of a pair batch are read once each for both
-// their positive and their negative row.  `dependent`: see PdlLaunch.
+// their positive and their negative row.  Launched plainly, except with
+// `dependent` (predict, where another kernel of the call comes before it),
+// with programmatic stream serialization.
 cudaError_t launch_overlay(const float* x, const int* labels, int rows, int F, void* out,
                            int ldo, bool out_bf16, float* s_out, int mode, cudaStream_t st, int src_rows = 0,
                            bool dependent = false);
-// s_r = 1 / max(||x_r||, 1e-12) of an activation buffer (the first kernel of
-// its call: launched plainly).
+// s_r = 1 / max(||x_r||, 1e-12) of an activation buffer.
 cudaError_t launch_row_scale(const void* x, int ldx, bool x_bf16, int rows, int F,
                              float* s_out, cudaStream_t st);
 // Goodness from the forward GEMM's per-tile partials (forward and predict).
@@ -222,13 +223,8 @@ struct AdamArgs {
 void add_dead(AdamArgs& a, void* p, size_t bytes);
 
 // Launch configuration with programmatic stream serialization: the kernel
-// may start while the previous kernel of its stream finishes, and waits for it
-// with griddep_wait() before touching memory.  Only where it is `dependent`:
-// another kernel of the same call comes before it in the stream, with no
-// cudaStreamWaitEvent between the two.  The first kernel of a call is not --
-// the caller's stream, or a net's layer stream, may just have taken such a
-// wait -- and is launched plainly, so that a programmatic launch waits for
-// nothing but the kernel before it (captured: its node has no other edge in).
+// may start while the previous kernel of the stream finishes and waits for it
+// with griddep_wait() before touching memory.
 struct PdlLaunch {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
@@ -296,12 +292,11 @@ struct EpiArgs {
 //   wgrad:     C[N,K] = G[R,N]^T X[R,K]  (contraction over R rows)
 // Goodness partials per row the forward GEMM writes for an M x N output (its
 // tile shape depends on both and on EpiArgs::narrow), and the most it writes
-// for any M.  `dependent`: see PdlLaunch (a
-// weight gradient always is).
+// for any M.
 int tc_fwd_ntiles(int M, int N, bool narrow);
 int tc_fwd_ntiles_max(int N);
 cudaError_t tc_gemm_fwd(const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K,
-                        const EpiArgs& ep, int* err, cudaStream_t st, bool dependent);
+                        const EpiArgs& ep, int* err, cudaStream_t st);
 // The train step's forward with the local step fused into its epilogue: the
 // forward above (H into ep.out) and everything the local-gradient kernel
 // (launch_grad_prep) computes from it -- dZ' into dZ ([M, ep.ldo] bf16), the
@@ -311,9 +306,9 @@ cudaError_t tc_gemm_fwd(const bf16* A, int lda, const bf16* B, int ldb, int M, i
 // clusters (tc_fwd_lg_supported); cudaErrorInvalidValue otherwise.
 bool tc_fwd_lg_supported(int M, int N);
 cudaError_t tc_gemm_fwd_lg(const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K, const EpiArgs& ep,
-                           const GradPrepArgs& lg, bf16* dZ, int* err, cudaStream_t st, bool dependent);
+                           const GradPrepArgs& lg, bf16* dZ, int* err, cudaStream_t st);
 cudaError_t tc_gemm_store(const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K,
-                          float* C, int ldc, int* err, cudaStream_t st, bool dependent);
+                          float* C, int ldc, int* err, cudaStream_t st);
 // The same forward (without gpart_in or block logits) on fp32 operands, as
 // three TF32 tensor-core products per term (Ah Bh + Ah Bl +
 // Al Bh; relative error near 2^-21 per product); H is written in fp32.  For K
@@ -322,7 +317,7 @@ cudaError_t tc_gemm_store(const bf16* A, int lda, const bf16* B, int ldb, int M,
 bool tc_full_shape(int M, int N);
 bool tc_f32_supported(int K, int lda, int ldb);
 cudaError_t tc_gemm_fwd_f32(const float* A, int lda, const float* B, int ldb, int M, int N, int K, const EpiArgs& ep,
-                            int* err, cudaStream_t st, bool dependent);
+                            int* err, cudaStream_t st);
 cudaError_t tc_gemm_wgrad(const bf16* G, int ldg, const bf16* X, int ldx, int R, int N, int K,
                           float* C, int ldc, int* err, cudaStream_t st);
 bool tc_supported();
@@ -354,17 +349,17 @@ constexpr int kF32InOrder = 0;
 int f32_fwd_ntiles(int plan_rows, int N, int K);
 int f32_fwd_ntiles_max(int N);
 cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
-                         const EpiArgs& ep, int* err, cudaStream_t st, bool dependent);
+                         const EpiArgs& ep, int* err, cudaStream_t st);
 cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K,
-                           float* C, int ldc, int* err, cudaStream_t st, bool dependent);
+                           float* C, int ldc, int* err, cudaStream_t st);
 cudaError_t f32_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K,
                            float* C, int ldc, bool in_order, int* err, cudaStream_t st);
 // The tensor-core forms (S: slices of K; pair: 256 x 256 tiles by CTA pairs),
 // ff_gemm_f32tc.cu.
 cudaError_t f32tc_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, bool pair,
-                           const EpiArgs& ep, int* err, cudaStream_t st, bool dependent);
+                           const EpiArgs& ep, int* err, cudaStream_t st);
 cudaError_t f32tc_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, bool pair,
-                             float* C, int ldc, int* err, cudaStream_t st, bool dependent);
+                             float* C, int ldc, int* err, cudaStream_t st);
 cudaError_t f32tc_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, int S, bool pair,
                              float* C, int ldc, int* err, cudaStream_t st);
 // The weight gradient of a.N x a.K outputs over R rows and the Adam step it

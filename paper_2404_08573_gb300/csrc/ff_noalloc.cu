@@ -64,7 +64,7 @@ extern "C" FF_API ff_status ff_forward_noalloc(const void* x, const float* row_s
   float* gpart = scratch + kNoAllocPartialOffset;
   EpiArgs ep{row_scale, bias, h_out, ldN, gpart};
   e = tc_gemm_fwd(static_cast<const bf16*>(x), ldK, static_cast<const bf16*>(W_bf16), ldK, rows, out_features,
-                  in_features, ep, err, st, false);
+                  in_features, ep, err, st);
   if (e == cudaErrorInvalidValue) return FF_ERR_INVALID_ARG;  // operand alignment / tensor-map limits
   if (e != cudaSuccess) return FF_ERR_CUDA;
   FinalizeArgs fa{};
