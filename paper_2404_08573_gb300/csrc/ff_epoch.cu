@@ -1243,7 +1243,7 @@ ff_status build_plan(ff_net* n, int B, int nb, int xrp, cudaStream_t st, EpochPl
     epoch_plan_free(p);
     return s;
   }
-  static cudaError_t attr = cudaFuncSetAttribute(k_epoch, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+  const cudaError_t attr = allow_smem<k_epoch>(SMEM_BYTES);
   if (attr != cudaSuccess) {
     epoch_plan_free(p);
     return cuda_status(attr, "epoch kernel attributes");

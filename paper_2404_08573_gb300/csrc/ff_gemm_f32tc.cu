@@ -420,12 +420,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 template <bool MN, int MODE>
 cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, bool pair,
                    const EpiArgs& ep, int* err, cudaStream_t st) {
-  static const cudaError_t attr = [] {
-    cudaError_t e = cudaFuncSetAttribute(k_f32tc_gemm<MN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_f32tc_pair<MN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-    return e;
-  }();
+  const cudaError_t attr = pair ? allow_smem<k_f32tc_pair<MN, MODE>>(SMEM) : allow_smem<k_f32tc_gemm<MN, MODE>>(SMEM);
   if (attr != cudaSuccess) return attr;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = pair ? dim3(2 * cdiv(M, 2 * T), cdiv(N, 2 * T), S) : dim3(cdiv(M, T), cdiv(N, T), S);

@@ -284,8 +284,7 @@ template <int T, int KGRP, bool MN, int MODE>
 cudaError_t launch_plan(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, const EpiArgs& ep,
                         const AdamArgs& ad, cudaStream_t st) {
   using C = Cfg<T, KGRP>;
-  static const cudaError_t attr = cudaFuncSetAttribute(k_simt_gemm<T, KGRP, MN, MODE>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+  const cudaError_t attr = allow_smem<k_simt_gemm<T, KGRP, MN, MODE>>(C::SMEM);
   if (attr != cudaSuccess) return attr;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cdiv(M, T), cdiv(N, T) + (MODE == MODE_ADAM ? 1 : 0), S);

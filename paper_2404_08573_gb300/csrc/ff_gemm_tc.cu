@@ -214,16 +214,13 @@ struct TcLaunch {
     cfg.attrs = at;
     cfg.numAttrs = 2;
   }
-  static auto kernel() {
+  static constexpr auto kernel() {
     if constexpr (KB == 64)
       return k_tc_gemm_r88<BN, A_MN, B_MN, MODE, PAIR, NSTAGE, MT, NT, OPB, KB>;
     else
       return k_tc_gemm<BN, A_MN, B_MN, MODE, PAIR, NSTAGE, MT, NT, OPB, KB>;
   }
-  static cudaError_t set_attrs() {
-    static cudaError_t e = cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-    return e;
-  }
+  static cudaError_t set_attrs() { return allow_smem<kernel()>(SMEM); }
 };
 
 template <int BN, bool A_MN, bool B_MN, int MODE, bool PAIR, int NSTAGE, int MT, int NT = 1, int OPB = 2,

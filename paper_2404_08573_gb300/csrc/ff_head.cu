@@ -1286,9 +1286,7 @@ ff_status head_logits(ff_head* hd, const Segs& sg, bool b16, int n, const int* l
   dim3 grid(S, cdiv(n, kDotRows));
   const double work = (double)n * sg.F_total * es + (double)n * (2 * S + 2) * kClasses * 4;
   if (b16) {
-    static const cudaError_t attr = cudaFuncSetAttribute(k_head_dot_mma, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         mma_smem(kMmaSplit));
-    FF_TRY(attr, "head kernel attributes");
+    FF_TRY(allow_smem<k_head_dot_mma>(mma_smem(kMmaSplit)), "head kernel attributes");
     PdlLaunch l(grid, dim3(256), st, mma_smem(split));
     FF_LAUNCH(K_HEAD_LOGITS, work, st, cudaLaunchKernelEx(&l.cfg, k_head_dot_mma, sg, split, n, V, zpart, fa, err),
               "head logits, softmax and cross-entropy");
@@ -1299,9 +1297,7 @@ ff_status head_logits(ff_head* hd, const Segs& sg, bool b16, int n, const int* l
   for (int k = 0; k < sg.nseg; ++k)
     if (!make_plain_map(&maps.m[k], sg.H[k], es, sg.ld[k], n, sg.ld[k], 512 / es, kDotRows))
       return FF_ERR_INVALID_ARG;
-  static const cudaError_t attr_f = cudaFuncSetAttribute(k_head_dot, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         kDotSmem);
-  FF_TRY(attr_f, "head kernel attributes");
+  FF_TRY(allow_smem<k_head_dot>(kDotSmem), "head kernel attributes");
   PdlLaunch l(grid, dim3(256), st, kDotSmem);
   FF_LAUNCH(K_HEAD_LOGITS, work, st, cudaLaunchKernelEx(&l.cfg, k_head_dot, maps, sg, split, n, V, zpart, fa, err),
             "head logits, softmax and cross-entropy");

@@ -9,6 +9,7 @@
 #include <cstdint>
 
 #include "ff.h"
+#include "ff_once.h"
 
 typedef __nv_bfloat16 bf16;
 
@@ -221,6 +222,15 @@ struct AdamArgs {
 // Adds [p, p + bytes) to the Adam step's dead buffers (its whole 128-byte
 // lines; nothing when p is not 128-byte aligned).
 void add_dead(AdamArgs& a, void* p, size_t bytes);
+
+// Opts Kernel into `bytes` of dynamic shared memory on the current device.
+template <auto Kernel>
+cudaError_t allow_smem(int bytes) {
+  static std::atomic<unsigned long long> done{0};
+  return once_per_device<cudaError_t>(
+      done, [](int* dev) { return cudaGetDevice(dev); },
+      [&] { return cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
+}
 
 // Launch configuration with programmatic stream serialization: the kernel
 // may start while the previous kernel of the stream finishes and waits for it
