@@ -167,7 +167,11 @@ struct FinishArgs {
 // tcgen05 tile would leave most SMs idle and wait on TMEM and barrier set-up.
 // The fp32 operand (V, or dz times the row scale) enters as three bf16 parts
 // of 8 mantissa bits each, x = hi + mid + lo exactly, whose products with the
-// activity are exact and summed in fp32: nothing is lost against fp32 FMAs.
+// activity are exact.  The tensor cores' running sum is not rounded to nearest:
+// kept in it for a whole batch it drifted by 1.5e-6 of dV at 1024 rows and
+// 1.9e-5 at 16384.  So only 32 features, or 16 rows with the small parts first,
+// are summed there, and each such sum is added to fp32 registers with rounded
+// adds (mma_add).
 __device__ __forceinline__ void split3(float x, bf16 (&p)[3]) {
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -576,10 +580,13 @@ __global__ void __launch_bounds__(256, 2) k_head_dot_mma(Segs sg, int split, int
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const uint4 v0 = vf[(2 * i * 2 + j) * 32], v1 = vf[((2 * i + 1) * 2 + j) * 32];
-      mma16816(d[2 * j], ha[i].x, hb[i].x, ha[i].y, hb[i].y, v0.x, v0.y);
-      mma16816(d[2 * j + 1], ha[i].x, hb[i].x, ha[i].y, hb[i].y, v0.z, v0.w);
-      mma16816(d[2 * j], ha[i].z, hb[i].z, ha[i].w, hb[i].w, v1.x, v1.y);
-      mma16816(d[2 * j + 1], ha[i].z, hb[i].z, ha[i].w, hb[i].w, v1.z, v1.w);
+      float t0[4] = {}, t1[4] = {};
+      mma16816(t0, ha[i].x, hb[i].x, ha[i].y, hb[i].y, v0.x, v0.y);
+      mma16816(t1, ha[i].x, hb[i].x, ha[i].y, hb[i].y, v0.z, v0.w);
+      mma16816(t0, ha[i].z, hb[i].z, ha[i].w, hb[i].w, v1.x, v1.y);
+      mma16816(t1, ha[i].z, hb[i].z, ha[i].w, hb[i].w, v1.z, v1.w);
+      mma_add(d[2 * j], t0);
+      mma_add(d[2 * j + 1], t1);
     }
   }
   __syncthreads();  // the operands' memory takes the sums
@@ -1028,8 +1035,10 @@ __global__ void __launch_bounds__(256, 2) k_head_wgrad_adam(Segs sg, int n, cons
       const uint32_t sel = j & 1 ? 0x7632u : 0x5410u;
       const uint32_t b0 = __byte_perm(j < 2 ? h[0].x : h[0].y, j < 2 ? h[1].x : h[1].y, sel);
       const uint32_t b1 = __byte_perm(j < 2 ? h[2].x : h[2].y, j < 2 ? h[3].x : h[3].y, sel);
+      float sum16[4] = {};
 #pragma unroll
-      for (int q = 0; q < 3; ++q) mma16816(d[j], av[q].x, av[q].y, av[q].z, av[q].w, b0, b1);
+      for (int q = 2; q >= 0; --q) mma16816(sum16, av[q].x, av[q].y, av[q].z, av[q].w, b0, b1);
+      mma_add(d[j], sum16);
     }
   }
   // the eight warps' sums in warp order, then Adam: a thread per element

@@ -19,4 +19,11 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// A short MMA chain's sums into fp32 registers, rounded to nearest (the
+// chain itself is not: the shorter, the less it drifts).
+__device__ __forceinline__ void mma_add(float (&d)[4], const float (&t)[4]) {
+#pragma unroll
+  for (int e = 0; e < 4; ++e) d[e] = __fadd_rn(d[e], t[e]);
+}
+
 }  // namespace ff
