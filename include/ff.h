@@ -26,6 +26,11 @@
  *     FF_ERR_CUDA.  Errors found by kernels (a bounded wait that timed out, a
  *     non-finite goodness) are latched in the layer and reported by
  *     ff_layer_check().
+ *   - FF_FP32: finite values count exactly as such, also where their products
+ *     overflow (a pre-activation of -inf is an activity of 0).  An infinite
+ *     weight or input gives NaN on the larger GEMMs (they run on the tensor
+ *     cores, in parts) even where the plain product would be -inf and its
+ *     activity 0: reported as FF_ERR_NONFINITE.
  *   - A layer must not be used from two streams at the same time.
  *   - Activation buffers (the layer input when no labels are given, h_out)
  *     are row-major in the layer's precision (float for FF_FP32, bfloat16 for

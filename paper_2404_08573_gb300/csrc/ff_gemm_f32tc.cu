@@ -1,8 +1,9 @@
 // fp32 GEMMs on the tensor cores without loss of precision, for the exact fp32
 // mode's larger training GEMMs (the contracts of ff_gemm_simt.cu).
 //
-// Each fp32 operand value enters as three bf16 parts, hi = rn(x), mid =
-// rn(x - hi), lo = x - hi - mid (exact): 24 bits in all.  Six of the nine
+// Each fp32 operand value enters as three bf16 parts, hi = rn(x) (at most the
+// largest finite bf16), mid = rn(x - hi), lo = x - hi - mid: exact, 24 bits in
+// all, but for what lies below bf16's smallest number, 2^-133.  Six of the nine
 // part products are formed (lo-hi, mid-mid, mid-hi and hi-hi, both ways); the
 // three dropped ones are below 2^-25 of the term.  Every product is exact in
 // fp32.  The tensor cores' running sum is not rounded to nearest, and a sum of
@@ -28,8 +29,8 @@
 // its 16,384 values are written as 96 KB of parts and cost about 7
 // instructions each; measured 1.7 us a chunk, 136 TFLOP/s of fp32 terms on
 // the 2048-row weight gradient (the CUDA-core GEMM reaches 50).
-// Infinities and values that round to infinity in bf16 come out as NaN
-// (inf - inf), which the non-finite check reports as it does infinities.
+// An infinite operand comes out as NaN (its parts are an infinity and inf -
+// inf), which the non-finite check reports as it does infinities.
 #include "ff_f32_epilogue.cuh"
 #include "ff_internal.cuh"
 #include "ff_ptx.cuh"
@@ -56,8 +57,13 @@ __device__ __forceinline__ uint32_t cvt2(float x0, float x1) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(x0, x1);
   return *reinterpret_cast<const uint32_t*>(&v);
 }
+__device__ __forceinline__ uint32_t cvt2_finite(float x0, float x1) {
+  uint32_t v;
+  asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(v) : "f"(x1), "f"(x0));
+  return v;
+}
 __device__ __forceinline__ void split2(float x0, float x1, uint32_t (&p)[3]) {
-  p[0] = cvt2(x0, x1);
+  p[0] = cvt2_finite(x0, x1);
   x0 = __fsub_rn(x0, __uint_as_float(p[0] << 16));
   x1 = __fsub_rn(x1, __uint_as_float(p[0] & 0xFFFF0000u));
   p[1] = cvt2(x0, x1);

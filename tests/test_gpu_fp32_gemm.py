@@ -69,3 +69,32 @@ def test_fp32_forward_and_weight_gradient_at_tile_edges(M, K, N):
     dW = torch.from_numpy(layer.get_grad()[0]).cuda().double()
     xd = x[:, :K].double()
     assert bool(((dW - G.T @ xd).abs() <= (M + 8) * U32 * (G.abs().T @ xd.abs())).all())
+
+
+# the first two take the tensor cores' bf16 parts, the last the CUDA cores
+@pytest.mark.parametrize("M,K,N", [(512, 768, 2048), (2048, 2000, 2000), (64, 32, 64)])
+def test_values_past_the_largest_bf16(M, K, N):
+    """Finite values that bf16 rounds to infinity count like any other, and a
+    sum that overflows to -inf is a zero activity, whatever the GEMM."""
+    torch = torch_cuda()
+    ff = lib_ready()
+    g = torch.Generator("cuda").manual_seed(K)
+    layer = ff.Layer(K, N, prec="fp32", max_rows=M)
+    W = layer.get_state()["W"]
+    W[0, 5], W[1, 5], W[2, 9] = 3.4e38, -3.4e38, -3e38
+    layer.set_state(W=W, b=np.zeros(N, np.float32))
+    x = layer.new_activation(M, K)
+    x[:, :K] = torch.rand(M, K, device="cuda", generator=g)
+    x[:, 5] = 2.0 ** -120   # times 3.4e38: 256
+    x[:, 9] = 0.0
+    x[7, 9] = 4.0           # row 7, unit 2: -1.2e39
+    h = layer.new_activation(M)
+    good = torch.empty(M, device="cuda")
+    layer.forward(x, row_scale=torch.ones(M, device="cuda"), h_out=h, goodness=good)
+    torch.cuda.synchronize()
+    layer.check()           # nothing non-finite
+    xd, Wd = x[:, :K].double(), torch.from_numpy(W).cuda().double()
+    ref = torch.relu(xd @ Wd.T)
+    bound = (K + 8) * U32 * (xd.abs() @ Wd.abs().T)
+    assert bool(((h[:, :N].double() - ref).abs() <= bound).all())
+    assert float(ref[0, 0]) > 100 and float(h[7, 2]) == 0.0
