@@ -147,7 +147,14 @@ FF_API ff_status ff_layer_train_step(ff_layer* layer, const void* x, const int* 
  * into goodness[r, c] ([n, 10] float32, or NULL) and pred[r] (int32) is the
  * label with the largest sum, the lowest label on ties.  All layers must share
  * one precision and chain (out_features of layer k == in_features of k+1).
- * Scratch space is owned by layers[0] (grown on demand). n == 0 is a no-op. */
+ * Scratch space is owned by layers[0], grown on demand and kept: about 80 MB
+ * of activations, and for n of several chunks up to 96 MB of layer-1 rows
+ * more.  n == 0 is a no-op.
+ * FF_FP32: GEMMs that fill the GPU take three TF32 products a term (goodness
+ * within 1e-4 of the exact sums, 2e-5 measured), smaller ones -- few samples,
+ * the last ones of a call -- exact products.  So a sample's goodness may
+ * differ by up to 1e-4 of it between calls of different n, and between places
+ * in one call, and a label whose two best sums are that close may too. */
 FF_API ff_status ff_predict(ff_layer* const* layers, int n_layers, const float* x, int n,
                      int* pred, float* goodness, void* stream);
 
