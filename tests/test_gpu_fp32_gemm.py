@@ -18,7 +18,10 @@ SHAPES = [(2, 10, 8), (2, 33, 1), (62, 31, 63), (64, 32, 64), (66, 65, 65), (128
           (254, 1001, 127), (256, 256, 2000), (600, 129, 1023), (1538, 300, 1027),
           # large enough for the tensor cores: whole tiles; every edge ragged;
           # a last chunk of 4; several K slices, the last one short
-          (512, 768, 2048), (1022, 1004, 1001), (1150, 2052, 643), (258, 2500, 1500)]
+          (512, 768, 2048), (1022, 1004, 1001), (1150, 2052, 643), (258, 2500, 1500),
+          # forwards by CTA pairs: a last 256-column tile of 4 columns (its second half empty) and
+          # a last row tile two rows short; two K slices
+          (2046, 1004, 2052), (1022, 784, 2000)]
 
 
 @pytest.mark.parametrize("M,K,N", SHAPES)

@@ -206,6 +206,7 @@ def test_head_predict_matches_oracle(env, prec, dims, n, max_rows):
 @pytest.mark.parametrize("prec,dims,n,B", [
     ("bf16", (784, 256, 256, 128), 5 * 512 + 100, 512),      # one forward pass, a ragged last step
     ("bf16", (784, 512, 256), 17 * 1024 + 300, 1024),        # two forward passes (16384 rows, then the rest)
+    ("bf16", (784, 2000, 2000), 20 * 1024 + 300, 1024),      # three passes of at most two GEMM waves: a workspace reused
     ("fp32", (784, 200, 136), 3 * 256 + 17, 256),
 ])
 def test_head_train_epoch_is_bitwise_the_per_step_calls(env, prec, dims, n, B):
