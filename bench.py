@@ -666,8 +666,9 @@ def _kernel_profile(lib, torch, stream, fn, pk, workload=None, tf32x3=False):
     by CUDA events on its own stream by libff's profiler: the kernel table and
     the roofline of the kernel with the most device time (tensor-core GEMMs
     against the measured bf16 peak -- fp32 ones, tf32x3, against the TF32
-    peak it implies over the three products each fp32 term takes -- fp32 SIMT
-    GEMMs against the fp32 FMA peak, the rest against the measured HBM copy
+    peak it implies over the three products each fp32 term takes, and those of
+    bf16 parts (f32tc) against it over their six products -- fp32 SIMT GEMMs
+    against the fp32 FMA peak, the rest against the measured HBM copy
     bandwidth)."""
     import ctypes
     STAGES.start("kernel profile")
@@ -696,7 +697,11 @@ def _kernel_profile(lib, torch, stream, fn, pk, workload=None, tf32x3=False):
     if kernels:
         top = max(kernels, key=lambda k: k["ms"])
         if "simt" in top["kernel"]:
-            bound, peak, src = "alu", FP32_ALU_TFLOPS, "fp32 FMA peak from unit counts and clock (152 x 128 x 2 x 2.07 GHz)"
+            bound, peak = "alu", FP32_ALU_TFLOPS
+            src = "fp32 FMA peak from unit counts and clock (152 x 128 x 2 x 2.07 GHz)"
+        elif "f32tc" in top["kernel"]:
+            bound, peak = "tensor", pk["bf16"] / 6
+            src = pk["src"] + " bf16 burst / 6 products of bf16 parts per fp32 term"
         elif top["unit"] == "TFLOP/s" and tf32x3:
             bound, peak = "tensor", pk["bf16"] * TF32_PER_BF16 / 3
             src = pk["src"] + " bf16 burst x nominal TF32/bf16 ratio (1.1/2.25) / 3 TF32 products per fp32 term"

@@ -1,7 +1,7 @@
 // The libff C ABI: FF layer lifecycle, the layer-local train step, the
 // forward pass L_i(x), goodness prediction, and state access.  Host code only
 // orchestrates; every step of the path runs in the kernels of ff_elem.cu,
-// ff_gemm_tc.cu (bf16 mode) and ff_gemm_simt.cu (fp32 mode).
+// ff_gemm_tc.cu (bf16 mode), ff_gemm_simt.cu and ff_gemm_f32tc.cu (fp32 mode).
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -195,7 +195,8 @@ static ff_status forward_core(ff_layer* L, const void* x, const int* labels, con
               "forward GEMM (tcgen05)");
   } else {
     ntiles = f32_fwd_ntiles(M, N, K);
-    FF_LAUNCH(K_FWD_SIMT, 2.0 * M * N * K, st,
+    const bool tc = f32_fwd_on_tensor_cores(static_cast<const float*>(X), L->ldK, L->W, K, M, N, K);
+    FF_LAUNCH(tc ? K_FWD_F32TC : K_FWD_SIMT, 2.0 * M * N * K, st,
               f32_gemm_fwd(static_cast<const float*>(X), L->ldK, L->W, K, M, N, K, M, ep, &L->ds->err, st), "forward GEMM (fp32)");
   }
   r->s = s;
@@ -313,7 +314,9 @@ ff_status weight_update(ff_layer* L, const void* X, int M, AdamArgs& aa, cudaStr
                             L->K, L->dW, L->K, &L->ds->err, st),
               "weight-gradient GEMM (tcgen05)");
   } else {
-    FF_LAUNCH(K_WGRAD_SIMT, flops, st,
+    const bool tc = f32_wgrad_on_tensor_cores(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(X),
+                                              L->ldK, M, L->N, L->K, in_order);
+    FF_LAUNCH(tc ? K_WGRAD_F32TC : K_WGRAD_SIMT, flops, st,
               f32_gemm_wgrad(static_cast<const float*>(L->dZ), L->ldN, static_cast<const float*>(X), L->ldK, M, L->N,
                               L->K, L->dW, L->K, in_order, &L->ds->err, st),
               "weight-gradient GEMM (fp32)");
@@ -599,7 +602,8 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
                                 err, st),
                   "layer-1 base GEMM (tcgen05)");
       } else {
-        FF_LAUNCH(K_STORE_SIMT, 2.0 * gn * N1 * L0->K, st,
+        const bool tc = f32_fwd_on_tensor_cores(static_cast<const float*>(X0), L0->ldK, L0->W, L0->K, gn, N1, L0->K);
+        FF_LAUNCH(tc ? K_STORE_F32TC : K_STORE_SIMT, 2.0 * gn * N1 * L0->K, st,
                   f32_gemm_store(static_cast<const float*>(X0), L0->ldK, L0->W, L0->K, gn, N1, L0->K, base, L0->ldN,
                                  err, st),
                   "layer-1 base GEMM (fp32)");
@@ -643,7 +647,9 @@ static ff_status predict_impl(ff_layer* const* layers, int n_layers, const float
                   "predict forward GEMM (fp32, tcgen05 TF32 x 3)");
       } else {
         nt = f32_fwd_ntiles(rows, Lk->N, Lk->K);
-        FF_LAUNCH(K_FWD_SIMT, 2.0 * rows * Lk->N * Lk->K, st,
+        const bool tc = f32_fwd_on_tensor_cores(static_cast<const float*>(Hb[cur]), Lk->ldK, Lk->W, Lk->K, rows, Lk->N,
+                                                Lk->K);
+        FF_LAUNCH(tc ? K_FWD_F32TC : K_FWD_SIMT, 2.0 * rows * Lk->N * Lk->K, st,
                   f32_gemm_fwd(static_cast<const float*>(Hb[cur]), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, rows, ep,
                                err, st),
                   "predict forward GEMM (fp32)");

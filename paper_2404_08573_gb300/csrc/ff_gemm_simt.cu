@@ -279,6 +279,10 @@ Plan plan_fwd(int plan_rows, int N, int K) {
 }
 
 bool aligned(const float* p, int ld) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (ld & 3) == 0; }
+bool on_tensor_cores(const Plan& p, const float* A, int lda, const float* B, int ldb) {
+  return p.kind >= TENSOR && aligned(A, lda) && aligned(B, ldb);
+}
+Plan plan_wgrad(int R, int N, int K, bool in_order) { return in_order ? Plan{TILE_128, 1} : plan_of(N, K, R, true); }
 
 template <int T, int KGRP, bool MN, int MODE>
 cudaError_t launch_plan(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int S, const EpiArgs& ep,
@@ -315,11 +319,17 @@ cudaError_t launch(const float* A, int lda, const float* B, int ldb, int M, int 
 
 int f32_fwd_ntiles(int plan_rows, int N, int K) { return cdiv(N, plan_fwd(plan_rows, N, K).kind == TILE_64 ? 64 : 128); }
 int f32_fwd_ntiles_max(int N) { return cdiv(N, 64); }
+bool f32_fwd_on_tensor_cores(const float* A, int lda, const float* B, int ldb, int plan_rows, int N, int K) {
+  return on_tensor_cores(plan_fwd(plan_rows, N, K), A, lda, B, ldb);
+}
+bool f32_wgrad_on_tensor_cores(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, bool in_order) {
+  return on_tensor_cores(plan_wgrad(R, N, K, in_order), G, ldg, X, ldx);
+}
 
 cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
                          const EpiArgs& ep, int* err, cudaStream_t st) {
   const Plan p = plan_fwd(plan_rows, N, K);
-  if (p.kind >= TENSOR && aligned(A, lda) && aligned(B, ldb))
+  if (on_tensor_cores(p, A, lda, B, ldb))
     return f32tc_gemm_fwd(A, lda, B, ldb, M, N, K, p.S, p.kind == TENSOR_PAIR, ep, err, st);
   return launch<false, MODE_FWD>(A, lda, B, ldb, M, N, K, p, ep, AdamArgs{}, st);
 }
@@ -327,7 +337,7 @@ cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M
 cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K, float* C, int ldc,
                            int* err, cudaStream_t st) {
   const Plan p = plan_kmajor(M, N, K);
-  if (p.kind >= TENSOR && aligned(A, lda) && aligned(B, ldb))
+  if (on_tensor_cores(p, A, lda, B, ldb))
     return f32tc_gemm_store(A, lda, B, ldb, M, N, K, p.S, p.kind == TENSOR_PAIR, C, ldc, err, st);
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
   return launch<false, MODE_STORE>(A, lda, B, ldb, M, N, K, p, ep, AdamArgs{}, st);
@@ -337,8 +347,8 @@ cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int
 // columns of C index X's columns (MN-major B), contraction over R.
 cudaError_t f32_gemm_wgrad(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, float* C, int ldc,
                            bool in_order, int* err, cudaStream_t st) {
-  const Plan p = in_order ? Plan{TILE_128, 1} : plan_of(N, K, R, true);
-  if (p.kind >= TENSOR && aligned(G, ldg) && aligned(X, ldx))
+  const Plan p = plan_wgrad(R, N, K, in_order);
+  if (on_tensor_cores(p, G, ldg, X, ldx))
     return f32tc_gemm_wgrad(G, ldg, X, ldx, R, N, K, p.S, p.kind == TENSOR_PAIR, C, ldc, err, st);
   EpiArgs ep{nullptr, nullptr, C, ldc, nullptr};
   return launch<true, MODE_STORE>(G, ldg, X, ldx, N, K, R, p, ep, AdamArgs{}, st);

@@ -1217,7 +1217,9 @@ ff_status head_forward(ff_layer* const* layers, int L, const float* x, int rows,
     } else {
       const int plan_rows = narrow ? rows : kTrainPlanRows;
       nt = f32_fwd_ntiles(plan_rows, Lk->N, Lk->K);
-      FF_LAUNCH(K_FWD_SIMT, 2.0 * rows * Lk->N * Lk->K, st,
+      const bool tc = f32_fwd_on_tensor_cores(static_cast<const float*>(in), Lk->ldK, Lk->W, Lk->K, plan_rows, Lk->N,
+                                              Lk->K);
+      FF_LAUNCH(tc ? K_FWD_F32TC : K_FWD_SIMT, 2.0 * rows * Lk->N * Lk->K, st,
                 f32_gemm_fwd(static_cast<const float*>(in), Lk->ldK, Lk->W, Lk->K, rows, Lk->N, Lk->K, plan_rows, ep,
                              err, st),
                 "head forward GEMM (fp32)");

@@ -358,6 +358,9 @@ bool make_sw128_map(CUtensorMap* m, const void* ptr, int esize, int cols, int ro
 constexpr int kF32InOrder = 0;
 int f32_fwd_ntiles(int plan_rows, int N, int K);
 int f32_fwd_ntiles_max(int N);
+// Which of the two a call takes (a store: as a forward of its M rows).
+bool f32_fwd_on_tensor_cores(const float* A, int lda, const float* B, int ldb, int plan_rows, int N, int K);
+bool f32_wgrad_on_tensor_cores(const float* G, int ldg, const float* X, int ldx, int R, int N, int K, bool in_order);
 cudaError_t f32_gemm_fwd(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int plan_rows,
                          const EpiArgs& ep, int* err, cudaStream_t st);
 cudaError_t f32_gemm_store(const float* A, int lda, const float* B, int ldb, int M, int N, int K,

@@ -24,7 +24,7 @@ const char* const kNames[K_NUM] = {"overlay",     "row_scale",    "fwd_gemm_tc",
                                    "adam",        "init_weights", "to_bf16",       "label_columns",
                                    "store_gemm_tc", "store_gemm_simt", "expand",   "argmax",
                                    "head_logits", "head_wgrad",   "head_adam",
-                                   "epoch_gemm_tc"};
+                                   "epoch_gemm_tc", "fwd_gemm_f32tc", "wgrad_gemm_f32tc", "store_gemm_f32tc"};
 
 struct Rec {
   int kind;

@@ -101,3 +101,25 @@ def test_values_past_the_largest_bf16(M, K, N):
     bound = (K + 8) * U32 * (xd.abs() @ Wd.abs().T)
     assert bool(((h[:, :N].double() - ref).abs() <= bound).all())
     assert float(ref[0, 0]) > 100 and float(h[7, 2]) == 0.0
+
+
+@pytest.mark.parametrize("M,K,N,kind", [(2048, 2000, 2000, "f32tc"), (128, 784, 500, "simt"), (2048, 2002, 2000, "mixed")])
+def test_profile_names_the_kernels_that_ran(M, K, N, kind):
+    import ctypes
+    torch = torch_cuda()
+    ff = lib_ready()
+    layer = ff.Layer(K, N, prec="fp32", max_rows=M)
+    x = layer.new_activation(M, K)
+    x[:, :K] = 0.5
+    s = torch.ones(M, device="cuda")
+    lib = ff.lib()
+    lib.ff_profile_enable(1)
+    layer.train_step(x, row_scale=s, B=M // 2)
+    torch.cuda.synchronize()
+    lib.ff_profile_enable(0)
+    names = (ctypes.c_char_p * 32)()
+    n = lib.ff_profile_read(32, names, None, None, None)
+    gemms = {names[i].decode() for i in range(n) if b"gemm" in names[i]}
+    # K = 2002: the weights' rows are not 16-byte aligned, the activities' are
+    assert gemms == {"f32tc": {"fwd_gemm_f32tc", "wgrad_gemm_f32tc"}, "simt": {"fwd_gemm_simt", "wgrad_gemm_simt"},
+                     "mixed": {"fwd_gemm_simt", "wgrad_gemm_f32tc"}}[kind]
