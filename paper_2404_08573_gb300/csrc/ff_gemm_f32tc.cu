@@ -24,11 +24,13 @@
 //                = 128, K = 16) into one of four TMEM buffers
 //   warps 8..15  add each finished chunk to their registers (a 32-row quarter
 //                of TMEM and half the columns each), then run the epilogue
-// Bound by shared memory and the splitting: a chunk's 24 MMAs read 192 KB of
-// operands (1536 clocks at 128 bytes a clock, as long as their arithmetic),
-// its 16,384 values are written as 96 KB of parts and cost about 7
-// instructions each; measured 1.7 us a chunk, 136 TFLOP/s of fp32 terms on
-// the 2048-row weight gradient (the CUDA-core GEMM reaches 50).
+// Bound by the chain of a chunk, no unit being full: its loads from L2, the
+// split (about 7 instructions for each of its 16,384 values), the 96 KB of
+// parts stored and the 24 MMAs' 192 KB of operand reads follow one another with
+// two stages in flight (512 x 2000 over 2000: tensor pipe 36 % active, the
+// tensor cores' shared-memory wavefronts 22 % of peak, the load/store unit's
+// 30 %, issue slots 40 %); measured 1.7 us a chunk, 136 TFLOP/s of fp32 terms
+// on the 2048-row weight gradient (the CUDA-core GEMM reaches 50).
 // An infinite operand comes out as NaN (its parts are an infinity and inf -
 // inf), which the non-finite check reports as it does infinities.
 #include "ff_f32_epilogue.cuh"
